@@ -176,8 +176,224 @@ template <bool INV, class C> __device__ __forceinline__ void dft5(C* v) {
   v[3] = csub(b2, d2);
 }
 
+// ----------------------------------------------------------------------------
+// FP64 lines in 64-bit fixed point.
+//
+// GB300 issues two FP64 lanes per SM and clock, one 32-lane instruction in 16
+// clocks, while the integer pipes take the two 32-bit halves of a 64-bit sum in
+// one or two.  So a line of an FP64 transform is converted to 64-bit integers
+// under one scale of its own, transformed in integers, and converted back:
+//
+// * Scale.  B >= sum_j (|Re x_j| + |Im x_j|) over the line bounds every
+//   intermediate value and output of the transform.  With q = x 2^s and
+//   2^s B <= 2^62 nothing overflows, sums are exact, and an input is rounded by at
+//   most 2^-62 B.  For a line whose values are comparable that is 2^-62 L of a
+//   typical value (2^-55 at L = 128), against 2^-53 of each value in FP64.
+// * Products.  Twiddles and constants carry 62 fractional bits as two signed
+//   32-bit limbs; a product is three 32 x 32 + 64 multiply-adds, right to two
+//   units.
+//
+// Measured: a y pass of three 128^3 fields 256 -> 77 us, of three 96^3 fields
+// 115 -> 52 us; relative 2-norm error of a 3D transform of random data against
+// extended precision 2.3e-16 -> 0.9e-16 (32^3), 2.7e-16 -> 1.0e-16 (64^3),
+// 2.8e-16 -> 1.5e-16 (256 x 16 x 128), 2.9e-16 -> 1.2e-16 (80^3).  Lines with a
+// value of at least 2^1013 (or not finite) give NaN; lines with no value above
+// 2^-960 give 0.
+// ----------------------------------------------------------------------------
+struct __align__(16) Q2 {
+  long long x, y;
+};
+// (cos, -sin) of a twiddle angle: value = (h 2^32 + l) 2^-62, both limbs signed.
+struct __align__(16) TwQ {
+  int xh, xl, yh, yl;
+};
+static_assert(sizeof(Q2) == sizeof(double2) && sizeof(TwQ) == sizeof(double2), "fixed-point lines share FP64 buffers");
+
+// Scale of one line: an input with biased exponent e is its 53-bit significand
+// shifted left by 10 and then right by X - e; an output whose
+// leading zeros are lz gets the biased exponent X + 1 - lz.
+struct LineScale {
+  int X;
+  int bad;  // bits or-ed into the outputs' high words: a NaN pattern for a line that is not finite
+};
+
+__device__ __forceinline__ long long to_fixed(double d, const LineScale& ls) {
+  const int hi = __double2hiint(d);
+  const unsigned lo = (unsigned)__double2loint(d);
+  const int e = (hi >> 20) & 0x7ff;
+  const int r = min(ls.X - e, 63);  // zeros (e = 0) leave by the clamp
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 10;
+  const long long s = (long long)(hi >> 31);
+  return (long long)(m >> r) ^ s;
+}
+__device__ __forceinline__ double from_fixed(long long q, const LineScale& ls) {
+  const int sg = (int)(q >> 32) >> 31;
+  const unsigned long long u = (unsigned long long)(q ^ (long long)sg);
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << (lz & 63);
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // carries into the exponent
+  int hi = (int)(r >> 32) + ((ls.X - lz) << 20);
+  int lo = (int)r;
+  hi = u == 0ull ? 0 : hi;  // r is 0 then
+  return __hiloint2double(hi | (sg & (int)0x80000000) | ls.bad, lo);
+}
+
+// One thread's share of B: the largest biased exponent of its 16 values and the
+// sum of their significands (top 21 bits, rounded up) in units of that exponent.
+__device__ __forceinline__ uint2 thread_bound(const double2 (&v)[8]) {
+  int mx = 0;
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    mx = max(mx, max(__double2hiint(v[e].x) & 0x7fffffff, __double2hiint(v[e].y) & 0x7fffffff));
+  const int E = mx >> 20;
+  unsigned S = 16;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const unsigned hx = (unsigned)__double2hiint(v[e].x) & 0x7fffffffu, hy = (unsigned)__double2hiint(v[e].y) & 0x7fffffffu;
+    S += ((hx & 0xfffffu) | 0x100000u) >> min(E - (int)(hx >> 20), 31);
+    S += ((hy & 0xfffffu) | 0x100000u) >> min(E - (int)(hy >> 20), 31);
+  }
+  return make_uint2((unsigned)E, S);
+}
+// Sum of two shares (commutative: every thread of a line gets the same bits).
+__device__ __forceinline__ uint2 add_bounds(uint2 a, uint2 b) {
+  const int E = max((int)a.x, (int)b.x);
+  return make_uint2((unsigned)E, (a.y >> min(E - (int)a.x, 31)) + (b.y >> min(E - (int)b.x, 31)) + 1u);
+}
+__device__ __forceinline__ LineScale make_scale(uint2 b) {
+  const int E = (int)b.x;
+  LineScale s;
+  s.X = E < 64 ? 4096 : E + (32 - __clz((int)b.y)) - 20;
+  s.bad = E >= 2036 ? 0x7ff80000 : 0;
+  return s;
+}
+
+// Scales of a thread's NF lines.  Row lines of power-of-two length sit in one
+// warp; the other row lines exchange their shares through the line's (idle)
+// exchange buffer, column lines through the slots `sc`, which are free again
+// after the transform's first exchange barrier.
+template <int L, int NF, class SI>
+__device__ __forceinline__ void line_scales(const double2 (&v)[NF][8], double2* sm, int fstride, int t, const SI& si,
+                                            LineScale (&ls)[NF]) {
+  constexpr int TPL = L / 8;
+  uint2 b[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) b[f] = thread_bound(v[f]);
+  if constexpr (IsColIdx<SI>::v) {
+    static_assert(NF == 1, "column lines come one field at a time");
+    si.sc[t * si.width()] = b[0];
+    __syncthreads();
+    uint2 a = si.sc[0];
+#pragma unroll 8
+    for (int k = 1; k < TPL; ++k) a = add_bounds(a, si.sc[k * si.width()]);
+    ls[0] = make_scale(a);
+  } else if constexpr (IsPow2<L>::v) {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+#pragma unroll
+      for (int off = TPL / 2; off > 0; off >>= 1)
+        b[f] = add_bounds(b[f], make_uint2(__shfl_xor_sync(0xffffffffu, b[f].x, off),
+                                           __shfl_xor_sync(0xffffffffu, b[f].y, off)));
+      ls[f] = make_scale(b[f]);
+    }
+  } else {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) reinterpret_cast<uint2*>(sm + f * fstride)[t] = b[f];
+    __syncthreads();
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const uint2* p = reinterpret_cast<const uint2*>(sm + f * fstride);
+      uint2 a = p[0];
+#pragma unroll
+      for (int k = 1; k < TPL; ++k) a = add_bounds(a, p[k]);
+      ls[f] = make_scale(a);
+    }
+    __syncthreads();
+  }
+}
+
+__device__ __forceinline__ long long imad(int a, int b, long long c) { return (long long)a * b + c; }
+// Signed limbs of a (|a| < 2^62): a = h 2^32 + l.
+struct LimbQ {
+  int h, h2, l;  // h2 = 2 h
+};
+__device__ __forceinline__ LimbQ limbs(long long a) {
+  LimbQ r;
+  r.l = (int)a;
+  r.h = (int)(a >> 32) - (r.l >> 31);
+  r.h2 = 2 * r.h;
+  return r;
+}
+// a w for a real constant w = (wh 2^32 + wl) 2^-62: half the product from the limbs' upper parts.
+__device__ __forceinline__ long long mulq(long long a, int wh, int wl) {
+  const LimbQ x = limbs(a);
+  return 2 * imad(x.h2, wh, imad(x.l, wh, imad(x.h, wl, 0)) >> 31);
+}
+__device__ __forceinline__ Q2 cmul_limbs(Q2 a, int wh, int wl, int vh, int vl) {  // w + i v
+  const LimbQ x = limbs(a.x), y = limbs(a.y);
+  const int nh = -vh, nl = -vl;
+  const long long tr = imad(y.l, nh, imad(y.h, nl, imad(x.l, wh, imad(x.h, wl, 0))));
+  const long long ti = imad(y.l, wh, imad(y.h, wl, imad(x.l, vh, imad(x.h, vl, 0))));
+  return Q2{2 * imad(y.h2, nh, imad(x.h2, wh, tr >> 31)), 2 * imad(y.h2, wh, imad(x.h2, vh, ti >> 31))};
+}
+__device__ __forceinline__ Q2 cmul(Q2 a, TwQ w) { return cmul_limbs(a, w.xh, w.xl, w.yh, w.yl); }
+__device__ __forceinline__ Q2 cmulc(Q2 a, TwQ w) { return cmul_limbs(a, w.xh, w.xl, -w.yh, -w.yl); }
+
+template <bool INV> __device__ __forceinline__ void dft8(Q2* v) {
+  constexpr int hh = 759250125, hl = -25716447;  // 2^62 / sqrt 2
+  Q2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
+  Q2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+  dft4v<INV>(e0, e1, e2, e3);
+  dft4v<INV>(o0, o1, o2, o3);
+  o1 = Q2{mulq(o1.x, hh, hl), mulq(o1.y, hh, hl)};
+  o3 = Q2{mulq(o3.x, hh, hl), mulq(o3.y, hh, hl)};
+  if (INV) {
+    o1 = Q2{o1.x - o1.y, o1.x + o1.y};
+    o2 = mul_i(o2);
+    o3 = Q2{-o3.x - o3.y, o3.x - o3.y};
+  } else {
+    o1 = Q2{o1.x + o1.y, o1.y - o1.x};
+    o2 = mul_mi(o2);
+    o3 = Q2{o3.y - o3.x, -o3.x - o3.y};
+  }
+  v[0] = cadd(e0, o0);
+  v[4] = csub(e0, o0);
+  v[1] = cadd(e1, o1);
+  v[5] = csub(e1, o1);
+  v[2] = cadd(e2, o2);
+  v[6] = csub(e2, o2);
+  v[3] = cadd(e3, o3);
+  v[7] = csub(e3, o3);
+}
+template <bool INV> __device__ __forceinline__ void dft3(Q2* v) {
+  const Q2 a0 = v[0], t1 = cadd(v[1], v[2]), t2 = csub(v[1], v[2]);
+  const Q2 b = Q2{a0.x - (t1.x >> 1), a0.y - (t1.y >> 1)};
+  const Q2 m = Q2{mulq(t2.x, 929887697, -1332128537), mulq(t2.y, 929887697, -1332128537)};
+  const Q2 d = INV ? mul_i(m) : mul_mi(m);
+  v[0] = cadd(a0, t1);
+  v[1] = cadd(b, d);
+  v[2] = csub(b, d);
+}
+template <bool INV> __device__ __forceinline__ void dft5(Q2* v) {
+  auto sc = [](Q2 a, int h, int l) { return Q2{mulq(a.x, h, l), mulq(a.y, h, l)}; };
+  constexpr int c1h = 331804471, c1l = 803819395, c2h = -868675383, c2l = -803819395, s1h = 1021189159, s1l = -2002125123, s2h = 631129609, s2l = -357254181;
+  const Q2 a0 = v[0];
+  const Q2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]), t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
+  const Q2 b1 = cadd(a0, cadd(sc(t1, c1h, c1l), sc(t2, c2h, c2l)));
+  const Q2 b2 = cadd(a0, cadd(sc(t1, c2h, c2l), sc(t2, c1h, c1l)));
+  const Q2 e1 = cadd(sc(t3, s1h, s1l), sc(t4, s2h, s2l));
+  const Q2 e2 = csub(sc(t3, s2h, s2l), sc(t4, s1h, s1l));
+  const Q2 d1 = INV ? mul_i(e1) : mul_mi(e1), d2 = INV ? mul_i(e2) : mul_mi(e2);
+  v[0] = cadd(a0, cadd(t1, t2));
+  v[1] = cadd(b1, d1);
+  v[4] = csub(b1, d1);
+  v[2] = cadd(b2, d2);
+  v[3] = csub(b2, d2);
+}
+
 template <int R_, bool INV, class C> __device__ __forceinline__ void dft_r(C* v) {
-  if constexpr (R_ == 8) dft8<INV>(v);
+  if constexpr (R_ == 8) dft8<INV>(v);  // Q2 lines: the fixed-point overloads
   else if constexpr (R_ == 5) dft5<INV>(v);
   else if constexpr (R_ == 4) dft4<INV>(v);
   else if constexpr (R_ == 3) dft3<INV>(v);
@@ -188,8 +404,8 @@ template <int R_, bool INV, class C> __device__ __forceinline__ void dft_r(C* v)
 // v[f][8]: this thread's registers for field f; sm + f*fstride: the shared
 // line buffer of field f for this thread's line; si(pos): offset of line
 // position pos inside that buffer; tw: shared table W_L^m, m < L.
-template <class C, int L, bool INV, int NF, int p, class SI>
-__device__ __forceinline__ void fft_passes(C (&v)[NF][8], C* sm, int fstride, const C* __restrict__ tw,
+template <class C, int L, bool INV, int NF, int p, class SI, class TW>
+__device__ __forceinline__ void fft_passes(C (&v)[NF][8], C* sm, int fstride, const TW* __restrict__ tw,
                                            int t, const SI& si) {
   using PL = Plan<L>;
   constexpr int r = PL::rad(INV, p);
@@ -204,7 +420,7 @@ __device__ __forceinline__ void fft_passes(C (&v)[NF][8], C* sm, int fstride, co
       const int k = j % Ns;
 #pragma unroll
       for (int q = 1; q < r; ++q) {
-        const C w = tw[q * k * STW];
+        const TW w = tw[q * k * STW];
 #pragma unroll
         for (int f = 0; f < NF; ++f) v[f][b * r + q] = INV ? cmulc(v[f][b * r + q], w) : cmul(v[f][b * r + q], w);
       }
@@ -243,7 +459,7 @@ __device__ __forceinline__ void fft_passes(C (&v)[NF][8], C* sm, int fstride, co
       }
     }
     if constexpr (!PingPong<SI>::v) line_sync<SI>();
-    fft_passes<C, L, INV, NF, p + 1, SI>(v, sm, fstride, tw, t, si);
+    fft_passes<C, L, INV, NF, p + 1, SI, TW>(v, sm, fstride, tw, t, si);
   }
 }
 
@@ -251,8 +467,8 @@ __device__ __forceinline__ void fft_passes(C (&v)[NF][8], C* sm, int fstride, co
 // pass are spread over the line's L/8 threads (some threads idle when they do
 // not divide evenly); each thread reads all inputs of its butterflies before
 // the block synchronises and the outputs overwrite them in place.
-template <class C, int L, bool INV, int NF, int p, class SI>
-__device__ __forceinline__ void fft_mixed_passes(C* sm, int fstride, const C* __restrict__ tw, int t, const SI& si) {
+template <class C, int L, bool INV, int NF, int p, class SI, class TW>
+__device__ __forceinline__ void fft_mixed_passes(C* sm, int fstride, const TW* __restrict__ tw, int t, const SI& si) {
   using PL = MixedPlan<L>;
   constexpr int r = PL::rad(p);
   constexpr int Ns = PL::ns(p);
@@ -278,7 +494,7 @@ __device__ __forceinline__ void fft_mixed_passes(C* sm, int fstride, const C* __
         const int k = j % Ns;
 #pragma unroll
         for (int q = 1; q < r; ++q) {
-          const C tq = tw[q * k * STW];
+          const TW tq = tw[q * k * STW];
           w[b][q] = INV ? cmulc(w[b][q], tq) : cmul(w[b][q], tq);
         }
         dft_r<r, INV>(w[b]);
@@ -289,15 +505,15 @@ __device__ __forceinline__ void fft_mixed_passes(C* sm, int fstride, const C* __
     }
     __syncthreads();
   }
-  if constexpr (p + 1 < PL::P) fft_mixed_passes<C, L, INV, NF, p + 1, SI>(sm, fstride, tw, t, si);
+  if constexpr (p + 1 < PL::P) fft_mixed_passes<C, L, INV, NF, p + 1, SI, TW>(sm, fstride, tw, t, si);
 }
 
 // Mixed-radix line transform with natural entry and exit layouts (register e
 // of thread t holds position t + e L/8): the radix-8 first pass runs on the
 // registers as loaded, the later passes in shared memory, and the result is
 // read back in the same layout.
-template <class C, int L, bool INV, int NF, class SI>
-__device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, const C* __restrict__ tw, int t,
+template <class C, int L, bool INV, int NF, class SI, class TW>
+__device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, const TW* __restrict__ tw, int t,
                                           const SI& si) {
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
@@ -306,7 +522,7 @@ __device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, con
     for (int q = 0; q < 8; ++q) sm[f * fstride + si(8 * t + q)] = v[f][q];
   }
   __syncthreads();
-  fft_mixed_passes<C, L, INV, NF, 1, SI>(sm, fstride, tw, t, si);
+  fft_mixed_passes<C, L, INV, NF, 1, SI, TW>(sm, fstride, tw, t, si);
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
@@ -317,8 +533,26 @@ __device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, con
 template <class C, int L, bool INV, int NF, class SI>
 __device__ __forceinline__ void fft_line(C (&v)[NF][8], C* sm, int fstride, const C* __restrict__ tw, int t,
                                          const SI& si) {
-  if constexpr (IsPow2<L>::v) fft_passes<C, L, INV, NF, 0, SI>(v, sm, fstride, tw, t, si);
-  else fft_mixed<C, L, INV, NF, SI>(v, sm, fstride, tw, t, si);
+  if constexpr (std::is_same<C, double2>::value) {
+    Q2* qs = reinterpret_cast<Q2*>(sm);
+    const TwQ* qt = reinterpret_cast<const TwQ*>(tw);
+    Q2 q[NF][8];
+    LineScale ls[NF];
+    line_scales<L, NF>(v, sm, fstride, t, si, ls);
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) q[f][e] = Q2{to_fixed(v[f][e].x, ls[f]), to_fixed(v[f][e].y, ls[f])};
+    if constexpr (IsPow2<L>::v) fft_passes<Q2, L, INV, NF, 0, SI, TwQ>(q, qs, fstride, qt, t, si);
+    else fft_mixed<Q2, L, INV, NF, SI, TwQ>(q, qs, fstride, qt, t, si);
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[f][e] = make_double2(from_fixed(q[f][e].x, ls[f]), from_fixed(q[f][e].y, ls[f]));
+  } else {
+    if constexpr (IsPow2<L>::v) fft_passes<C, L, INV, NF, 0, SI, C>(v, sm, fstride, tw, t, si);
+    else fft_mixed<C, L, INV, NF, SI, C>(v, sm, fstride, tw, t, si);
+  }
 }
 
 // Shared-memory index maps.  Row tiles (lines contiguous in global memory):
@@ -334,9 +568,15 @@ template <int PADSHIFT> struct RowIdx {
 // MC = 0: M at run time (the other tile widths).
 template <int MC> struct ColIdxT {
   int M;
-  int alt;  // offset (elements) of the second exchange buffer from the first
-  __device__ __forceinline__ int operator()(int pos) const { return pos * (MC > 0 ? MC : M); }
+  int alt;    // offset (elements) of the second exchange buffer from the first
+  uint2* sc;  // this column's slots of the FP64 line scales, one per thread of the line, M apart
+  __device__ __forceinline__ int width() const { return MC > 0 ? MC : M; }
+  __device__ __forceinline__ int operator()(int pos) const { return pos * width(); }
 };
+// Bytes of those slots in a column block of `threads` threads (FP64 only).
+template <class R> __host__ __device__ constexpr size_t line_slots(int threads) {
+  return sizeof(R) == sizeof(double) ? (size_t)threads * sizeof(uint2) : 0;
+}
 using ColIdx = ColIdxT<0>;
 // A column transform of power-of-two length L makes P - 1 exchanges, the first
 // through the second buffer.  When that count is odd the transform ends having

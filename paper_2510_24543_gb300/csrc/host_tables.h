@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -23,6 +24,24 @@ template <class R> inline void twiddle_table(int L, C2<R>* out) {
   for (int m = 0; m < L; ++m) {
     const long double ang = 2.0L * pi * (long double)m / (long double)L;
     out[m] = cmk<C2<R>>((R)cosl(ang), (R)(-sinl(ang)));
+  }
+}
+
+// FP64 transforms run in fixed point (fft.cuh): cos and -sin to 62 fractional
+// bits as two signed 32-bit limbs each, in the storage of a double2.
+template <> inline void twiddle_table<double>(int L, double2* out) {
+  const long double pi = 3.141592653589793238462643383279502884L;
+  auto limbs = [](long double v, int& h, int& l) {
+    const long long q = llroundl(v * 4611686018427387904.0L);  // 2^62
+    h = (int)((q + (1ll << 31)) >> 32);
+    l = (int)(q - ((long long)h << 32));
+  };
+  for (int m = 0; m < L; ++m) {
+    const long double ang = 2.0L * pi * (long double)m / (long double)L;
+    int w[4];
+    limbs(cosl(ang), w[0], w[1]);
+    limbs(-sinl(ang), w[2], w[3]);
+    std::memcpy((void*)&out[m], w, sizeof(w));
   }
 }
 

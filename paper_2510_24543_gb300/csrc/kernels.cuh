@@ -304,7 +304,8 @@ template <class Op, int MC> __device__ __forceinline__ void colpass_body(const K
   extern __shared__ __align__(16) unsigned char smraw[];
   C* tw = reinterpret_cast<C*>(smraw);
   C* buf = tw + L;  // two exchange buffers of M lines each
-  RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(buf + 2 * M * L);
+  uint2* slots = reinterpret_cast<uint2*>(buf + 2 * M * L);
+  RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(reinterpret_cast<unsigned char*>(slots) + line_slots<R>(M * (L / 8)));
   const int tid = threadIdx.x;
   const int m = tid % M, t = tid / M;
   const C* twsrc = (Op::AXIS == 1) ? a.twy : a.twz;
@@ -328,7 +329,7 @@ template <class Op, int MC> __device__ __forceinline__ void colpass_body(const K
     C v[1][8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[0][e] = src[base + (size_t)Plan<L>::entry_pos(Op::FIRST_INV, t, e) * lstride];
-    Op::process(a, u, f, x, o, base, lstride, t, v, buf + m, tw, ColIdxT<MC>{M, M * L}, acc);
+    Op::process(a, u, f, x, o, base, lstride, t, v, buf + m, tw, ColIdxT<MC>{M, M * L, slots + m}, acc);
     // the last exchange's reads end before the next tile's first writes
     if constexpr (IsPow2<L>::v) __syncthreads();
   }
@@ -372,7 +373,8 @@ __device__ __forceinline__ void colpass_tma_body(const CUtensorMap* tm, const KA
   C* xbuf = tiles + NST * tileC;
   C* tw = xbuf + tileC;
   uint64_t* bar = reinterpret_cast<uint64_t*>(tw + L);
-  RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(bar + NST);
+  uint2* slots = reinterpret_cast<uint2*>(bar + NST);
+  RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(reinterpret_cast<unsigned char*>(slots) + line_slots<R>(M * (L / 8)));
   const int tid = threadIdx.x;
   const int m = tid % M, t = tid / M;
   const C* twsrc = (Op::AXIS == 1) ? a.twy : a.twz;
@@ -438,7 +440,7 @@ __device__ __forceinline__ void colpass_tma_body(const CUtensorMap* tm, const KA
     const int f = a.f0 + rest / other_n;
     const int x = xb * M + m;
     const size_t base = (size_t)f * a.N + (Op::AXIS == 1 ? (size_t)o * a.nx * a.ny : (size_t)o * a.nx) + x;
-    Op::process(a, u, f, x, o, base, lstride, t, v, tb + m, tw, ColIdxT<MC>{M, (int)(xbuf - tb)}, acc);
+    Op::process(a, u, f, x, o, base, lstride, t, v, tb + m, tw, ColIdxT<MC>{M, (int)(xbuf - tb), slots + m}, acc);
     __syncthreads();  // buffer b may be refilled, and the second buffer rewritten, from here on
   }
   if (timed_out) {
