@@ -214,6 +214,7 @@ static_assert(sizeof(Q2) == sizeof(double2) && sizeof(TwQ) == sizeof(double2), "
 // leading zeros are lz gets the biased exponent X + 1 - lz.
 struct LineScale {
   int X;
+  int keep;  // 0 for a line that is taken as 0: clears the signs of its values too
   int bad;  // bits or-ed into the outputs' high words: a NaN pattern for a line that is not finite
 };
 
@@ -224,8 +225,8 @@ __device__ __forceinline__ long long to_fixed(double d, const LineScale& ls) {
   const int r = min(ls.X - e, 63);  // zeros (e = 0) leave by the clamp
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 10;
-  const long long s = (long long)(hi >> 31);
-  return (long long)(m >> r) ^ s;
+  const long long s = (long long)((hi >> 31) & ls.keep);
+  return (long long)(m >> r) ^ s;  // floor: ones' complement of a negative value's magnitude
 }
 __device__ __forceinline__ double from_fixed(long long q, const LineScale& ls) {
   const int sg = (int)(q >> 32) >> 31;
@@ -265,6 +266,7 @@ __device__ __forceinline__ LineScale make_scale(uint2 b) {
   const int E = (int)b.x;
   LineScale s;
   s.X = E < 64 ? 4096 : E + (32 - __clz((int)b.y)) - 20;
+  s.keep = E < 64 ? 0 : -1;
   s.bad = E >= 2036 ? 0x7ff80000 : 0;
   return s;
 }

@@ -74,3 +74,13 @@ def test_zero_and_nonfinite(n):
         y = _field(n, 4)
         y[0, 1, 2, 3] = bad
         assert np.all(np.isnan(_fft(n, y, False)))
+
+
+@pytest.mark.parametrize("n", [(16, 32, 48), (80, 16, 16)])
+@pytest.mark.parametrize("tiny", [-1e-300, -0.0, -5e-324])
+def test_lines_below_the_range(n, tiny):
+    """Negative values below 2^-960 are zeros: alone, and in lines beside ordinary ones."""
+    x = np.full((1, n[2], n[1], n[0]), tiny + 1j * tiny)
+    assert not np.any(_fft(n, x, False))
+    x[0, 4, 3] = _field(n, 5)[0, 4, 3]
+    assert _err(_fft(n, x, False), x, False) < TOL
