@@ -27,6 +27,12 @@ template <class C> __device__ __forceinline__ C cmulc(C a, C b) {
   return cmk<C>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 template <class C, class R> __device__ __forceinline__ C cscale(C a, R s) { return cmk<C>(a.x * s, a.y * s); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+// s += Re(conj(a) b) in two FMAs.
+template <class C, class R> __device__ __forceinline__ void cdot_add(R& s, C a, C b) {
+  s = fma_(a.x, b.x, fma_(a.y, b.y, s));
+}
 // Re(conj(a) b)
 template <class C> __device__ __forceinline__ auto cdot(C a, C b) -> decltype(a.x) { return a.x * b.x + a.y * b.y; }
 template <class C> __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x) { return a.x * a.x + a.y * a.y; }
@@ -34,8 +40,9 @@ template <class C> __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x) {
 // ---------------------------------------------------------------------------
 // Scalar slots written by the deterministic reductions (FP64 always).
 // ---------------------------------------------------------------------------
-enum EgSlot {  // pointwise part of one energy/gradient evaluation (x dV later)
-  EG_TRAP = 0, EG_CONTACT, EG_DIPOLAR, EG_LHY, EG_MU1, EG_MU2, EG_NPHI1, EG_NPHI2,
+enum EgSlot {  // pointwise part of one energy/gradient evaluation (x dV later):
+  // int of n_i V, n_i sum_j g_ij n_j, n_i Phi_i, n_i mu_LHY,i, n_i
+  EG_TRAP1 = 0, EG_TRAP2, EG_CON1, EG_CON2, EG_NPHI1, EG_NPHI2,
   EG_NMUL1, EG_NMUL2, EG_NORM1, EG_NORM2, EG_NS
 };
 enum EgzSlot { EGZ_KIN1 = 0, EGZ_KIN2, EGZ_NS };  // Parseval sums of the z pass

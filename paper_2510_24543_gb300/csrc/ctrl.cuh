@@ -25,19 +25,21 @@ struct EnergyOut {
   double E, kin[2], trap, contact, dipolar, lhy, mu[2], norm2[2], shift[2], nmuL[2];
 };
 
-// Energy terms from the raw sums of one evaluation (sums are over grid points;
-// the kinetic sums are Parseval sums of |k|^2/2 |psi^|^2 over the unnormalised DFT).
-__host__ __device__ inline void finalize_energy(const double* eg, const double* egz, double dV, double invN,
-                                                EnergyOut& o) {
-  o.kin[0] = egz[EGZ_KIN1] * dV * invN;
-  o.kin[1] = egz[EGZ_KIN2] * dV * invN;
-  o.trap = eg[EG_TRAP] * dV;
-  o.contact = eg[EG_CONTACT] * dV;
-  o.dipolar = eg[EG_DIPOLAR] * dV;
-  o.lhy = eg[EG_LHY] * dV;
+// Energy terms and chemical potentials from the raw sums of one evaluation
+// (sums over grid points; the kinetic sums are Parseval sums of
+// |k|^2/(2N) |psi^|^2 over the unnormalised DFT): every term of
+// mu_i = <psi_i, (T + V + sum_j g_ij n_j + Phi_i + mu_LHY,i) psi_i> is one sum, the
+// contact and dipolar energies are half of theirs and the LHY energy 2/5 (Euler).
+__host__ __device__ inline void finalize_energy(const double* eg, const double* egz, double dV, EnergyOut& o) {
+  o.trap = (eg[EG_TRAP1] + eg[EG_TRAP2]) * dV;
+  o.contact = 0.5 * (eg[EG_CON1] + eg[EG_CON2]) * dV;
+  o.dipolar = 0.5 * (eg[EG_NPHI1] + eg[EG_NPHI2]) * dV;
+  o.lhy = 0.4 * (eg[EG_NMUL1] + eg[EG_NMUL2]) * dV;
+  for (int i = 0; i < 2; ++i) {
+    o.kin[i] = egz[EGZ_KIN1 + i] * dV;
+    o.mu[i] = o.kin[i] + (eg[EG_TRAP1 + i] + eg[EG_CON1 + i] + eg[EG_NPHI1 + i] + eg[EG_NMUL1 + i]) * dV;
+  }
   o.E = o.kin[0] + o.kin[1] + o.trap + o.contact + o.dipolar + o.lhy;
-  o.mu[0] = eg[EG_MU1] * dV;
-  o.mu[1] = eg[EG_MU2] * dV;
   o.norm2[0] = eg[EG_NORM1] * dV;
   o.norm2[1] = eg[EG_NORM2] * dV;
   // alpha_i = mu_i - Re<psi_i, Phi_i psi_i>  (preconditioner shift)
@@ -57,12 +59,12 @@ struct LineOut {
 // which regroups the paper's E'_i, E''_ij, E'_LHY, E''_LHY (Sec. V): the n''
 // terms of E''_LHY combine with the H_MF terms into the full H_i (incl. mu_LHY).
 __host__ __device__ inline void finalize_line(const double* lc, const double* lcz, const double mu[2], double dV,
-                                              double invN, LineOut& o) {
+                                              LineOut& o) {
   double Epp = 0.0;
   for (int i = 0; i < 2; ++i) {
     o.pnorm2[i] = lc[LC_P1 + i] * dV;
     o.psip[i] = lc[LC_PSIP1 + i] * dV;
-    const double tpp = lcz[LCZ_TPP1 + i] * dV * invN;
+    const double tpp = lcz[LCZ_TPP1 + i] * dV;
     const double upp = lc[LC_UPP1 + i] * dV;
     Epp += 2.0 * (-o.pnorm2[i] * mu[i] + tpp + upp);
   }
@@ -104,7 +106,7 @@ __device__ inline bool ctrl_timed_out(DevState* st) {
 
 __device__ inline void load_point(DevState* st, int slot) {
   EnergyOut o;
-  finalize_energy(st->eg[slot], st->egz[slot], st->dV, st->invN, o);
+  finalize_energy(st->eg[slot], st->egz[slot], st->dV, o);
   st->E = o.E;
   for (int i = 0; i < 2; ++i) {
     st->mu[i] = o.mu[i];
@@ -114,9 +116,12 @@ __device__ inline void load_point(DevState* st, int slot) {
   }
 }
 
+// The controller steps are not inlined: one thread of the grid runs them, and
+// inside a pass their FP64 chains would set its register count.
+
 // After an energy/gradient evaluation.  mode 0: evaluation of the current
 // point (start of a solve, or a standalone call); mode 1: trial point.
-__device__ inline void ctrl_after_eg(DevState* st, int mode, TraceDev* trace) {
+static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, TraceDev* trace) {
   if (ctrl_timed_out(st)) return;
   if (mode == 0) {
     load_point(st, st->cur);
@@ -126,7 +131,7 @@ __device__ inline void ctrl_after_eg(DevState* st, int mode, TraceDev* trace) {
   }
   const int slot = st->cur ^ 1;
   EnergyOut o;
-  finalize_energy(st->eg[slot], st->egz[slot], st->dV, st->invN, o);
+  finalize_energy(st->eg[slot], st->egz[slot], st->dV, o);
   st->attempts += 1;
   st->E_trial = o.E;
   const SolveOptsDev& op = st->opt;
@@ -186,7 +191,7 @@ __device__ inline void ctrl_after_eg(DevState* st, int mode, TraceDev* trace) {
 
 // End of one imaginary-time step: the energy of the renormalised state, the
 // |E^{k+1} - E^k| < tol_dE stopping rule of the ITE comparison (Sec. VI.A).
-__device__ inline void ctrl_after_ite(DevState* st) {
+static __device__ __noinline__ void ctrl_after_ite(DevState* st) {
   if (ctrl_timed_out(st)) return;
   const double Eold = st->E;
   load_point(st, st->cur);
@@ -206,7 +211,7 @@ __device__ inline void ctrl_after_ite(DevState* st) {
 
 // After the preconditioned residual and its sums: convergence test, beta,
 // projection coefficients, restart rules.
-__device__ inline void ctrl_after_pc(DevState* st) {
+static __device__ __noinline__ void ctrl_after_pc(DevState* st) {
   if (ctrl_timed_out(st)) return;
   const double* pc = st->pc;
   const double dV = st->dV;
@@ -276,10 +281,10 @@ __device__ inline void ctrl_after_pc(DevState* st) {
 }
 
 // After the line-search sums: E', E'', alpha, theta, retraction coefficients.
-__device__ inline void ctrl_after_lc(DevState* st) {
+static __device__ __noinline__ void ctrl_after_lc(DevState* st) {
   if (ctrl_timed_out(st)) return;
   LineOut o;
-  finalize_line(st->lc, st->lcz, st->mu, st->dV, st->invN, o);
+  finalize_line(st->lc, st->lcz, st->mu, st->dV, o);
   st->Ep = o.Ep;
   st->Epp = o.Epp;
   st->pnorm2[0] = o.pnorm2[0];

@@ -216,6 +216,7 @@ template <class R> class Engine {
   LhyNode<R>* xnodes_ = nullptr;    // nodes evaluated exactly beside the LHY table
   R* tab_ = nullptr;                // LHY interpolation table (host_tables.h)
   size_t tab_elems_ = 0;
+  R* axis_tab_ = nullptr;           // k_a^2/(2N), then lambda_a^2 x_a^2/2, per index of x, y, z
   double* partials_ = nullptr;
   unsigned* counter_ = nullptr;
   DevState* st_ = nullptr;

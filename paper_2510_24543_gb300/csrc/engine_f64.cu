@@ -38,6 +38,7 @@ namespace {
 constexpr int kNoAllocMaxN = 32;                         // points per axis
 constexpr size_t kNoAllocMaxPoints = 32 * 32 * 32;
 constexpr size_t kNoAllocBlocks = 1024;                  // partial-sum slots
+constexpr int kNoAllocSMs = 152;                         // SMs the row passes are spread over
 constexpr size_t kNoAllocBytes = (size_t)4 << 20;        // 4 MiB
 
 constexpr size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -49,7 +50,8 @@ constexpr size_t kOffSt = al256(kOffPart + kNoAllocBlocks * egpe::MAX_NS * sizeo
 constexpr size_t kOffCnt = al256(kOffSt + sizeof(egpe::DevState));
 constexpr size_t kOffTw = al256(kOffCnt + 64 * sizeof(unsigned));
 constexpr size_t kOffNodes = al256(kOffTw + 3 * kNoAllocMaxN * sizeof(double2));
-constexpr size_t kOffEnd = al256(kOffNodes + 64 * sizeof(egpe::LhyNode<double>));
+constexpr size_t kOffAxes = al256(kOffNodes + 64 * sizeof(egpe::LhyNode<double>));
+constexpr size_t kOffEnd = al256(kOffAxes + 6 * kNoAllocMaxN * sizeof(double));
 static_assert(kOffEnd <= kNoAllocBytes, "no-alloc scratch layout exceeds its array");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
@@ -74,17 +76,14 @@ cudaError_t noalloc_scratch(int dev, unsigned char** out) {
 
 template <class Op> cudaError_t noalloc_launch_x(egpe::KArgs<double> a, int rows, cudaStream_t s) {
   using namespace egpe;
-  constexpr int L = Op::L, TPL = L / 8, NF = Op::NF, NS = Op::NS;
-  constexpr int LP = row_len_padded<double, L>();
-  const size_t rowbytes = (size_t)NF * LP * sizeof(double2);
-  int mx = whole_warp_rows(L);
-  while ((mx * 2) * TPL <= MaxThreads<Op>::v && (size_t)(mx * 2) * rowbytes <= 46 * 1024) mx *= 2;
+  constexpr int L = Op::L, NS = Op::NS;
+  const int mx = default_rows<Op>(rows, kNoAllocSMs);
   a.MX = mx;
   const size_t smem = L * sizeof(double2) + (Op::USES_LHY ? lhy_stage_bytes<double>(a.Q) : 0) +
-                      mx * rowbytes + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
+                      mx * row_pass_bytes<Op>() + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
   const int groups = (rows + mx - 1) / mx;
   const int grid = std::min(groups, (int)kNoAllocBlocks);
-  xpass_kernel<Op><<<grid, mx * TPL, smem, s>>>(a);
+  xpass_kernel<Op><<<grid, mx * RowGroups<Op>::v * L / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -191,6 +190,14 @@ extern "C" egpe_status egpe_energy_grad_noalloc(const egpe_grid* grid, const egp
       return EGPE_ERR_CUDA;
     }
   }
+  double axes[6 * kNoAllocMaxN];
+  axis_tables<double>(g, p, axes);
+  const int na = nx + ny + nz;
+  ce = cudaMemcpyAsync(base + kOffAxes, axes, 2 * na * sizeof(double), cudaMemcpyHostToDevice, s);
+  if (ce != cudaSuccess) {
+    set_error("cudaMemcpyAsync", ce);
+    return EGPE_ERR_CUDA;
+  }
   ce = cudaMemcpyAsync(base + kOffNodes, nodes, p.lhy_nodes * sizeof(LhyNode<double>), cudaMemcpyHostToDevice, s);
   // the previous call's state and arrival counter must not leak into this one
   if (ce == cudaSuccess) ce = cudaMemsetAsync(base + kOffSt, 0, kOffTw - kOffSt, s);
@@ -202,7 +209,6 @@ extern "C" egpe_status egpe_energy_grad_noalloc(const egpe_grid* grid, const egp
   KArgs<double> a;
   std::memset((void*)&a, 0, sizeof(a));
   const double hx = 2.0 * g.L[0] / nx, hy = 2.0 * g.L[1] / ny, hz = 2.0 * g.L[2] / nz;
-  const double dpi = 3.14159265358979323846;
   a.nx = nx;
   a.ny = ny;
   a.nz = nz;
@@ -213,12 +219,9 @@ extern "C" egpe_status egpe_energy_grad_noalloc(const egpe_grid* grid, const egp
   a.Lx = g.L[0];
   a.Ly = g.L[1];
   a.Lz = g.L[2];
-  a.dkx = dpi / g.L[0];
-  a.dky = dpi / g.L[1];
-  a.dkz = dpi / g.L[2];
+  a.kq = (const double*)(base + kOffAxes);
+  a.vt = a.kq + na;
   a.vx = 0.5 * p.trap[0] * p.trap[0];
-  a.vy = 0.5 * p.trap[1] * p.trap[1];
-  a.vz = 0.5 * p.trap[2] * p.trap[2];
   a.g11 = p.g[0][0];
   a.g12 = p.g[0][1];
   a.g21 = p.g[1][0];
@@ -272,7 +275,7 @@ extern "C" egpe_status egpe_energy_grad_noalloc(const egpe_grid* grid, const egp
     return EGPE_ERR_CUDA;
   }
   EnergyOut o;
-  finalize_energy(sums, sums + EG_NS, hx * hy * hz, 1.0 / (double)N, o);
+  finalize_energy(sums, sums + EG_NS, hx * hy * hz, o);
   if (E) *E = o.E;
   if (mu) {
     mu[0] = o.mu[0];

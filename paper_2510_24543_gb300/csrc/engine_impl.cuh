@@ -158,8 +158,15 @@ template <class R> egpe_status Engine<R>::apply_params(const egpe_params& p) {
   a.tab.ni = T.ni;
   a.tab.tscale = (R)(T.ni * 1.4142135623730950488);
   a.vx = (R)(0.5 * p.trap[0] * p.trap[0]);
-  a.vy = (R)(0.5 * p.trap[1] * p.trap[1]);
-  a.vz = (R)(0.5 * p.trap[2] * p.trap[2]);
+  {
+    const int na = nx + ny + nz;
+    std::vector<R> ax(2 * na);
+    axis_tables<R>(grid_, p, ax.data());
+    if (!axis_tab_) EGPE_CUDA(cudaMalloc(&axis_tab_, ax.size() * sizeof(R)));
+    EGPE_CUDA(cudaMemcpy(axis_tab_, ax.data(), ax.size() * sizeof(R), cudaMemcpyHostToDevice));
+    a.kq = axis_tab_;
+    a.vt = axis_tab_ + na;
+  }
   a.g11 = (R)p.g[0][0];
   a.g12 = (R)p.g[0][1];
   a.g21 = (R)p.g[1][0];
@@ -276,10 +283,6 @@ template <class R> egpe_status Engine<R>::create(const egpe_grid& g, const egpe_
   a.Lx = (R)g.L[0];
   a.Ly = (R)g.L[1];
   a.Lz = (R)g.L[2];
-  const double pi = 3.14159265358979323846;
-  a.dkx = (R)(pi / g.L[0]);
-  a.dky = (R)(pi / g.L[1]);
-  a.dkz = (R)(pi / g.L[2]);
   a.invN = (R)(1.0 / (double)N);
   EGPE_TRY(apply_params(p));
   a.twx = twx_;
@@ -343,6 +346,7 @@ template <class R> void Engine<R>::destroy() {
   if (nodes_) cudaFree(nodes_);
   if (xnodes_) cudaFree(xnodes_);
   if (tab_) cudaFree(tab_);
+  if (axis_tab_) cudaFree(axis_tab_);
   if (partials_) cudaFree(partials_);
   if (counter_) cudaFree(counter_);
   if (st_) cudaFree(st_);
@@ -355,6 +359,7 @@ template <class R> void Engine<R>::destroy() {
   xnodes_ = nullptr;
   tab_ = nullptr;
   tab_elems_ = 0;
+  axis_tab_ = nullptr;
   partials_ = nullptr;
   counter_ = nullptr;
   st_ = nullptr;
@@ -599,7 +604,7 @@ egpe_status Engine<R>::autotune(const C* psi, int precond, int reps, std::vector
     std::vector<int> cand;
     if (r.kind == 0) {
       for (int mx = r.mx; mx >= 1; mx /= 2)
-        if ((mx * r.tpl) % 32 == 0) cand.push_back(mx);  // whole warps only
+        if (mx % whole_warp_rows(r.L) == 0) cand.push_back(mx);  // whole warps only
       const int up = r.mx * 2;
       if (up * r.tpl <= r.max_threads && (size_t)up * r.rowbytes + r.smem_fixed <= 200 * 1024) cand.push_back(up);
     } else {
@@ -678,25 +683,25 @@ egpe_status Engine<R>::launch_point(void (*kern)(KArgs<R>), void (*kern_b)(KBatc
 }
 
 template <class R> template <class Op> egpe_status Engine<R>::launch_x(KArgs<R> a) {
-  constexpr int L = Op::L, TPL = L / 8, NF = Op::NF, NS = Op::NS;
-  constexpr int LP = row_len_padded<R, L>();
-  const size_t rowbytes = (size_t)NF * LP * sizeof(C);
-  int mx = whole_warp_rows(L);
-  while ((mx * 2) * TPL <= MaxThreads<Op>::v && (size_t)(mx * 2) * rowbytes <= 46 * 1024) mx *= 2;
-  const int mx_default = mx;
+  // TPL: threads of one row
+  constexpr int L = Op::L, NS = Op::NS, TPL = RowGroups<Op>::v * L / 8;
+  const size_t rowbytes = row_pass_bytes<Op>();
+  const size_t smem_fixed =
+      L * sizeof(C) + (Op::USES_LHY ? lhy_stage_bytes<R>(a.Q) : 0) + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
+  const int rows = ny * nz;
+  const int mx_default = default_rows<Op>(rows, nsm_);
+  int mx = mx_default;
   if (!tune_.empty()) {
     auto it = tune_.find(typeid(Op).name());
     if (it != tune_.end() && it->second >= 1 && it->second * TPL <= MaxThreads<Op>::v &&
-        (it->second * TPL) % 32 == 0 && (size_t)it->second * rowbytes <= 200 * 1024)
+        (it->second * TPL) % 32 == 0 && it->second % whole_warp_rows(L) == 0 &&
+        (size_t)it->second * rowbytes <= 200 * 1024)
       mx = it->second;
   }
   a.MX = mx;
   const int block = mx * TPL;
   EGPE_TRY(check_whole_warps(Op::NAME, L, block));
-  const size_t smem_fixed =
-      L * sizeof(C) + (Op::USES_LHY ? lhy_stage_bytes<R>(a.Q) : 0) + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
   const size_t smem = smem_fixed + mx * rowbytes;
-  const int rows = ny * nz;
   const int groups = (rows + mx - 1) / mx;
   void (*kern)(KArgs<R>);
   if constexpr (MinBlocks<Op>::v > 1) kern = xpass_kernel_mb<Op>;
@@ -982,7 +987,7 @@ template <class R> egpe_status Engine<R>::energy_grad(const C* psi, egpe_energy_
   EGPE_TRY(read_state(hs));
   if (out) {
     EnergyOut o;
-    finalize_energy(hs.eg[0], hs.egz[0], hs.dV, hs.invN, o);
+    finalize_energy(hs.eg[0], hs.egz[0], hs.dV, o);
     out->E = o.E;
     for (int i = 0; i < 2; ++i) {
       out->kin[i] = o.kin[i];
@@ -1006,7 +1011,7 @@ template <class R> egpe_status Engine<R>::line_coeffs(const C* psi, const C* p, 
   DevState hs;
   EGPE_TRY(read_state(hs));
   LineOut o;
-  finalize_line(hs.lc, hs.lcz, hs.mu, hs.dV, hs.invN, o);
+  finalize_line(hs.lc, hs.lcz, hs.mu, hs.dV, o);
   coeffs[0] = t.E;
   coeffs[1] = o.Ep;
   coeffs[2] = o.Epp;

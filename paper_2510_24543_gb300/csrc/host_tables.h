@@ -45,6 +45,23 @@ template <> inline void twiddle_table<double>(int L, double2* out) {
   }
 }
 
+// Per-index tables of the grid's axes, x then y then z: k_a^2/(2N) with
+// k_a = (pi/L_a)(j or j - n_a), then lambda_a^2 x_a^2/2 with x_a = -L_a + j h_a.
+template <class R> inline void axis_tables(const egpe_grid& g, const egpe_params& p, R* out) {
+  const int na = g.n[0] + g.n[1] + g.n[2];
+  const long double pi = 3.141592653589793238462643383279502884L;
+  const long double inv2n = 0.5L / ((long double)g.n[0] * g.n[1] * g.n[2]);
+  for (int a = 0, o = 0; a < 3; o += g.n[a++]) {
+    const int n = g.n[a];
+    for (int j = 0; j < n; ++j) {
+      const long double k = pi / g.L[a] * (j < n / 2 ? j : j - n);
+      const long double x = -(long double)g.L[a] + j * (2.0L * g.L[a] / n);
+      out[o + j] = (R)(k * k * inv2n);
+      out[na + o + j] = (R)(0.5L * p.trap[a] * p.trap[a] * x * x);
+    }
+  }
+}
+
 // Legendre polynomial P_Q(x) and its predecessor P_{Q-1}(x) by the three-term
 // recurrence (P_0 = 1, P_1 = x).
 inline void legendre_pq(int Q, long double x, long double& pq, long double& pq1) {

@@ -20,29 +20,15 @@
 #include "reduce.cuh"
 #include "tma.cuh"
 
-// Resident blocks per SM asked of the FP32 x-inverse epilogue passes, which
-// caps their registers: energy 4 x 128 threads (128 registers, no spills),
-// line coefficients 2 x 256 (128 registers, a few spilled bytes),
-// preconditioner 1 (at 128 registers it spills ~250 bytes).  At 128^3 the
-// energy pass went from 55.5 to 49.5 us and the line pass from 59 to 57 us.
-#ifndef EGPE_EG_MINB
-#define EGPE_EG_MINB 4
-#endif
-#ifndef EGPE_LC_MINB
-#define EGPE_LC_MINB 2
-#endif
-#ifndef EGPE_PC_MINB
-#define EGPE_PC_MINB 1
-#endif
-
 namespace egpe {
 
 template <class R> struct KArgs {
   using C = C2<R>;
   int nx, ny, nz, N;
   R hx, hy, hz, Lx, Ly, Lz;
-  R dkx, dky, dkz;           // pi / L_a
-  R vx, vy, vz;              // lambda_a^2 / 2
+  const R* kq;               // k_a^2 / (2 N) per index: [nx] x, [ny] y, [nz] z
+  const R* vt;               // lambda_a^2 x_a^2 / 2 per index, same layout
+  R vx;                      // lambda_x^2 / 2
   R g11, g12, g21, g22;      // contact couplings
   R d11, d12, d21, d22;      // k-space dipolar coefficients
   R invN;
@@ -101,12 +87,6 @@ template <class R> struct ChunkW;
 template <> struct ChunkW<float> { static constexpr int v = 4; };
 template <> struct ChunkW<double> { static constexpr int v = 2; };
 
-// Grid points evaluated together in the LHY node loops (independent chains;
-// FP32: two pairs of packed lanes).
-template <class R> struct LhyNP;
-template <> struct LhyNP<float> { static constexpr int v = 4; };
-template <> struct LhyNP<double> { static constexpr int v = 2; };
-
 template <class R> __device__ __forceinline__ LhyCoef<R> lhy_coef(const KArgs<R>& a) {
   LhyCoef<R> c;
   c.g11 = a.g11;
@@ -119,26 +99,38 @@ template <class R> __device__ __forceinline__ LhyCoef<R> lhy_coef(const KArgs<R>
   return c;
 }
 
-template <class R> __device__ __forceinline__ R wavenum(int j, int n, R dk) {
-  return dk * (R)(j < (n >> 1) ? j : j - n);
+// One of a pair, by a select: a run-time index would put the pair in local memory.
+template <class T> __device__ __forceinline__ T pick(const T (&p)[2], int i) { return i ? p[1] : p[0]; }
+
+// Terms of the trap and of |k|^2/2 (over N) that depend on one index come from
+// tables: forming them per point took an integer conversion and three products in
+// each of a dozen places, on the FP64 pipe of the FP64 kernels.  FP32 kernels form
+// the trap's x term (the load's latency costs them more: line pass 57 against 54 us).
+template <class R> __device__ __forceinline__ R trap_x(const KArgs<R>& a, int x) {
+  if constexpr (sizeof(R) == 8) {
+    return a.vt[x];
+  } else {
+    const R X = fma_((R)x, a.hx, -a.Lx);
+    return a.vx * X * X;
+  }
 }
-
-// Row-pass ops that read their transform outputs back from shared memory.
-template <class Op, class = void> struct StageOut {
-  static constexpr bool v = false;
+template <class R> __device__ __forceinline__ R trap_yz(const KArgs<R>& a, int row) {
+  const int y = row % a.ny, z = row / a.ny;
+  return a.vt[a.nx + y] + a.vt[a.nx + a.ny + z];
+}
+template <class R> __device__ __forceinline__ R kq_xy(const KArgs<R>& a, int x, int y) { return __ldg(a.kq + x) + __ldg(a.kq + a.nx + y); }
+// k_z^2/(2N) at a thread's positions of a z line (the same in every tile).
+template <class R, int L> struct KzLine {
+  R kz[8];
+  __device__ __forceinline__ void set(const KArgs<R>& a, int t) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) kz[e] = a.kq[a.nx + a.ny + Plan<L>::exit_pos(false, t, e)];
+  }
 };
-template <class Op> struct StageOut<Op, std::void_t<decltype(Op::STAGE_OUT)>> {
-  static constexpr bool v = Op::STAGE_OUT;
-};
-
-// Minimum resident blocks per SM a row-pass op asks the compiler to allow for
-// (caps its registers); 1 unless the op says otherwise.
-template <class Op, class = void> struct MinBlocks {
-  static constexpr int v = 1;
-};
-template <class Op> struct MinBlocks<Op, std::void_t<decltype(Op::MINB)>> {
-  static constexpr int v = Op::MINB;
-};
+// Dipolar kernel (3 k_z^2/|k|^2 - 1)/N from the table's k_z^2/(2N) and |k|^2/(2N); 0 at k = 0.
+template <class R> __device__ __forceinline__ R dip_mult(const KArgs<R>& a, R kz, R k2) {
+  return k2 > R(0) ? fma_(R(3) * a.invN * kz, rcp_(k2), -a.invN) : R(0);
+}
 
 // Row-pass ops whose LHY terms come from the interpolation table plus the
 // exactly evaluated nodes (they stage the exact nodes only).
@@ -164,19 +156,89 @@ template <class Op, class = void> struct MaxThreadsWant {
 template <class Op> struct MaxThreadsWant<Op, std::void_t<decltype(Op::MAXT)>> {
   static constexpr int v = Op::MAXT;
 };
+// Field groups of a row pass: FP64 fields give every field of a row its own L/8
+// threads, FP32 fields one group that holds all fields of the row.  The FP64
+// passes wait on FP64 and integer chains, which more warps overlap; the FP32
+// passes wait on memory, where one thread's loads for all fields of eight points
+// are what is in flight (with groups the FP32 x-inverse passes took 62-66 us for
+// 48-54 at 128^3).
+template <class Op> struct RowGroups {
+  static constexpr int v = sizeof(typename Op::R) == 8 ? Op::NF : 1;
+};
 template <class Op> struct MaxThreads {
-  static constexpr int G = whole_warp_rows(Op::L) * (Op::L / 8);
+  static constexpr int G = whole_warp_rows(Op::L) * (Op::L / 8) * RowGroups<Op>::v;
   static constexpr int W = MaxThreadsWant<Op>::v;
   static constexpr int v = W >= G ? W - W % G : G;
+};
+
+// Minimum resident blocks per SM a row-pass op asks the compiler to allow for
+// (caps its registers); 1 unless the op says otherwise.
+template <class Op, class = void> struct MinBlocks {
+  static constexpr int v = 1;
+};
+template <class Op> struct MinBlocks<Op, std::void_t<decltype(Op::MINB)>> {
+  static constexpr int v = Op::MINB;
 };
 
 // ----------------------------------------------------------------------------
 // Row (x) pass kernel
 // ----------------------------------------------------------------------------
+// One point of a row pass's epilogue: its index in a field, its x, the trap terms
+// of its row, and its transform outputs: out(f), from registers or from where the
+// rows are parked in shared memory.
+template <class R, int NF, bool STAGED> struct RowPt {
+  C2<R> reg[STAGED ? 1 : NF];
+  const C2<R>* sm;
+  size_t idx;
+  int fs, x;
+  R vyz;
+  __device__ __forceinline__ C2<R> out(int f) const {
+    if constexpr (STAGED) return sm[f * fs];
+    else return reg[f];
+  }
+};
+// Row-pass ops that park their outputs with FP32 fields too, which frees the
+// transform's registers for the epilogue.
+template <class Op, class = void> struct StageOut {
+  static constexpr bool v = RowGroups<Op>::v > 1 || sizeof(typename Op::R) == 8;
+};
+template <class Op> struct StageOut<Op, std::void_t<decltype(Op::STAGE_OUT)>> {
+  static constexpr bool v = true;
+};
+
+// A thread's NV lines (fields f, f + 1, ...) to or from consecutive fields.
+template <class Op, int NV>
+__device__ __forceinline__ void store_rows(const KArgs<typename Op::R>& a, C2<typename Op::R>* dst, int f, int row, bool valid,
+                                           int t, const C2<typename Op::R> (&v)[NV][8]) {
+  if (!valid) return;
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      dst[(size_t)(f + k) * a.N + (size_t)row * a.nx + Plan<Op::L>::exit_pos(Op::INV, t, e)] = v[k][e];
+}
+template <class Op, int NV>
+__device__ __forceinline__ void load_rows(const KArgs<typename Op::R>& a, const C2<typename Op::R>* src, int f, int row,
+                                          bool valid, int t, C2<typename Op::R> (&v)[NV][8]) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      v[k][e] = valid ? src[(size_t)(f + k) * a.N + (size_t)row * a.nx + Plan<Op::L>::entry_pos(Op::INV, t, e)]
+                      : cmk<C2<typename Op::R>>(0, 0);
+}
+
+// A block takes MX rows of the op's NF fields.  With field groups (FP64), field f of
+// row m belongs to the L/8 threads of group (f, m): a thread holds eight values of
+// one line whatever the op (it used to transform all fields of its row: up to 255
+// registers, 8 warps per SM), and the points of the parked rows are then taken in
+// order by all threads of the block.  Forward ops, whose fields cost differently,
+// rotate the fields among the groups.  Without groups (FP32) a thread keeps to the
+// points of its own row.
 template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typename Op::R>& a) {
   using R = typename Op::R;
   using C = C2<R>;
-  constexpr int L = Op::L, NF = Op::NF, NS = Op::NS;
+  constexpr int L = Op::L, NF = Op::NF, NS = Op::NS, G = RowGroups<Op>::v, NV = NF / G;
   constexpr int NSR = NS > 0 ? NS : 1;
   constexpr int TPL = L / 8;
   constexpr int LP = row_len_padded<R, L>();
@@ -185,9 +247,14 @@ template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typen
   C* tw = reinterpret_cast<C*>(smraw);
   LhyNode<R>* nodes = reinterpret_cast<LhyNode<R>*>(tw + L);
   C* buf = reinterpret_cast<C*>(reinterpret_cast<unsigned char*>(nodes) + (Op::USES_LHY ? lhy_stage_bytes<R>(a.Q) : 0));
-  RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(buf + NF * a.MX * LP);
+  double* vrow = reinterpret_cast<double*>(buf + NF * a.MX * LP);  // trap terms of the rows (block-wide epilogues)
+  RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(vrow + a.MX);
   const int tid = threadIdx.x;
-  const int mrow = tid / TPL, t = tid - mrow * TPL;
+  const int g = G > 1 ? tid / (a.MX * TPL) : 0;
+  const int rt = tid - g * a.MX * TPL;
+  const int mrow = rt / TPL, t = rt - mrow * TPL;
+  const int fs = a.MX * LP;  // a field's rows in buf
+  C* line = buf + g * fs + mrow * LP;
   for (int i = tid; i < L; i += blockDim.x) tw[i] = a.twx[i];
   if constexpr (Op::USES_LHY) {
     if constexpr (LhyTabOp<Op>::v) stage_lhy_nodes(nodes, a.xnodes, a.Qx);
@@ -199,28 +266,72 @@ template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typen
   PAcc<R> acc[NSR];
   const int rows = a.ny * a.nz;
   const int ngroups = (rows + a.MX - 1) / a.MX;
+  const RowIdx<PadShift<R>::v> si{};
+  int f = g;
   for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
     const int row = grp * a.MX + mrow;
     const bool valid = row < rows;
-    C v[NF][8];
-    Op::load(a, u, row, valid, t, v, acc);
-    fft_line<C, L, Op::INV, NF>(v, buf + mrow * LP, a.MX * LP, tw, t, RowIdx<PadShift<R>::v>{});
-    if constexpr (StageOut<Op>::v) {
-      // park the transform outputs in the (idle) exchange buffer: the FFT
-      // registers are dead during the epilogue, which frees them for it
-      C* sm = buf + mrow * LP;
-      const RowIdx<PadShift<R>::v> si{};
-#pragma unroll
-      for (int f = 0; f < NF; ++f)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) sm[f * a.MX * LP + si(Plan<L>::exit_pos(Op::INV, t, e))] = v[f][e];
-      Op::store_staged(a, u, row, valid, t, sm, a.MX * LP, acc, nodes);
-      // the next row group's exchanges reuse the buffer (a warp's own rows when
-      // the length is a power of two, else rows that may straddle warps)
-      if constexpr (IsPow2<L>::v) __syncwarp();
-      else __syncthreads();
+    C v[NV][8];
+    Op::load(a, u, f, row, valid, t, v);
+    fft_line<C, L, Op::INV, NV>(v, line, fs, tw, t, si);
+    if constexpr (!Op::POINTS) {
+      Op::store(a, u, f, row, valid, t, v, acc);
+      if constexpr (G > 1 && !Op::INV) f = f + 1 < G ? f + 1 : 0;
     } else {
-      Op::store(a, u, row, valid, t, v, acc, nodes);
+      constexpr bool ST = StageOut<Op>::v;
+      if constexpr (ST) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+#pragma unroll
+          for (int e = 0; e < 8; ++e) line[k * fs + si(Plan<L>::exit_pos(Op::INV, t, e))] = v[k][e];
+      }
+      R s[NSR];
+#pragma unroll
+      for (int k = 0; k < NSR; ++k) s[k] = 0;
+      if constexpr (sizeof(R) == 8) {  // all points of the block's rows, one at a time
+        if (tid < a.MX) vrow[tid] = grp * a.MX + tid < rows ? trap_yz(a, grp * a.MX + tid) : 0.0;
+        __syncthreads();
+        const int P = min(a.MX, rows - grp * a.MX) * L;
+        for (int i = tid; i < P; i += blockDim.x) {
+          RowPt<R, NF, ST> pt[1];
+          const int m = i / L;
+          pt[0].x = i - m * L;
+          pt[0].idx = (size_t)(grp * a.MX) * L + i;
+          pt[0].vyz = vrow[m];
+          pt[0].sm = buf + m * LP + si(pt[0].x);
+          pt[0].fs = fs;
+          Op::points(a, u, pt, s, nodes);
+        }
+        __syncthreads();  // the next row group reuses the buffers
+      } else if (valid) {
+        constexpr int NP = Op::PTS;
+        const R vyz = trap_yz(a, row);
+#pragma unroll
+        for (int e0 = 0; e0 < 8; e0 += NP) {
+          RowPt<R, NF, ST> pt[NP];
+#pragma unroll
+          for (int j = 0; j < NP; ++j) {
+            pt[j].x = Plan<L>::exit_pos(Op::INV, t, e0 + j);
+            pt[j].idx = (size_t)row * L + pt[j].x;
+            pt[j].vyz = vyz;
+            pt[j].sm = line + si(pt[j].x);
+            pt[j].fs = fs;
+            if constexpr (!ST) {
+#pragma unroll
+              for (int k = 0; k < NF; ++k) pt[j].reg[k] = v[k][e0 + j];
+            }
+          }
+          Op::points(a, u, pt, s, nodes);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NSR; ++k) acc[k].add(s[k]);
+      // a thread reads back what it parked; the next exchange overwrites its warp's
+      // rows (rows that straddle warps for the mixed-radix lengths)
+      if constexpr (ST && sizeof(R) == 4) {
+        if constexpr (IsPow2<L>::v) __syncwarp();
+        else __syncthreads();
+      }
     }
   }
   if constexpr (NS > 0) {
@@ -228,6 +339,22 @@ template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typen
       if (threadIdx.x == 0) Op::finish(a, u);
     }
   }
+}
+
+// Shared memory per row of a block, and the rows per block unless tuned: as many
+// as the op's threads and 46 KB allow; FP64 passes (bound by arithmetic) halve them
+// while there are fewer row groups than SMs: at 32^3 the line pass ran on 16 SMs,
+// 80 us against 51.
+template <class Op> __host__ __device__ constexpr size_t row_pass_bytes() {
+  return (size_t)Op::NF * row_len_padded<typename Op::R, Op::L>() * sizeof(C2<typename Op::R>) + sizeof(double);
+}
+template <class Op> inline int default_rows(int rows, int nsm) {
+  constexpr int TPL = RowGroups<Op>::v * Op::L / 8;
+  int mx = whole_warp_rows(Op::L);
+  while (mx * 2 * TPL <= MaxThreads<Op>::v && mx * 2 * row_pass_bytes<Op>() <= 46 * 1024 &&
+         (sizeof(typename Op::R) == 4 || rows >= mx * 2 * nsm))
+    mx *= 2;
+  return mx;
 }
 
 // Row-pass entry points.  A min-blocks bound is given only when the op asks for
@@ -282,9 +409,12 @@ template <class Op> struct ColDefaultM {
 // Launch bounds of a column kernel: the run-time width keeps ColMaxThreads; a
 // compile-time width MC has exactly MC L/8 threads, and the FP32 plain y/z
 // passes (the ColPlain op, small epilogue) of up to 256 threads ask for three
-// resident blocks, as their run-time-width build reached without a bound.
+// resident blocks, as their run-time-width build reached without a bound.  The
+// FP32 mixed-radix passes ask for about 576 threads per SM: at 96^3 the energy
+// pass takes 24 us with three blocks of 192 and 33 us with two.
 template <class Op> struct ColMinB {
-  static constexpr int v = 1;
+  static constexpr int threads = ColDefaultM<Op>::v * (Op::L / 8);
+  static constexpr int v = sizeof(typename Op::R) == 4 && !IsPow2<Op::L>::v ? 576 / threads : 1;
 };
 template <class Op, int MC> struct ColBounds {
   static constexpr int threads = MC > 0 ? MC * (Op::L / 8) : ColMaxThreads<Op>::v;
@@ -312,7 +442,7 @@ template <class Op, int MC> __device__ __forceinline__ void colpass_body(const K
   for (int i = tid; i < L; i += blockDim.x) tw[i] = twsrc[i];
   __syncthreads();
   typename Op::Uni u;
-  Op::uniform(a, u);
+  Op::uniform(a, u, t);
   PAcc<R> acc[NSR];
   const int xb_n = a.nx / M;
   const int other_n = (Op::AXIS == 1) ? a.nz : a.ny;
@@ -386,7 +516,7 @@ __device__ __forceinline__ void colpass_tma_body(const CUtensorMap* tm, const KA
   }
   __syncthreads();
   typename Op::Uni u;
-  Op::uniform(a, u);
+  Op::uniform(a, u, t);
   PAcc<R> acc[NSR];
   const int xb_n = a.nx / M;
   const int other_n = (Op::AXIS == 1) ? a.nz : a.ny;
@@ -483,19 +613,16 @@ template <class R_, int L_, bool INV_> struct XPlain {
   static constexpr const char* NAME = "x-plain";
   static double alg_bytes(const KArgs<R>& a) { return 2.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 1, NS = 0;
-  static constexpr bool INV = INV_, USES_LHY = false;
+  static constexpr bool INV = INV_, USES_LHY = false, POINTS = false;
   using Uni = NoUni;
   static __device__ void uniform(const KArgs<R>&, Uni&) {}
-  static __device__ void load(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[1][8], PAcc<R>*) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      v[0][e] = valid ? a.gin[(size_t)row * a.nx + Plan<L>::entry_pos(INV, t, e)] : cmk<C>(0, 0);
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    load_rows<XPlain>(a, a.gin, f, row, valid, t, v);
   }
-  static __device__ void store(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[1][8], PAcc<R>*,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) a.gout[(size_t)row * a.nx + Plan<L>::exit_pos(INV, t, e)] = v[0][e];
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XPlain>(a, a.gout, f, row, valid, t, v);
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -509,7 +636,7 @@ template <class R_, int L_, int AXIS_, bool INV_> struct ColPlain {
   static constexpr int L = L_, NS = 0, AXIS = AXIS_;
   static constexpr bool INV = INV_;
   using Uni = NoUni;
-  static __device__ void uniform(const KArgs<R>&, Uni&) {}
+  static __device__ void uniform(const KArgs<R>&, Uni&, int) {}
   static constexpr bool FIRST_INV = INV_;
   static __device__ const C* src(const KArgs<R>& a) { return a.gin; }
   template <class SI>
@@ -558,7 +685,7 @@ template <class R_, int L_> struct XFwdEG {
   static constexpr const char* NAME = "x-fwd energy";
   static double alg_bytes(const KArgs<R>& a) { return (a.flag ? 9.0 : 5.0) * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 3, NS = 0;
-  static constexpr bool INV = false, USES_LHY = false;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   using Uni = EgUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) {
     u.cur = __ldcg(&a.st->cur);
@@ -571,53 +698,84 @@ template <class R_, int L_> struct XFwdEG {
     u.cb[0] = c[2];
     u.cb[1] = c[3];
   }
-  static __device__ void load(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[3][8], PAcc<R>*) {
-    const C* src = a.psi[u.cur];
-    const C* pd = a.pb[u.nsel];
-    C* dst = a.psi[u.slot];
-    const size_t N = a.N;
-    constexpr int CH = ChunkW<R>::v;
+  // fields 0, 1: psi or the trial point on the geodesic (Sec. III), renormalised
+  // (Sec. V) and stored; field 2: the dipolar source from both components (a group
+  // of its own reads what the other two read at the same time, from L1/L2)
+  static __device__ C source(const KArgs<R>& a, C p1, C p2) {
+    const R n1 = cabs2(p1), n2 = cabs2(p2);
+    return cmk<C>(fma_(a.d12, n2, a.d11 * n1), fma_(a.d22, n2, a.d21 * n1));
+  }
+  static __device__ C point(const KArgs<R>& a, const Uni& u, int i, size_t idx) {
+    const C p = pick(a.psi, u.cur)[(size_t)i * a.N + idx];
+    if (!a.flag) return p;
+    const C q = pick(a.pb, u.nsel)[(size_t)i * a.N + idx];
+    return cmk<C>(fma_(pick(u.cb, i), q.x, pick(u.ca, i) * p.x), fma_(pick(u.cb, i), q.y, pick(u.ca, i) * p.y));
+  }
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    const size_t base = (size_t)row * a.nx, N = a.N;
+    if (!valid) {
 #pragma unroll
-    for (int e0 = 0; e0 < 8; e0 += CH) {
-      C p1[CH], p2[CH], q1[CH], q2[CH];
+      for (int e = 0; e < 8; ++e)
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
-        p1[j] = valid ? src[idx] : cmk<C>(0, 0);
-        p2[j] = valid ? src[N + idx] : cmk<C>(0, 0);
+        for (int k = 0; k < NV; ++k) v[k][e] = cmk<C>(0, 0);
+      return;
+    }
+    if constexpr (NV == 1) {
+      if (f < 2) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[0][e] = point(a, u, f, base + Plan<L>::entry_pos(false, t, e));
         if (a.flag) {
-          q1[j] = valid ? pd[idx] : cmk<C>(0, 0);
-          q2[j] = valid ? pd[N + idx] : cmk<C>(0, 0);
+          C* dst = pick(a.psi, u.slot) + (size_t)f * N + base;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) dst[Plan<L>::entry_pos(false, t, e)] = v[0][e];
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const size_t idx = base + Plan<L>::entry_pos(false, t, e);
+          v[0][e] = source(a, point(a, u, 0, idx), point(a, u, 1, idx));
         }
       }
+    } else {
+      // both components at once, the loads of a chunk before its arithmetic
+      constexpr int CH = ChunkW<R>::v;
+      const C* src = pick(a.psi, u.cur);
+      const C* pd = pick(a.pb, u.nsel);
+      C* dst = pick(a.psi, u.slot);
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const int e = e0 + j;
-        if (a.flag) {  // trial point on the geodesic (Sec. III), renormalised (Sec. V)
-          p1[j] = cmk<C>(u.ca[0] * p1[j].x + u.cb[0] * q1[j].x, u.ca[0] * p1[j].y + u.cb[0] * q1[j].y);
-          p2[j] = cmk<C>(u.ca[1] * p2[j].x + u.cb[1] * q2[j].x, u.ca[1] * p2[j].y + u.cb[1] * q2[j].y);
-          if (valid) {
-            const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e);
-            dst[idx] = p1[j];
-            dst[N + idx] = p2[j];
+      for (int e0 = 0; e0 < 8; e0 += CH) {
+        C q1[CH], q2[CH];
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          const size_t idx = base + Plan<L>::entry_pos(false, t, e0 + j);
+          v[0][e0 + j] = src[idx];
+          v[1][e0 + j] = src[N + idx];
+          if (a.flag) {
+            q1[j] = pd[idx];
+            q2[j] = pd[N + idx];
           }
         }
-        const R n1 = cabs2(p1[j]), n2 = cabs2(p2[j]);
-        v[0][e] = p1[j];
-        v[1][e] = p2[j];
-        v[2][e] = cmk<C>(a.d11 * n1 + a.d12 * n2, a.d21 * n1 + a.d22 * n2);
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          C p1 = v[0][e0 + j], p2 = v[1][e0 + j];
+          if (a.flag) {
+            p1 = cmk<C>(fma_(u.cb[0], q1[j].x, u.ca[0] * p1.x), fma_(u.cb[0], q1[j].y, u.ca[0] * p1.y));
+            p2 = cmk<C>(fma_(u.cb[1], q2[j].x, u.ca[1] * p2.x), fma_(u.cb[1], q2[j].y, u.ca[1] * p2.y));
+            const size_t idx = base + Plan<L>::entry_pos(false, t, e0 + j);
+            dst[idx] = p1;
+            dst[N + idx] = p2;
+            v[0][e0 + j] = p1;
+            v[1][e0 + j] = p2;
+          }
+          v[2][e0 + j] = source(a, p1, p2);
+        }
       }
     }
   }
-  static __device__ void store(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[3][8], PAcc<R>*,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::exit_pos(false, t, e);
-#pragma unroll
-      for (int f = 0; f < 3; ++f) a.W[(size_t)f * a.N + idx] = v[f][e];
-    }
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XFwdEG>(a, a.W, f, row, valid, t, v);
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -629,37 +787,32 @@ template <class R_, int L_> struct ZEg {
   static constexpr const char* NAME = "z fused energy";
   static double alg_bytes(const KArgs<R>& a) { return 6.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NS = 2, AXIS = 2;
-  struct Uni {
+  struct Uni : KzLine<R, L_> {
     int slot;
   };
-  static __device__ void uniform(const KArgs<R>& a, Uni& u) {
+  static __device__ void uniform(const KArgs<R>& a, Uni& u, int t) {
     const int cur = __ldcg(&a.st->cur);
     u.slot = a.flag ? (cur ^ 1) : cur;
+    u.set(a, t);
   }
   static constexpr bool FIRST_INV = false;
   static __device__ const C* src(const KArgs<R>& a) { return a.W; }
   template <class SI>
-  static __device__ void process(const KArgs<R>& a, Uni&, int f, int x, int y, size_t base, size_t ls, int t,
+  static __device__ void process(const KArgs<R>& a, Uni& u, int f, int x, int y, size_t base, size_t ls, int t,
                                  C (&v)[1][8], C* sm, const C* tw, SI si, PAcc<R>* acc) {
     fft_line<C, L, false, 1>(v, sm, 0, tw, t, si);
-    const R kx = wavenum<R>(x, a.nx, a.dkx), ky = wavenum<R>(y, a.ny, a.dky);
-    const R kxy2 = kx * kx + ky * ky;
+    const R kxy = kq_xy(a, x, y);
     R ekin = 0;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const R kz = wavenum<R>(Plan<L>::exit_pos(false, t, e), a.nz, a.dkz);
-      const R k2 = kxy2 + kz * kz;
-      R mult;
-      if (f < 2) {
-        const R t2 = R(0.5) * k2;
-        ekin += t2 * cabs2(v[0][e]);
-        mult = t2 * a.invN;
-      } else {
-        mult = (k2 > R(0)) ? (R(3) * kz * kz / k2 - R(1)) * a.invN : R(0);
-      }
+      const R kz = u.kz[e];
+      R mult = kxy + kz;  // |k|^2/(2N)
+      if (f < 2) ekin = fma_(mult, cabs2(v[0][e]), ekin);
+      else mult = dip_mult(a, kz, mult);
       v[0][e] = cscale(v[0][e], mult);
     }
-    if (f < 2) acc[f].add(ekin);
+    if (f == 0) acc[0].add(ekin);
+    else if (f == 1) acc[1].add(ekin);
     col_after<L>(sm, si);
     fft_line<C, L, true, 1>(v, sm, 0, tw, t, si);
 #pragma unroll
@@ -669,26 +822,29 @@ template <class R_, int L_> struct ZEg {
   static __device__ void finish(const KArgs<R>&, Uni&) {}
 };
 
-// mu_LHY,i and the LHY energy density at NP points: the interpolation table
-// plus the exactly evaluated nodes; F from Euler's identity for the degree-5/2
-// density, F = (2/5)(n1 mu1 + n2 mu2).
+// mu_LHY,i at NP points: the interpolation table plus the exactly evaluated
+// nodes.  (The LHY density is F = (2/5)(n1 mu1 + n2 mu2), Euler's identity for
+// degree 5/2; finalize_energy takes it from the sums of n_i mu_i.)
 template <class R, int NP>
 __device__ __forceinline__ void lhy_terms(const KArgs<R>& a, const LhyNode<R>* nodes, const LhyCoef<R>& cf,
-                                          const R (&n1)[NP], const R (&n2)[NP], R (&F)[NP], R (&m1)[NP],
-                                          R (&m2)[NP]) {
+                                          const R (&n1)[NP], const R (&n2)[NP], R (&m1)[NP], R (&m2)[NP]) {
 #pragma unroll
   for (int j = 0; j < NP; ++j) m1[j] = m2[j] = R(0);
   if (a.Qx > 0) {
-    // exact nodes two points at a time (few registers for a rarely long loop)
+    if constexpr (NP == 1) {
+      lhy_points<R, 1>(nodes, a.Qx, a.Qxm, cf, n1, n2, m1, m2);
+    } else {
+      // exact nodes two points at a time (few registers for a rarely long loop)
 #pragma unroll
-    for (int j = 0; j < NP; j += 2) {
-      const R q1[2] = {n1[j], n1[j + 1]}, q2[2] = {n2[j], n2[j + 1]};
-      R f[2], x1[2], x2[2];
-      lhy_points<R, 2>(nodes, a.Qx, a.Qxm, cf, q1, q2, f, x1, x2);
-      m1[j] = x1[0];
-      m1[j + 1] = x1[1];
-      m2[j] = x2[0];
-      m2[j + 1] = x2[1];
+      for (int j = 0; j < NP; j += 2) {
+        const R q1[2] = {n1[j], n1[j + 1]}, q2[2] = {n2[j], n2[j + 1]};
+        R x1[2], x2[2];
+        lhy_points<R, 2>(nodes, a.Qx, a.Qxm, cf, q1, q2, x1, x2);
+        m1[j] = x1[0];
+        m1[j + 1] = x1[1];
+        m2[j] = x2[0];
+        m2[j + 1] = x2[1];
+      }
     }
   }
   if (a.tab.ni > 0) {
@@ -700,8 +856,6 @@ __device__ __forceinline__ void lhy_terms(const KArgs<R>& a, const LhyNode<R>* n
       m2[j] += t2[j];
     }
   }
-#pragma unroll
-  for (int j = 0; j < NP; ++j) F[j] = R(0.4) * (n1[j] * m1[j] + n2[j] * m2[j]);
 }
 
 // n'^T (d^2 F/dn dn) n' at NP points: table plus exactly evaluated nodes.
@@ -712,14 +866,18 @@ __device__ __forceinline__ void lhy_second(const KArgs<R>& a, const LhyNode<R>* 
 #pragma unroll
   for (int j = 0; j < NP; ++j) H[j] = R(0);
   if (a.Qx > 0) {
+    if constexpr (NP == 1) {
+      lhy_hess<R, 1>(nodes, a.Qx, a.Qxm, cf, n1, n2, n1p, n2p, H);
+    } else {
 #pragma unroll
-    for (int j = 0; j < NP; j += 2) {
-      const R q1[2] = {n1[j], n1[j + 1]}, q2[2] = {n2[j], n2[j + 1]};
-      const R p1[2] = {n1p[j], n1p[j + 1]}, p2[2] = {n2p[j], n2p[j + 1]};
-      R hx[2];
-      lhy_hess<R, 2>(nodes, a.Qx, a.Qxm, cf, q1, q2, p1, p2, hx);
-      H[j] = hx[0];
-      H[j + 1] = hx[1];
+      for (int j = 0; j < NP; j += 2) {
+        const R q1[2] = {n1[j], n1[j + 1]}, q2[2] = {n2[j], n2[j + 1]};
+        const R p1[2] = {n1p[j], n1p[j + 1]}, p2[2] = {n2p[j], n2p[j + 1]};
+        R hx[2];
+        lhy_hess<R, 2>(nodes, a.Qx, a.Qxm, cf, q1, q2, p1, p2, hx);
+        H[j] = hx[0];
+        H[j + 1] = hx[1];
+      }
     }
   }
   if (a.tab.ni > 0) {
@@ -733,86 +891,62 @@ __device__ __forceinline__ void lhy_second(const KArgs<R>& a, const LhyNode<R>* 
 template <class R_, int L_> struct XInvEG {
   using R = R_;
   using C = C2<R>;
-  static constexpr int MAXT = 128;
-  static constexpr int MINB = sizeof(R_) == 4 ? EGPE_EG_MINB : 1;
+  // FP32: 128 threads, 4 blocks per SM (128 registers; the mixed-radix lengths 3, which
+  // spill at 4); FP64: three groups of 32 threads
+  static constexpr int PTS = 4, MAXT = sizeof(R_) == 4 ? 128 : 96, MINB = sizeof(R_) == 4 ? (IsPow2<L_>::v ? 4 : 3) : 1;
+  static constexpr bool STAGE_OUT = true;
   static constexpr const char* NAME = "x-inv energy+LHY";
   static double alg_bytes(const KArgs<R>& a) { return 9.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 3, NS = EG_NS;
-  static constexpr bool INV = true, USES_LHY = true, LHY_TAB = true;
+  static constexpr bool INV = true, USES_LHY = true, LHY_TAB = true, POINTS = true;
   using Uni = EgUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { XFwdEG<R, L>::uniform(a, u); }
-  static __device__ void load(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[3][8], PAcc<R>*) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(true, t, e);
-#pragma unroll
-      for (int f = 0; f < 3; ++f) v[f][e] = valid ? a.W[(size_t)f * a.N + idx] : cmk<C>(0, 0);
-    }
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    load_rows<XInvEG>(a, a.W, f, row, valid, t, v);
   }
-  static constexpr int NP = LhyNP<R>::v;
-  static constexpr bool STAGE_OUT = true;
-  static __device__ void store_staged(const KArgs<R>& a, Uni& u, int row, bool valid, int t, const C* sm, int fs,
-                                      PAcc<R>* acc, const LhyNode<R>* nodes) {
-    const RowIdx<PadShift<R>::v> si{};
-    if (!valid) return;
-    const C* ps = a.psi[u.slot];
-    C* hp = a.hp[u.slot];
-    C* ax = a.ax[u.slot];
+  template <int NP, bool ST>
+  static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[EG_NS],
+                                const LhyNode<R>* nodes) {
+    const C* ps = pick(a.psi, u.slot);
+    C* hp = pick(a.hp, u.slot);
+    C* ax = pick(a.ax, u.slot);
     const size_t N = a.N;
-    const int y = row % a.ny, z = row / a.ny;
-    const R Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
-    const R vyz = a.vy * Y * Y + a.vz * Z * Z;
-    const LhyCoef<R> cf = lhy_coef(a);
-    R s[EG_NS];
+    C p1[NP], p2[NP];
+    R n1[NP], n2[NP], m1[NP], m2[NP];
 #pragma unroll
-    for (int k = 0; k < EG_NS; ++k) s[k] = 0;
-#pragma unroll
-    for (int e0 = 0; e0 < 8; e0 += NP) {
-      C p1[NP], p2[NP];
-      R n1[NP], n2[NP], F[NP], m1[NP], m2[NP];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        const size_t idx = (size_t)row * a.nx + Plan<L>::exit_pos(true, t, e0 + j);
-        p1[j] = ps[idx];
-        p2[j] = ps[N + idx];
-        n1[j] = cabs2(p1[j]);
-        n2[j] = cabs2(p2[j]);
-      }
-      lhy_terms<R, NP>(a, nodes, cf, n1, n2, F, m1, m2);
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        const int e = e0 + j;
-        const int x = Plan<L>::exit_pos(true, t, e);
-        const size_t idx = (size_t)row * a.nx + x;
-        const R X = -a.Lx + (R)x * a.hx;
-        const R V = a.vx * X * X + vyz;
-        const int o = si(x);
-        const C T1 = sm[o], T2 = sm[fs + o], PH = sm[2 * fs + o];
-        const R phi1 = PH.x, phi2 = PH.y;
-        const R U1 = V + a.g11 * n1[j] + a.g12 * n2[j] + phi1 + m1[j];
-        const R U2 = V + a.g21 * n1[j] + a.g22 * n2[j] + phi2 + m2[j];
-        const C H1 = cmk<C>(T1.x + U1 * p1[j].x, T1.y + U1 * p1[j].y);
-        const C H2 = cmk<C>(T2.x + U2 * p2[j].x, T2.y + U2 * p2[j].y);
-        hp[idx] = H1;
-        hp[N + idx] = H2;
-        ax[idx] = cmk<C>(phi1, phi2);
-        ax[N + idx] = cmk<C>(m1[j], m2[j]);
-        s[EG_TRAP] += V * (n1[j] + n2[j]);
-        s[EG_CONTACT] += R(0.5) * (a.g11 * n1[j] * n1[j] + (a.g12 + a.g21) * n1[j] * n2[j] + a.g22 * n2[j] * n2[j]);
-        s[EG_DIPOLAR] += R(0.5) * (n1[j] * phi1 + n2[j] * phi2);
-        s[EG_LHY] += F[j];
-        s[EG_MU1] += cdot(p1[j], H1);
-        s[EG_MU2] += cdot(p2[j], H2);
-        s[EG_NPHI1] += n1[j] * phi1;
-        s[EG_NPHI2] += n2[j] * phi2;
-        s[EG_NMUL1] += n1[j] * m1[j];
-        s[EG_NMUL2] += n2[j] * m2[j];
-        s[EG_NORM1] += n1[j];
-        s[EG_NORM2] += n2[j];
-      }
+    for (int j = 0; j < NP; ++j) {
+      p1[j] = ps[pt[j].idx];
+      p2[j] = ps[N + pt[j].idx];
+      n1[j] = cabs2(p1[j]);
+      n2[j] = cabs2(p2[j]);
     }
+    lhy_terms<R, NP>(a, nodes, lhy_coef(a), n1, n2, m1, m2);
 #pragma unroll
-    for (int k = 0; k < EG_NS; ++k) acc[k].add(s[k]);
+    for (int j = 0; j < NP; ++j) {
+      const size_t idx = pt[j].idx;
+      const R V = trap_x(a, pt[j].x) + pt[j].vyz;
+      const C T1 = pt[j].out(0), T2 = pt[j].out(1), PH = pt[j].out(2);
+      const R phi1 = PH.x, phi2 = PH.y;
+      const R c1 = fma_(a.g12, n2[j], a.g11 * n1[j]), c2 = fma_(a.g22, n2[j], a.g21 * n1[j]);
+      const R U1 = (V + c1) + (phi1 + m1[j]);
+      const R U2 = (V + c2) + (phi2 + m2[j]);
+      hp[idx] = cmk<C>(fma_(U1, p1[j].x, T1.x), fma_(U1, p1[j].y, T1.y));
+      hp[N + idx] = cmk<C>(fma_(U2, p2[j].x, T2.x), fma_(U2, p2[j].y, T2.y));
+      ax[idx] = PH;
+      ax[N + idx] = cmk<C>(m1[j], m2[j]);
+      // the energies and mu_i are combinations of these (finalize_energy)
+      s[EG_TRAP1] = fma_(V, n1[j], s[EG_TRAP1]);
+      s[EG_TRAP2] = fma_(V, n2[j], s[EG_TRAP2]);
+      s[EG_CON1] = fma_(c1, n1[j], s[EG_CON1]);
+      s[EG_CON2] = fma_(c2, n2[j], s[EG_CON2]);
+      s[EG_NPHI1] = fma_(n1[j], phi1, s[EG_NPHI1]);
+      s[EG_NPHI2] = fma_(n2[j], phi2, s[EG_NPHI2]);
+      s[EG_NMUL1] = fma_(n1[j], m1[j], s[EG_NMUL1]);
+      s[EG_NMUL2] = fma_(n2[j], m2[j], s[EG_NMUL2]);
+      s[EG_NORM1] += n1[j];
+      s[EG_NORM2] += n2[j];
+    }
   }
   static __device__ double* out(const KArgs<R>& a, Uni& u) { return a.st->eg[u.slot]; }
   static __device__ void finish(const KArgs<R>& a, Uni&) { eg_ctrl(a); }
@@ -852,52 +986,56 @@ template <class R> __device__ __forceinline__ void pc_uniform(const KArgs<R>& a,
   }
 }
 
-// Inputs of the preconditioner prologue at one point.
-template <class R> struct PcIn {
-  C2<R> p1, p2, h1, h2, ml;
-};
+// P_V,i of component i at a point (Sec. IV.B), with the floor.
 template <class R>
-__device__ __forceinline__ void pc_load(const KArgs<R>& a, const PcUni<R>& u, size_t idx, PcIn<R>& in) {
-  const size_t N = a.N;
-  if (u.rgiven) {
-    in.h1 = a.rb[u.nsel][idx];
-    in.h2 = a.rb[u.nsel][N + idx];
-  } else {
-    in.h1 = a.hp[u.cur][idx];
-    in.h2 = a.hp[u.cur][N + idx];
-  }
-  if (a.diag || !u.rgiven) {
-    in.p1 = a.psi[u.cur][idx];
-    in.p2 = a.psi[u.cur][N + idx];
-  }
-  if (a.diag) in.ml = a.ax[u.cur][N + idx];
+__device__ __forceinline__ R pv_at(const KArgs<R>& a, const PcUni<R>& u, int i, R V, R n1, R n2, R ml) {
+  const R P = fma_(i ? a.g22 : a.g12, n2, fma_(i ? a.g21 : a.g11, n1, (pick(u.shift, i) + V) + ml));
+  const R fl = pick(u.floor_, i);
+  return P > fl ? P : fl;
 }
-// r_i = H_i psi_i - mu_i psi_i (stored unless given) and w_i = P_V^{-1} r_i when diag.
-template <class R>
-__device__ __forceinline__ void pc_apply(const KArgs<R>& a, const PcUni<R>& u, size_t idx, R V, const PcIn<R>& in,
-                                         C2<R>& w1, C2<R>& w2) {
+// r_i = H_i psi_i - mu_i psi_i (stored unless given) and w_i = P_V^{-1} r_i when
+// diag, at CH points: both components (NV = 2, i = 0) or component i alone.
+template <class R, int CH, int NV>
+__device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u, int i, const size_t (&idx)[CH],
+                                            const R (&V)[CH], C2<R> (&w)[NV][CH]) {
   using C = C2<R>;
-  C r1, r2;
-  if (u.rgiven) {
-    r1 = in.h1;
-    r2 = in.h2;
-  } else {
-    r1 = cmk<C>(in.h1.x - u.mu[0] * in.p1.x, in.h1.y - u.mu[0] * in.p1.y);
-    r2 = cmk<C>(in.h2.x - u.mu[1] * in.p2.x, in.h2.y - u.mu[1] * in.p2.y);
-    a.rb[u.nsel][idx] = r1;
-    a.rb[u.nsel][(size_t)a.N + idx] = r2;
+  const size_t N = a.N;
+  C h[NV][CH], p[2][CH], ml[CH];  // NV = 1: p[0] is component i, p[1] the other
+#pragma unroll
+  for (int j = 0; j < CH; ++j) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const size_t q = (size_t)(i + k) * N + idx[j];
+      h[k][j] = u.rgiven ? pick(a.rb, u.nsel)[q] : pick(a.hp, u.cur)[q];
+      if (a.diag || !u.rgiven) p[k][j] = pick(a.psi, u.cur)[q];
+    }
+    if (a.diag) {
+      if constexpr (NV == 1) p[1][j] = pick(a.psi, u.cur)[(i ? 0 : N) + idx[j]];
+      ml[j] = pick(a.ax, u.cur)[N + idx[j]];
+    }
   }
-  if (a.diag) {
-    const R n1 = cabs2(in.p1), n2 = cabs2(in.p2);
-    R P1 = u.shift[0] + V + a.g11 * n1 + a.g12 * n2 + in.ml.x;
-    R P2 = u.shift[1] + V + a.g21 * n1 + a.g22 * n2 + in.ml.y;
-    P1 = P1 > u.floor_[0] ? P1 : u.floor_[0];
-    P2 = P2 > u.floor_[1] ? P2 : u.floor_[1];
-    w1 = cscale(r1, R(1) / P1);
-    w2 = cscale(r2, R(1) / P2);
-  } else {
-    w1 = r1;
-    w2 = r2;
+#pragma unroll
+  for (int j = 0; j < CH; ++j) {
+    R nn[2];
+    if (a.diag) {
+      nn[0] = cabs2(p[0][j]);
+      nn[1] = cabs2(p[1][j]);
+    }
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int c = i + k;
+      C r = h[k][j];
+      if (!u.rgiven) {
+        const R mu = pick(u.mu, c);
+        r = cmk<C>(fma_(-mu, p[k][j].x, r.x), fma_(-mu, p[k][j].y, r.y));
+        pick(a.rb, u.nsel)[(size_t)c * N + idx[j]] = r;
+      }
+      if (a.diag) {
+        const R n1 = NV == 1 && i ? nn[1] : nn[0], n2 = NV == 1 && i ? nn[0] : nn[1];
+        r = cscale(r, rcp_(pv_at(a, u, c, V[j], n1, n2, c ? ml[j].y : ml[j].x)));
+      }
+      w[k][j] = r;
+    }
   }
 }
 
@@ -908,32 +1046,34 @@ template <class R> struct PcSumIn {
 template <class R>
 __device__ __forceinline__ void pc_sum_load(const KArgs<R>& a, const PcUni<R>& u, size_t idx, PcSumIn<R>& in) {
   const size_t N = a.N;
-  in.r1 = a.rb[u.nsel][idx];
-  in.r2 = a.rb[u.nsel][N + idx];
-  in.q1 = a.rb[u.nsel ^ 1][idx];
-  in.q2 = a.rb[u.nsel ^ 1][N + idx];
-  in.d1 = a.pb[u.nsel ^ 1][idx];
-  in.d2 = a.pb[u.nsel ^ 1][N + idx];
-  in.p1 = a.psi[u.cur][idx];
-  in.p2 = a.psi[u.cur][N + idx];
+  in.r1 = pick(a.rb, u.nsel)[idx];
+  in.r2 = pick(a.rb, u.nsel)[N + idx];
+  in.q1 = pick(a.rb, u.nsel ^ 1)[idx];
+  in.q2 = pick(a.rb, u.nsel ^ 1)[N + idx];
+  in.d1 = pick(a.pb, u.nsel ^ 1)[idx];
+  in.d2 = pick(a.pb, u.nsel ^ 1)[N + idx];
+  in.p1 = pick(a.psi, u.cur)[idx];
+  in.p2 = pick(a.psi, u.cur)[N + idx];
 }
 template <class R>
 __device__ __forceinline__ void pc_sum_add(const PcSumIn<R>& in, C2<R> z1, C2<R> z2, R* s) {
   const C2<R> dr1 = csub(in.r1, in.q1), dr2 = csub(in.r2, in.q2);
-  s[PC_SRZ] += cdot(dr1, z1) + cdot(dr2, z2);
-  s[PC_SRP] += cdot(dr1, in.d1) + cdot(dr2, in.d2);
-  s[PC_ZPSI1] += cdot(z1, in.p1);
-  s[PC_ZPSI2] += cdot(z2, in.p2);
-  s[PC_PPPSI1] += cdot(in.d1, in.p1);
-  s[PC_PPPSI2] += cdot(in.d2, in.p2);
-  s[PC_ZR1] += cdot(z1, in.r1);
-  s[PC_ZR2] += cdot(z2, in.r2);
-  s[PC_PPR1] += cdot(in.d1, in.r1);
-  s[PC_PPR2] += cdot(in.d2, in.r2);
-  s[PC_PSIR1] += cdot(in.p1, in.r1);
-  s[PC_PSIR2] += cdot(in.p2, in.r2);
-  s[PC_RR1] += cabs2(in.r1);
-  s[PC_RR2] += cabs2(in.r2);
+  cdot_add(s[PC_SRZ], dr1, z1);
+  cdot_add(s[PC_SRZ], dr2, z2);
+  cdot_add(s[PC_SRP], dr1, in.d1);
+  cdot_add(s[PC_SRP], dr2, in.d2);
+  cdot_add(s[PC_ZPSI1], z1, in.p1);
+  cdot_add(s[PC_ZPSI2], z2, in.p2);
+  cdot_add(s[PC_PPPSI1], in.d1, in.p1);
+  cdot_add(s[PC_PPPSI2], in.d2, in.p2);
+  cdot_add(s[PC_ZR1], z1, in.r1);
+  cdot_add(s[PC_ZR2], z2, in.r2);
+  cdot_add(s[PC_PPR1], in.d1, in.r1);
+  cdot_add(s[PC_PPR2], in.d2, in.r2);
+  cdot_add(s[PC_PSIR1], in.p1, in.r1);
+  cdot_add(s[PC_PSIR2], in.p2, in.r2);
+  cdot_add(s[PC_RR1], in.r1, in.r1);
+  cdot_add(s[PC_RR2], in.r2, in.r2);
 }
 
 template <class R_, int L_> struct XFwdPC {
@@ -942,44 +1082,41 @@ template <class R_, int L_> struct XFwdPC {
   static constexpr const char* NAME = "x-fwd precond";
   static double alg_bytes(const KArgs<R>& a) { return (a.diag ? 9.0 : 8.0) * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 2, NS = 0;
-  static constexpr bool INV = false, USES_LHY = false;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   using Uni = PcUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { pc_uniform(a, u); }
-  static __device__ void load(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[2][8], PAcc<R>*) {
-    const int y = row % a.ny, z = row / a.ny;
-    const R Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
-    const R vyz = a.vy * Y * Y + a.vz * Z * Z;
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    if (!valid) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k][e] = cmk<C>(0, 0);
+      return;
+    }
+    const R vyz = trap_yz(a, row);
     constexpr int CH = ChunkW<R>::v;
 #pragma unroll
     for (int e0 = 0; e0 < 8; e0 += CH) {
-      PcIn<R> in[CH];
-      if (valid) {
-#pragma unroll
-        for (int j = 0; j < CH; ++j)
-          pc_load<R>(a, u, (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j), in[j]);
-      }
+      size_t idx[CH];
+      R V[CH];
+      C w[NV][CH];
 #pragma unroll
       for (int j = 0; j < CH; ++j) {
-        const int e = e0 + j;
-        v[0][e] = cmk<C>(0, 0);
-        v[1][e] = cmk<C>(0, 0);
-        if (valid) {
-          const int x = Plan<L>::entry_pos(false, t, e);
-          const R X = -a.Lx + (R)x * a.hx;
-          pc_apply<R>(a, u, (size_t)row * a.nx + x, a.vx * X * X + vyz, in[j], v[0][e], v[1][e]);
-        }
+        const int x = Plan<L>::entry_pos(false, t, e0 + j);
+        idx[j] = (size_t)row * a.nx + x;
+        V[j] = trap_x(a, x) + vyz;
       }
+      pc_residual<R, CH, NV>(a, u, f, idx, V, w);
+#pragma unroll
+      for (int j = 0; j < CH; ++j)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k][e0 + j] = w[k][j];
     }
   }
-  static __device__ void store(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[2][8], PAcc<R>*,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::exit_pos(false, t, e);
-      a.W[idx] = v[0][e];
-      a.W[(size_t)a.N + idx] = v[1][e];
-    }
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XFwdPC>(a, a.W, f, row, valid, t, v);
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -991,11 +1128,12 @@ template <class R_, int L_> struct ZPc {
   static constexpr const char* NAME = "z fused precond";
   static double alg_bytes(const KArgs<R>& a) { return 4.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NS = 0, AXIS = 2;
-  struct Uni {
+  struct Uni : KzLine<R, L_> {
     R shift[2];
   };
-  static __device__ void uniform(const KArgs<R>& a, Uni& u) {
+  static __device__ void uniform(const KArgs<R>& a, Uni& u, int t) {
     load_uniforms<R, 2>({&a.st->shift[0], &a.st->shift[1]}, u.shift);
+    u.set(a, t);
   }
   static constexpr bool FIRST_INV = false;
   static __device__ const C* src(const KArgs<R>& a) { return a.W; }
@@ -1003,13 +1141,13 @@ template <class R_, int L_> struct ZPc {
   static __device__ void process(const KArgs<R>& a, Uni& u, int f, int x, int y, size_t base, size_t ls, int t,
                                  C (&v)[1][8], C* sm, const C* tw, SI si, PAcc<R>*) {
     fft_line<C, L, false, 1>(v, sm, 0, tw, t, si);
-    const R kx = wavenum<R>(x, a.nx, a.dkx), ky = wavenum<R>(y, a.ny, a.dky);
-    const R kxy2 = kx * kx + ky * ky;
-    const R sh = f == 0 ? u.shift[0] : u.shift[1];
+    const R kxy = kq_xy(a, x, y);
+    const R sh = a.invN * (f == 0 ? u.shift[0] : u.shift[1]);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const R kz = wavenum<R>(Plan<L>::exit_pos(false, t, e), a.nz, a.dkz);
-      v[0][e] = cscale(v[0][e], a.invN / (sh + R(0.5) * (kxy2 + kz * kz)));
+      // invN / (shift + |k|^2/2), numerator and denominator over N
+      const R kz = u.kz[e];
+      v[0][e] = cscale(v[0][e], a.invN * a.invN * rcp_(sh + (kxy + kz)));
     }
     col_after<L>(sm, si);
     fft_line<C, L, true, 1>(v, sm, 0, tw, t, si);
@@ -1023,63 +1161,40 @@ template <class R_, int L_> struct ZPc {
 template <class R_, int L_> struct XInvPC {
   using R = R_;
   using C = C2<R>;
-  static constexpr int MAXT = 128;  // heavy epilogue: smaller blocks, more of them per SM
-  static constexpr int MINB = sizeof(R_) == 4 ? EGPE_PC_MINB : 1;
+  static constexpr int PTS = 4, MAXT = sizeof(R_) == 4 ? 128 : 64;  // heavy epilogue: small blocks, more of them per SM
   static constexpr const char* NAME = "x-inv precond sums";
   static double alg_bytes(const KArgs<R>& a) { return 12.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 2, NS = PC_NS;
-  static constexpr bool INV = true, USES_LHY = false;
+  static constexpr bool INV = true, USES_LHY = false, POINTS = true;
   using Uni = PcUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { pc_uniform(a, u); }
-  static __device__ void load(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[2][8], PAcc<R>*) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(true, t, e);
-      v[0][e] = valid ? a.W[idx] : cmk<C>(0, 0);
-      v[1][e] = valid ? a.W[(size_t)a.N + idx] : cmk<C>(0, 0);
-    }
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    load_rows<XInvPC>(a, a.W, f, row, valid, t, v);
   }
-  static __device__ void store(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[2][8], PAcc<R>* acc,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-    const int yy = row % a.ny, zz = row / a.ny;
-    const R Yc = -a.Ly + (R)yy * a.hy, Zc = -a.Lz + (R)zz * a.hz;
-    const R vyz = a.vy * Yc * Yc + a.vz * Zc * Zc;
-    R s[PC_NS];
+  template <int NP, bool ST>
+  static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[PC_NS],
+                                const LhyNode<R>*) {
+    PcSumIn<R> in[NP];
 #pragma unroll
-    for (int k = 0; k < PC_NS; ++k) s[k] = 0;
-    constexpr int CH = ChunkW<R>::v;
+    for (int j = 0; j < NP; ++j) pc_sum_load<R>(a, u, pt[j].idx, in[j]);
 #pragma unroll
-    for (int e0 = 0; e0 < 8; e0 += CH) {
-      PcSumIn<R> in[CH];
-#pragma unroll
-      for (int j = 0; j < CH; ++j) pc_sum_load<R>(a, u, (size_t)row * a.nx + Plan<L>::exit_pos(true, t, e0 + j), in[j]);
-#pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const int e = e0 + j;
-        const int x = Plan<L>::exit_pos(true, t, e);
-        const size_t idx = (size_t)row * a.nx + x;
-        C z1 = v[0][e], z2 = v[1][e];
-        if (a.blend) {  // z = (1 - w) P_Delta^{-1} r + w P_V^{-1} r
-          const C ml = a.ax[u.cur][(size_t)a.N + idx];
-          const R X = -a.Lx + (R)x * a.hx;
-          const R V = a.vx * X * X + vyz;
-          const R n1 = cabs2(in[j].p1), n2 = cabs2(in[j].p2);
-          R P1 = u.shift[0] + V + a.g11 * n1 + a.g12 * n2 + ml.x;
-          R P2 = u.shift[1] + V + a.g21 * n1 + a.g22 * n2 + ml.y;
-          P1 = P1 > u.floor_[0] ? P1 : u.floor_[0];
-          P2 = P2 > u.floor_[1] ? P2 : u.floor_[1];
-          const R wd = R(1) - u.wv, w1 = u.wv / P1, w2 = u.wv / P2;
-          z1 = cmk<C>(wd * z1.x + w1 * in[j].r1.x, wd * z1.y + w1 * in[j].r1.y);
-          z2 = cmk<C>(wd * z2.x + w2 * in[j].r2.x, wd * z2.y + w2 * in[j].r2.y);
-        }
-        a.z[idx] = z1;
-        a.z[(size_t)a.N + idx] = z2;
-        pc_sum_add<R>(in[j], z1, z2, s);
+    for (int j = 0; j < NP; ++j) {
+      const size_t idx = pt[j].idx;
+      C z1 = pt[j].out(0), z2 = pt[j].out(1);
+      if (a.blend) {  // z = (1 - w) P_Delta^{-1} r + w P_V^{-1} r
+        const C ml = pick(a.ax, u.cur)[(size_t)a.N + idx];
+        const R V = trap_x(a, pt[j].x) + pt[j].vyz;
+        const R n1 = cabs2(in[j].p1), n2 = cabs2(in[j].p2);
+        const R wd = R(1) - u.wv;
+        const R w1 = u.wv * rcp_(pv_at(a, u, 0, V, n1, n2, ml.x)), w2 = u.wv * rcp_(pv_at(a, u, 1, V, n1, n2, ml.y));
+        z1 = cmk<C>(wd * z1.x + w1 * in[j].r1.x, wd * z1.y + w1 * in[j].r1.y);
+        z2 = cmk<C>(wd * z2.x + w2 * in[j].r2.x, wd * z2.y + w2 * in[j].r2.y);
       }
+      a.z[idx] = z1;
+      a.z[(size_t)a.N + idx] = z2;
+      pc_sum_add<R>(in[j], z1, z2, s);
     }
-#pragma unroll
-    for (int k = 0; k < PC_NS; ++k) acc[k].add(s[k]);
   }
   static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->pc; }
   static __device__ void finish(const KArgs<R>& a, Uni&) {
@@ -1105,12 +1220,12 @@ __device__ __forceinline__ void pc_point_body(const KArgs<R>& a) {
     const int x = (int)(idx % a.nx);
     const int y = (int)((idx / a.nx) % a.ny);
     const int z = (int)(idx / nxy);
-    const R X = -a.Lx + (R)x * a.hx, Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
-    const R V = a.vx * X * X + a.vy * Y * Y + a.vz * Z * Z;
-    C w1, w2;
-    PcIn<R> in;
-    pc_load<R>(a, u, idx, in);
-    pc_apply<R>(a, u, idx, V, in, w1, w2);
+    const R V = trap_x(a, x) + (a.vt[a.nx + y] + a.vt[a.nx + a.ny + z]);
+    C w[2][1];
+    const size_t id[1] = {idx};
+    const R Vp[1] = {V};
+    pc_residual<R, 1, 2>(a, u, 0, id, Vp, w);
+    const C w1 = w[0][0], w2 = w[1][0];
     a.z[idx] = w1;
     a.z[N + idx] = w2;
     R s[PC_NS];
@@ -1159,71 +1274,109 @@ template <class R_, int L_> struct XFwdLC {
   static constexpr const char* NAME = "x-fwd line dir";
   static double alg_bytes(const KArgs<R>& a) { return 11.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 3, NS = 0;
-  static constexpr bool INV = false, USES_LHY = false;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   using Uni = LcUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { lc_uniform(a, u); }
-  static __device__ void load(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[3][8], PAcc<R>*) {
-    const size_t N = a.N;
-    const C* ps = a.psi[u.cur];
-    C* pd = a.pb[u.nsel];
-    const C* pp = a.pb[u.nsel ^ 1];
-    const C* wsrc = u.fallback ? a.rb[u.nsel] : a.z;
-    const bool usepp = !u.pgiven && u.beta != R(0);
-    constexpr int CH = ChunkW<R>::v;
+  // direction p_i = -z_i + beta p_prev_i - c_i psi_i (the residual in place of z in
+  // a fallback step) at one point; psi_i is returned beside it
+  static __device__ C dir(const KArgs<R>& a, const Uni& u, int i, size_t idx, C& p) {
+    const size_t k = (size_t)i * a.N + idx;
+    p = pick(a.psi, u.cur)[k];
+    if (u.pgiven) return pick(a.pb, u.nsel)[k];
+    const C w = u.fallback ? pick(a.rb, u.nsel)[k] : a.z[k];
+    const R c = pick(u.c, i);
+    C q = cmk<C>(fma_(-c, p.x, -w.x), fma_(-c, p.y, -w.y));
+    if (u.beta != R(0)) {
+      const C d = pick(a.pb, u.nsel ^ 1)[k];
+      q = cmk<C>(fma_(u.beta, d.x, q.x), fma_(u.beta, d.y, q.y));
+    }
+    return q;
+  }
+  static __device__ C source(const KArgs<R>& a, C p1, C q1, C p2, C q2) {
+    const R rho1 = cdot(p1, q1), rho2 = cdot(p2, q2);
+    return cmk<C>(fma_(a.d12, rho2, a.d11 * rho1), fma_(a.d22, rho2, a.d21 * rho1));
+  }
+  // fields 0, 1: p (stored unless given); field 2: the packed source of rho = Re(psi conj p)
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    const size_t base = (size_t)row * a.nx, N = a.N;
+    if (!valid) {
 #pragma unroll
-    for (int e0 = 0; e0 < 8; e0 += CH) {
-      C p1[CH], p2[CH], w1[CH], w2[CH], d1[CH], d2[CH];
+      for (int e = 0; e < 8; ++e)
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
-        const size_t id = valid ? idx : 0;
-        p1[j] = ps[id];
-        p2[j] = ps[N + id];
-        w1[j] = u.pgiven ? pd[id] : wsrc[id];
-        w2[j] = u.pgiven ? pd[N + id] : wsrc[N + id];
-        if (usepp) {
-          d1[j] = pp[id];
-          d2[j] = pp[N + id];
+        for (int k = 0; k < NV; ++k) v[k][e] = cmk<C>(0, 0);
+      return;
+    }
+    C* dst = pick(a.pb, u.nsel);
+    if constexpr (NV == 1) {
+      if (f < 2) {
+        C p;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[0][e] = dir(a, u, f, base + Plan<L>::entry_pos(false, t, e), p);
+        if (!u.pgiven) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) dst[(size_t)f * N + base + Plan<L>::entry_pos(false, t, e)] = v[0][e];
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const size_t idx = base + Plan<L>::entry_pos(false, t, e);
+          C p1, p2;
+          const C q1 = dir(a, u, 0, idx, p1), q2 = dir(a, u, 1, idx, p2);
+          v[0][e] = source(a, p1, q1, p2, q2);
         }
       }
+    } else {
+      // both components at once, the loads of a chunk before its arithmetic
+      const C* ps = pick(a.psi, u.cur);
+      const C* pp = pick(a.pb, u.nsel ^ 1);
+      const C* ws = u.pgiven ? dst : u.fallback ? pick(a.rb, u.nsel) : a.z;
+      const bool usepp = !u.pgiven && u.beta != R(0);
+      constexpr int CH = ChunkW<R>::v;
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const int e = e0 + j;
-        C q1 = cmk<C>(0, 0), q2 = cmk<C>(0, 0);
-        R rho1 = 0, rho2 = 0;
-        if (valid) {
-          if (u.pgiven) {
-            q1 = w1[j];
-            q2 = w2[j];
-          } else {
-            q1 = cmk<C>(-w1[j].x - u.c[0] * p1[j].x, -w1[j].y - u.c[0] * p1[j].y);
-            q2 = cmk<C>(-w2[j].x - u.c[1] * p2[j].x, -w2[j].y - u.c[1] * p2[j].y);
-            if (usepp) {
-              q1 = cmk<C>(q1.x + u.beta * d1[j].x, q1.y + u.beta * d1[j].y);
-              q2 = cmk<C>(q2.x + u.beta * d2[j].x, q2.y + u.beta * d2[j].y);
-            }
-            const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e);
-            pd[idx] = q1;
-            pd[N + idx] = q2;
+      for (int e0 = 0; e0 < 8; e0 += CH) {
+        C p1[CH], p2[CH], d1[CH], d2[CH];
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          const size_t idx = base + Plan<L>::entry_pos(false, t, e0 + j);
+          p1[j] = ps[idx];
+          p2[j] = ps[N + idx];
+          v[0][e0 + j] = ws[idx];
+          v[1][e0 + j] = ws[N + idx];
+          if (usepp) {
+            d1[j] = pp[idx];
+            d2[j] = pp[N + idx];
           }
-          rho1 = cdot(p1[j], q1);
-          rho2 = cdot(p2[j], q2);
         }
-        v[0][e] = q1;
-        v[1][e] = q2;
-        v[2][e] = cmk<C>(a.d11 * rho1 + a.d12 * rho2, a.d21 * rho1 + a.d22 * rho2);
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          if (u.pgiven) continue;
+          C q1 = v[0][e0 + j], q2 = v[1][e0 + j];
+          q1 = cmk<C>(fma_(-u.c[0], p1[j].x, -q1.x), fma_(-u.c[0], p1[j].y, -q1.y));
+          q2 = cmk<C>(fma_(-u.c[1], p2[j].x, -q2.x), fma_(-u.c[1], p2[j].y, -q2.y));
+          if (usepp) {
+            q1 = cmk<C>(fma_(u.beta, d1[j].x, q1.x), fma_(u.beta, d1[j].y, q1.y));
+            q2 = cmk<C>(fma_(u.beta, d2[j].x, q2.x), fma_(u.beta, d2[j].y, q2.y));
+          }
+          v[0][e0 + j] = q1;
+          v[1][e0 + j] = q2;
+        }
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          const int e = e0 + j;
+          if (!u.pgiven) {
+            const size_t idx = base + Plan<L>::entry_pos(false, t, e);
+            dst[idx] = v[0][e];
+            dst[N + idx] = v[1][e];
+          }
+          v[2][e] = source(a, p1[j], v[0][e], p2[j], v[1][e]);
+        }
       }
     }
   }
-  static __device__ void store(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[3][8], PAcc<R>*,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::exit_pos(false, t, e);
-#pragma unroll
-      for (int f = 0; f < 3; ++f) a.W[(size_t)f * a.N + idx] = v[f][e];
-    }
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XFwdLC>(a, a.W, f, row, valid, t, v);
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -1235,32 +1388,30 @@ template <class R_, int L_> struct ZLc {
   static constexpr const char* NAME = "z line coeffs";
   static double alg_bytes(const KArgs<R>& a) { return 4.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NS = 2, AXIS = 2;
-  using Uni = NoUni;
-  static __device__ void uniform(const KArgs<R>&, Uni&) {}
+  using Uni = KzLine<R, L_>;
+  static __device__ void uniform(const KArgs<R>& a, Uni& u, int t) { u.set(a, t); }
   static constexpr bool FIRST_INV = false;
   static __device__ const C* src(const KArgs<R>& a) { return a.W; }
   template <class SI>
-  static __device__ void process(const KArgs<R>& a, Uni&, int f, int x, int y, size_t base, size_t ls, int t,
+  static __device__ void process(const KArgs<R>& a, Uni& u, int f, int x, int y, size_t base, size_t ls, int t,
                                  C (&v)[1][8], C* sm, const C* tw, SI si, PAcc<R>* acc) {
     fft_line<C, L, false, 1>(v, sm, 0, tw, t, si);
-    const R kx = wavenum<R>(x, a.nx, a.dkx), ky = wavenum<R>(y, a.ny, a.dky);
-    const R kxy2 = kx * kx + ky * ky;
+    const R kxy = kq_xy(a, x, y);
     if (f < 2) {  // <p_f | T | p_f> by Parseval: forward transform only
       R tk = 0;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        const R kz = wavenum<R>(Plan<L>::exit_pos(false, t, e), a.nz, a.dkz);
-        tk += R(0.5) * (kxy2 + kz * kz) * cabs2(v[0][e]);
+        const R kz = u.kz[e];
+        tk = fma_(kxy + kz, cabs2(v[0][e]), tk);
       }
-      acc[f].add(tk);
+      if (f == 0) acc[0].add(tk);
+      else acc[1].add(tk);
       return;
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const R kz = wavenum<R>(Plan<L>::exit_pos(false, t, e), a.nz, a.dkz);
-      const R k2 = kxy2 + kz * kz;
-      const R mult = (k2 > R(0)) ? (R(3) * kz * kz / k2 - R(1)) * a.invN : R(0);
-      v[0][e] = cscale(v[0][e], mult);
+      const R kz = u.kz[e];
+      v[0][e] = cscale(v[0][e], dip_mult(a, kz, kxy + kz));
     }
     col_after<L>(sm, si);
     fft_line<C, L, true, 1>(v, sm, 0, tw, t, si);
@@ -1274,72 +1425,66 @@ template <class R_, int L_> struct ZLc {
 template <class R_, int L_> struct XInvLC {
   using R = R_;
   using C = C2<R>;
-  static constexpr int MINB = sizeof(R_) == 4 ? EGPE_LC_MINB : 1;
+  static constexpr int PTS = 4, MAXT = sizeof(R_) == 4 ? 256 : 64, MINB = sizeof(R_) == 4 ? 2 : 1;
   static constexpr const char* NAME = "x-inv line sums+LHY";
   static double alg_bytes(const KArgs<R>& a) { return 9.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 1, NS = LC_NS;
-  static constexpr bool INV = true, USES_LHY = true, LHY_TAB = true;
+  static constexpr bool INV = true, USES_LHY = true, LHY_TAB = true, POINTS = true;
   using Uni = LcUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { lc_uniform(a, u); }
-  static __device__ void load(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[1][8], PAcc<R>*) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      v[0][e] = valid ? a.W[(size_t)2 * a.N + (size_t)row * a.nx + Plan<L>::entry_pos(true, t, e)] : cmk<C>(0, 0);
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni&, int, int row, bool valid, int t, C (&v)[NV][8]) {
+    load_rows<XInvLC>(a, a.W, 2, row, valid, t, v);
   }
-  static constexpr int NP = LhyNP<R>::v;
-  static __device__ void store(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[1][8], PAcc<R>* acc,
-                               const LhyNode<R>* nodes) {
-    if (!valid) return;
+  template <int NP, bool ST>
+  static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[LC_NS],
+                                const LhyNode<R>* nodes) {
     const size_t N = a.N;
-    const C* ps = a.psi[u.cur];
-    const C* pd = a.pb[u.nsel];
-    const C* hp = a.hp[u.cur];
-    const C* ax = a.ax[u.cur];
-    const int y = row % a.ny, z = row / a.ny;
-    const R Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
-    const R vyz = a.vy * Y * Y + a.vz * Z * Z;
-    const LhyCoef<R> cf = lhy_coef(a);
-    R s[LC_NS];
+    const C* ps = pick(a.psi, u.cur);
+    const C* pd = pick(a.pb, u.nsel);
+    const C* hp = pick(a.hp, u.cur);
+    const C* ax = pick(a.ax, u.cur);
+    R n1[NP], n2[NP], n1p[NP], n2p[NP], Hh[NP];
+    C p1[NP], p2[NP], q1[NP], q2[NP], h1[NP], h2[NP], phi[NP], ml[NP];
 #pragma unroll
-    for (int k = 0; k < LC_NS; ++k) s[k] = 0;
-#pragma unroll
-    for (int e0 = 0; e0 < 8; e0 += NP) {
-      R n1[NP], n2[NP], n1p[NP], n2p[NP], Hh[NP];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        const int e = e0 + j;
-        const int x = Plan<L>::exit_pos(true, t, e);
-        const size_t idx = (size_t)row * a.nx + x;
-        const C p1 = ps[idx], p2 = ps[N + idx];
-        const C q1 = pd[idx], q2 = pd[N + idx];
-        const C h1 = hp[idx], h2 = hp[N + idx];
-        const C phi = ax[idx], ml = ax[N + idx];
-        n1[j] = cabs2(p1);
-        n2[j] = cabs2(p2);
-        const R a1 = cabs2(q1), a2 = cabs2(q2);
-        const R rho1 = cdot(p1, q1), rho2 = cdot(p2, q2);
-        n1p[j] = R(2) * rho1;
-        n2p[j] = R(2) * rho2;
-        const R X = -a.Lx + (R)x * a.hx;
-        const R V = a.vx * X * X + vyz;
-        const R U1 = V + a.g11 * n1[j] + a.g12 * n2[j] + phi.x + ml.x;
-        const R U2 = V + a.g21 * n1[j] + a.g22 * n2[j] + phi.y + ml.y;
-        s[LC_P1] += a1;
-        s[LC_P2] += a2;
-        s[LC_PSIP1] += rho1;
-        s[LC_PSIP2] += rho2;
-        s[LC_PH1] += cdot(q1, h1);
-        s[LC_PH2] += cdot(q2, h2);
-        s[LC_UPP1] += U1 * a1;
-        s[LC_UPP2] += U2 * a2;
-        s[LC_SRHO] += rho1 * (a.g11 * rho1 + a.g12 * rho2 + v[0][e].x) + rho2 * (a.g21 * rho1 + a.g22 * rho2 + v[0][e].y);
-      }
-      lhy_second<R, NP>(a, nodes, cf, n1, n2, n1p, n2p, Hh);
-#pragma unroll
-      for (int j = 0; j < NP; ++j) s[LC_HLHY] += Hh[j];
+    for (int j = 0; j < NP; ++j) {
+      const size_t idx = pt[j].idx;
+      p1[j] = ps[idx];
+      p2[j] = ps[N + idx];
+      q1[j] = pd[idx];
+      q2[j] = pd[N + idx];
+      h1[j] = hp[idx];
+      h2[j] = hp[N + idx];
+      phi[j] = ax[idx];
+      ml[j] = ax[N + idx];
     }
 #pragma unroll
-    for (int k = 0; k < LC_NS; ++k) acc[k].add(s[k]);
+    for (int j = 0; j < NP; ++j) {
+      n1[j] = cabs2(p1[j]);
+      n2[j] = cabs2(p2[j]);
+      const R a1 = cabs2(q1[j]), a2 = cabs2(q2[j]);
+      const R rho1 = cdot(p1[j], q1[j]), rho2 = cdot(p2[j], q2[j]);
+      n1p[j] = rho1 + rho1;
+      n2p[j] = rho2 + rho2;
+      const C PR = pt[j].out(0);
+      const R V = trap_x(a, pt[j].x) + pt[j].vyz;
+      const R U1 = fma_(a.g12, n2[j], fma_(a.g11, n1[j], (V + phi[j].x) + ml[j].x));
+      const R U2 = fma_(a.g22, n2[j], fma_(a.g21, n1[j], (V + phi[j].y) + ml[j].y));
+      s[LC_P1] += a1;
+      s[LC_P2] += a2;
+      s[LC_PSIP1] += rho1;
+      s[LC_PSIP2] += rho2;
+      cdot_add(s[LC_PH1], q1[j], h1[j]);
+      cdot_add(s[LC_PH2], q2[j], h2[j]);
+      s[LC_UPP1] = fma_(U1, a1, s[LC_UPP1]);
+      s[LC_UPP2] = fma_(U2, a2, s[LC_UPP2]);
+      s[LC_SRHO] = fma_(rho1, fma_(a.g12, rho2, fma_(a.g11, rho1, PR.x)), s[LC_SRHO]);
+      s[LC_SRHO] = fma_(rho2, fma_(a.g22, rho2, fma_(a.g21, rho1, PR.y)), s[LC_SRHO]);
+    }
+    lhy_second<R, NP>(a, nodes, lhy_coef(a), n1, n2, n1p, n2p, Hh);
+#pragma unroll
+    for (int j = 0; j < NP; ++j)
+      s[LC_HLHY] += Hh[j];
   }
   static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->lc; }
   static __device__ void finish(const KArgs<R>& a, Uni&) {
@@ -1365,7 +1510,7 @@ template <class R_, int L_> struct XFwdKin {
   static constexpr const char* NAME = "x-fwd ITE half step";
   static double alg_bytes(const KArgs<R>& a) { return (a.flag ? 6.0 : 4.0) * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 2, NS = 0;
-  static constexpr bool INV = false, USES_LHY = false;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   struct Uni {
     int cur;
     R dtau;
@@ -1374,56 +1519,35 @@ template <class R_, int L_> struct XFwdKin {
     u.cur = __ldcg(&a.st->cur);
     u.dtau = a.kin_tab[a.nx + a.ny + a.nz];
   }
-  static __device__ void load(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[2][8], PAcc<R>*) {
-    const C* ps = a.psi[u.cur];
-    const C* ax = a.ax[u.cur];
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8]) {
     const size_t N = a.N;
-    const int y = row % a.ny, z = row / a.ny;
-    const R Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
-    const R vyz = a.vy * Y * Y + a.vz * Z * Z;
-    constexpr int CH = ChunkW<R>::v;
+    const C* ps = pick(a.psi, u.cur);
+    load_rows<XFwdKin>(a, ps, f, row, valid, t, v);
+    if (!a.flag || !valid) return;
+    const C* ax = pick(a.ax, u.cur);
+    const R vyz = trap_yz(a, row);
 #pragma unroll
-    for (int e0 = 0; e0 < 8; e0 += CH) {
-      C p1[CH], p2[CH], f0[CH], f1[CH];
+    for (int e = 0; e < 8; ++e) {
+      const int x = Plan<L>::entry_pos(false, t, e);
+      const size_t idx = (size_t)row * a.nx + x;
+      const R V = trap_x(a, x) + vyz;
+      const C phi = ax[idx], ml = ax[N + idx];
+      R n[2];  // NV = 1: component f, then the other
+      n[0] = cabs2(v[0][e]);
+      n[1] = cabs2(NV == 1 ? ps[(f ? 0 : N) + idx] : v[NV - 1][e]);
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
-        const size_t id = valid ? idx : 0;
-        p1[j] = ps[id];
-        p2[j] = ps[N + id];
-        if (a.flag) {
-          f0[j] = ax[id];
-          f1[j] = ax[N + id];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const int e = e0 + j;
-        C q1 = valid ? p1[j] : cmk<C>(0, 0), q2 = valid ? p2[j] : cmk<C>(0, 0);
-        if (a.flag && valid) {
-          const int x = Plan<L>::entry_pos(false, t, e);
-          const R X = -a.Lx + (R)x * a.hx;
-          const R V = a.vx * X * X + vyz;
-          const R n1 = cabs2(q1), n2 = cabs2(q2);
-          const R U1 = V + a.g11 * n1 + a.g12 * n2 + f0[j].x + f1[j].x;
-          const R U2 = V + a.g21 * n1 + a.g22 * n2 + f0[j].y + f1[j].y;
-          q1 = cscale(q1, exp(-u.dtau * U1));
-          q2 = cscale(q2, exp(-u.dtau * U2));
-        }
-        v[0][e] = q1;
-        v[1][e] = q2;
+      for (int k = 0; k < NV; ++k) {
+        const int c = f + k;
+        const R n1 = NV == 1 && f ? n[1] : n[0], n2 = NV == 1 && f ? n[0] : n[1];
+        const R U = fma_(c ? a.g22 : a.g12, n2, fma_(c ? a.g21 : a.g11, n1, V + ((c ? phi.y : phi.x) + (c ? ml.y : ml.x))));
+        v[k][e] = cscale(v[k][e], exp(-u.dtau * U));
       }
     }
   }
-  static __device__ void store(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[2][8], PAcc<R>*,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::exit_pos(false, t, e);
-      a.W[idx] = v[0][e];
-      a.W[(size_t)a.N + idx] = v[1][e];
-    }
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XFwdKin>(a, a.W, f, row, valid, t, v);
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -1436,7 +1560,7 @@ template <class R_, int L_> struct ZKin {
   static double alg_bytes(const KArgs<R>& a) { return 4.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NS = 0, AXIS = 2;
   using Uni = NoUni;
-  static __device__ void uniform(const KArgs<R>&, Uni&) {}
+  static __device__ void uniform(const KArgs<R>&, Uni&, int) {}
   static constexpr bool FIRST_INV = false;
   static __device__ const C* src(const KArgs<R>& a) { return a.W; }
   template <class SI>
@@ -1464,34 +1588,27 @@ template <class R_, int L_> struct XInvKin {
   static constexpr const char* NAME = "x-inv ITE half step";
   static double alg_bytes(const KArgs<R>& a) { return 4.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 2, NS = 2;
-  static constexpr bool INV = true, USES_LHY = false;
+  static constexpr bool INV = true, USES_LHY = false, POINTS = false;
   struct Uni {
     int cur;
   };
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { u.cur = __ldcg(&a.st->cur); }
-  static __device__ void load(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[2][8], PAcc<R>*) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(true, t, e);
-      v[0][e] = valid ? a.W[idx] : cmk<C>(0, 0);
-      v[1][e] = valid ? a.W[(size_t)a.N + idx] : cmk<C>(0, 0);
-    }
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    load_rows<XInvKin>(a, a.W, f, row, valid, t, v);
   }
-  static __device__ void store(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[2][8], PAcc<R>* acc,
-                               const LhyNode<R>*) {
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>* acc) {
     if (!valid) return;
-    C* ps = a.psi[u.cur];
-    R s0 = 0, s1 = 0;
+    store_rows<XInvKin>(a, pick(a.psi, u.cur), f, row, valid, t, v);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const size_t idx = (size_t)row * a.nx + Plan<L>::exit_pos(true, t, e);
-      ps[idx] = v[0][e];
-      ps[(size_t)a.N + idx] = v[1][e];
-      s0 += cabs2(v[0][e]);
-      s1 += cabs2(v[1][e]);
+    for (int k = 0; k < NV; ++k) {
+      R s = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) cdot_add(s, v[k][e], v[k][e]);
+      if (f + k == 0) acc[0].add(s);
+      else acc[1].add(s);
     }
-    acc[0].add(s0);
-    acc[1].add(s1);
   }
   static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->rt; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -1512,7 +1629,7 @@ template <class R> __device__ __forceinline__ void ite_scale_body(const KArgs<R>
     s1 = __shfl_sync(0xffffffffu, sc, 0);
     s2 = __shfl_sync(0xffffffffu, sc, 1);
   }
-  C2<R>* ps = a.psi[cur];
+  C2<R>* ps = pick(a.psi, cur);
   const size_t N = a.N;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += (size_t)gridDim.x * blockDim.x) {
     ps[idx] = cscale(ps[idx], s1);
@@ -1537,13 +1654,14 @@ template <class R_, int L_> struct XFwdPG {
   static constexpr const char* NAME = "x-fwd densities (param grad)";
   static double alg_bytes(const KArgs<R>& a) { return 3.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 1, NS = 0;
-  static constexpr bool INV = false, USES_LHY = false;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   struct Uni {
     int cur;
   };
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { u.cur = __ldcg(&a.st->cur); }
-  static __device__ void load(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[1][8], PAcc<R>*) {
-    const C* ps = a.psi[u.cur];
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int, int row, bool valid, int t, C (&v)[NV][8]) {
+    const C* ps = pick(a.psi, u.cur);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const size_t idx = valid ? (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e) : 0;
@@ -1551,11 +1669,9 @@ template <class R_, int L_> struct XFwdPG {
       v[0][e] = valid ? cmk<C>(cabs2(p1), cabs2(p2)) : cmk<C>(0, 0);
     }
   }
-  static __device__ void store(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[1][8], PAcc<R>*,
-                               const LhyNode<R>*) {
-    if (!valid) return;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) a.W[(size_t)row * a.nx + Plan<L>::exit_pos(false, t, e)] = v[0][e];
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XFwdPG>(a, a.W, f, row, valid, t, v);
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -1567,21 +1683,19 @@ template <class R_, int L_> struct ZPg {
   static constexpr const char* NAME = "z dipolar kernel (param grad)";
   static double alg_bytes(const KArgs<R>& a) { return 2.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NS = 0, AXIS = 2;
-  using Uni = NoUni;
-  static __device__ void uniform(const KArgs<R>&, Uni&) {}
+  using Uni = KzLine<R, L_>;
+  static __device__ void uniform(const KArgs<R>& a, Uni& u, int t) { u.set(a, t); }
   static constexpr bool FIRST_INV = false;
   static __device__ const C* src(const KArgs<R>& a) { return a.W; }
   template <class SI>
-  static __device__ void process(const KArgs<R>& a, Uni&, int, int x, int y, size_t base, size_t ls, int t,
+  static __device__ void process(const KArgs<R>& a, Uni& u, int, int x, int y, size_t base, size_t ls, int t,
                                  C (&v)[1][8], C* sm, const C* tw, SI si, PAcc<R>*) {
     fft_line<C, L, false, 1>(v, sm, 0, tw, t, si);
-    const R kx = wavenum<R>(x, a.nx, a.dkx), ky = wavenum<R>(y, a.ny, a.dky);
-    const R kxy2 = kx * kx + ky * ky;
+    const R kxy = kq_xy(a, x, y);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const R kz = wavenum<R>(Plan<L>::exit_pos(false, t, e), a.nz, a.dkz);
-      const R k2 = kxy2 + kz * kz;
-      v[0][e] = cscale(v[0][e], (k2 > R(0)) ? (R(3) * kz * kz / k2 - R(1)) * a.invN : R(0));
+      const R kz = u.kz[e];
+      v[0][e] = cscale(v[0][e], dip_mult(a, kz, kxy + kz));
     }
     col_after<L>(sm, si);
     fft_line<C, L, true, 1>(v, sm, 0, tw, t, si);
@@ -1595,45 +1709,40 @@ template <class R_, int L_> struct ZPg {
 template <class R_, int L_> struct XInvPG {
   using R = R_;
   using C = C2<R>;
-  static constexpr int MAXT = 128;
+  static constexpr int PTS = 1, MAXT = 128;
   static constexpr const char* NAME = "x-inv parameter sums";
   static double alg_bytes(const KArgs<R>& a) { return 3.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 1, NS = PG_NS;
-  static constexpr bool INV = true, USES_LHY = true;
+  static constexpr bool INV = true, USES_LHY = true, POINTS = true;
   struct Uni {
     int cur;
   };
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { u.cur = __ldcg(&a.st->cur); }
-  static __device__ void load(const KArgs<R>& a, Uni&, int row, bool valid, int t, C (&v)[1][8], PAcc<R>*) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      v[0][e] = valid ? a.W[(size_t)row * a.nx + Plan<L>::entry_pos(true, t, e)] : cmk<C>(0, 0);
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8]) {
+    load_rows<XInvPG>(a, a.W, f, row, valid, t, v);
   }
-  static __device__ void store(const KArgs<R>& a, Uni& u, int row, bool valid, int t, C (&v)[1][8], PAcc<R>* acc,
-                               const LhyNode<R>* nodes) {
-    if (!valid) return;
-    const C* ps = a.psi[u.cur];
-    const int y = row % a.ny, z = row / a.ny;
-    const R Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
+  template <int NP, bool ST>
+  static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[PG_NS],
+                                const LhyNode<R>* nodes) {
+    const C* ps = pick(a.psi, u.cur);
     const LhyCoef<R> cf = lhy_coef(a);
-    R s[PG_NS];
 #pragma unroll
-    for (int k = 0; k < PG_NS; ++k) s[k] = R(0);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int x = Plan<L>::exit_pos(true, t, e);
-      const size_t idx = (size_t)row * a.nx + x;
+    for (int j = 0; j < NP; ++j) {
+      const size_t idx = pt[j].idx;
+      const int row = (int)(idx / a.nx), y = row % a.ny, z = row / a.ny;
+      const R X = -a.Lx + (R)pt[j].x * a.hx, Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
       const R n1 = cabs2(ps[idx]), n2 = cabs2(ps[(size_t)a.N + idx]);
-      const R X = -a.Lx + (R)x * a.hx;
+      const C K = pt[j].out(0);
       const R nt = n1 + n2;
       R lh[7];
       lhy_eta_sums<R>(nodes, a.Q, cf, n1, n2, lh);
       s[PG_N11] += n1 * n1;
       s[PG_N12] += n1 * n2;
       s[PG_N22] += n2 * n2;
-      s[PG_K11] += n1 * v[0][e].x;
-      s[PG_K12] += n1 * v[0][e].y;
-      s[PG_K22] += n2 * v[0][e].y;
+      s[PG_K11] += n1 * K.x;
+      s[PG_K12] += n1 * K.y;
+      s[PG_K22] += n2 * K.y;
       s[PG_X2] += X * X * nt;
       s[PG_Y2] += Y * Y * nt;
       s[PG_Z2] += Z * Z * nt;
@@ -1645,8 +1754,6 @@ template <class R_, int L_> struct XInvPG {
       s[PG_M22] += lh[5];
       s[PG_M12] += lh[6];
     }
-#pragma unroll
-    for (int k = 0; k < PG_NS; ++k) acc[k].add(s[k]);
   }
   static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->pg; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
@@ -1689,8 +1796,8 @@ template <class R> __global__ void __launch_bounds__(256) resnorm_kernel(KArgs<R
   R mu[2];
   load_uniforms<R, 2>({&a.st->mu[0], &a.st->mu[1]}, mu);
   const size_t N = a.N;
-  const C2<R>* ps = a.psi[cur];
-  const C2<R>* hp = a.hp[cur];
+  const C2<R>* ps = pick(a.psi, cur);
+  const C2<R>* hp = pick(a.hp, cur);
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += (size_t)gridDim.x * blockDim.x) {
     for (int i = 0; i < 2; ++i) {
       const C2<R> u = ps[i * N + idx], h = hp[i * N + idx];

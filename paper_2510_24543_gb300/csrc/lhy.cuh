@@ -17,7 +17,26 @@
 
 namespace egpe {
 
-__device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
+// Reciprocal and reciprocal square root of the FP64 kernels, which the FP64 pipe
+// bounds: the hardware's approximate instruction (about 20 bits) and one
+// third-order step of Newton's family (Householder's method), three and five FP64
+// instructions without branches.  With e = 1 - x y for an approximation y of 1/x,
+// 1/x = y (1 + e + e^2 + ...): y + y (e + e^2) leaves e^3 ~ 2^-60.  With
+// e = 1 - x y^2, 1/sqrt(x) = y (1 - e)^{-1/2} = y (1 + e/2 + 3 e^2/8 + ...).
+// Arguments are positive and normal; 0, infinities and NaN give non-finite values.
+__device__ __forceinline__ double rcp_(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float rcp_(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rsqrt_(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 
 // Smallest s^2 treated as nonzero (below it the rsqrt of the field precision
@@ -26,10 +45,13 @@ template <class R> __device__ __forceinline__ R s2_min();
 template <> __device__ __forceinline__ double s2_min<double>() { return 1e-300; }
 template <> __device__ __forceinline__ float s2_min<float>() { return 1e-36f; }
 
-// sqrt(v) of a clamped v >= 0 without branches.  FP64: the library square
-// root; FP32: the translation unit is built with the approximate square root
-// (MUFU, a few ulp).
-__device__ __forceinline__ double sqrt_pos(double v) { return sqrt(v); }
+// sqrt(v) of a clamped v >= 0 without branches.  FP64: v / sqrt(v), 0 below the
+// normal range; FP32: the translation unit is built with the approximate square
+// root (MUFU, a few ulp).
+__device__ __forceinline__ double sqrt_pos(double v) {
+  const double r = v * rsqrt_(v);
+  return v > 1e-300 ? r : 0.0;
+}
 __device__ __forceinline__ float sqrt_pos(float v) { return sqrtf(v); }
 
 // 1/s (0 where s^2 is below the threshold) and s = s^2 / s.
@@ -151,8 +173,7 @@ template <class R> __device__ __forceinline__ LhyPt<R> lhy_pt(const LhyCoef<R>& 
 // (independent dependency chains per node).
 template <class R, int NP>
 __device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, int Q, int Qm, const LhyCoef<R>& c,
-                                           const R (&n1)[NP], const R (&n2)[NP], R (&F)[NP], R (&mu1)[NP],
-                                           R (&mu2)[NP]) {
+                                           const R (&n1)[NP], const R (&n2)[NP], R (&mu1)[NP], R (&mu2)[NP]) {
   if constexpr (std::is_same<R, double>::value) {
     // every term below FP64 rounding (see LhyCoef::nskip).  FP64 only: the FP32
     // transforms leave a round-off floor of ~1e-7 in amplitude everywhere, so
@@ -162,7 +183,7 @@ __device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, in
     for (int j = 0; j < NP; ++j) any |= n1[j] + n2[j] > c.nskip;
     if (!any) {
 #pragma unroll
-      for (int j = 0; j < NP; ++j) F[j] = mu1[j] = mu2[j] = R(0);
+      for (int j = 0; j < NP; ++j) mu1[j] = mu2[j] = R(0);
       return;
     }
   }
@@ -276,9 +297,6 @@ __device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, in
     const R s22 = -c.d22 * p[j].D1 + n1x2 * c.d12 * c.d12;
     mu1[j] = R(2.5) * (c.g11 * S0[j] + c.d11 * S1[j] + s10 * T0[j] + s11 * T1[j] + s12 * T2[j]);
     mu2[j] = R(2.5) * (c.g22 * S0[j] + c.d22 * S1[j] + s20 * T0[j] + s21 * T1[j] + s22 * T2[j]);
-    // V+- are homogeneous of degree 1 in (n1, n2), so F is of degree 5/2 and
-    // Euler's theorem gives F = (2/5)(n1 mu1 + n2 mu2) exactly
-    F[j] = R(0.4) * (n1[j] * mu1[j] + n2[j] * mu2[j]);
   }
 }
 
@@ -512,8 +530,24 @@ __device__ __forceinline__ double horner_tab(const double* c, double x) {
 template <class R>
 __device__ __forceinline__ const R* lhy_tab_locate(const LhyTab<R>& t, R n1, R n2, R& x, R& rs) {
   const R n = n1 + n2;
-  rs = rsqrt_(n > R(0) ? n : R(1));
   const bool h = n1 > n2;
+  if constexpr (std::is_same<R, double>::value) {
+    // interval index by adding 1.5 2^52 (round to nearest of the coordinate less
+    // 1/2), which leaves it in the low word: no conversions on the FP64 pipe
+    rs = rsqrt_(n > 1e-300 ? n : 1.0);
+    const double tt = fma(sqrt_pos(h ? n2 : n1) * rs, t.tscale, -0.5);
+    const double g = tt + 6755399441055744.0;
+    const double d = tt - (g - 6755399441055744.0);
+    x = d + d;
+    int i = __double2loint(g);
+    if (i > t.ni - 1) {  // a = 1/sqrt(2) up to rounding
+      x += (double)(2 * (i - (t.ni - 1)));
+      i = t.ni - 1;
+    }
+    i = i < 0 ? 0 : i;
+    return t.tab + (size_t)((h ? t.ni : 0) + i) * LhyTabDim<R>::rec;
+  }
+  rs = rsqrt_(n > R(0) ? n : R(1));
   const R a = sqrt_pos(h ? n2 : n1) * rs;
   const R tt = a * t.tscale;
   int i = (int)tt;  // a <= 1/sqrt(2) up to rounding: clamp to the last interval (NaN converts to 0)

@@ -153,9 +153,18 @@ __device__ __forceinline__ bool reduce_grid(T (&v)[pow2_ceil(NS)], double* __res
   T acc[P];
 #pragma unroll
   for (int s = 0; s < P; ++s) acc[s] = RedT<T>::zero();
-  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+  // two blocks' sums in flight per thread: the last block is small and the loads
+  // are what it waits for
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += 2 * blockDim.x) {
+    const unsigned b1 = b + blockDim.x;
+    T x[NS], y[NS];
 #pragma unroll
-    for (int s = 0; s < NS; ++s) acc[s] = RedT<T>::add(acc[s], RedT<T>::ldcg(&part[(size_t)b * NS + s]));
+    for (int s = 0; s < NS; ++s) {
+      x[s] = RedT<T>::ldcg(&part[(size_t)b * NS + s]);
+      y[s] = b1 < gridDim.x ? RedT<T>::ldcg(&part[(size_t)b1 * NS + s]) : RedT<T>::zero();
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) acc[s] = RedT<T>::add(acc[s], RedT<T>::add(x[s], y[s]));
   }
   const T tot = block_sum_to_thread<T, NS>(acc, sm);
   if (threadIdx.x < NS) out[threadIdx.x] = RedT<T>::value(tot);
