@@ -55,7 +55,7 @@ template <class R> class BatchRunner {
     long long replays = 0, kernels = 0;
     while (!active.empty() && replays < max_launch) {
       if (active != built_) EGPE_TRY(rebuild(active, mode));
-      for (int k = 0; k < poll; ++k) {
+      for (int k = attempts_ahead(poll, max_iter, replays); k > 0; --k) {
         EGPE_CUDA(cudaGraphLaunch(graph_, stream_));
         ++replays;
         kernels += per_replay_;

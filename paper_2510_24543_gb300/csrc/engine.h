@@ -62,6 +62,13 @@ struct SolveRun {
   long long ffts, kernels;
 };
 
+// Attempts to enqueue before the next look at the phase: `poll`, but none beyond
+// the one that finds max_iter reached unless line-search retries used some up.
+inline int attempts_ahead(int poll, int max_iter, long long launched) {
+  const long long left = (long long)max_iter + 1 - launched;
+  return left > 0 && left < poll ? (int)left : poll;
+}
+
 template <class R> class Engine {
  public:
   using C = C2<R>;

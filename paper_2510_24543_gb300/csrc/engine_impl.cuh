@@ -1345,7 +1345,7 @@ egpe_status Engine<R>::solve(const egpe_solve_opts& o, int fp32_phase, int max_i
   const int poll = std::max(1, o.poll_every);
   const long long max_launch = (long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4;
   while (run_launches_ < max_launch) {
-    EGPE_TRY(solve_launch(poll));
+    EGPE_TRY(solve_launch(attempts_ahead(poll, max_iter, run_launches_)));
     int phase = 0;
     EGPE_TRY(solve_poll(phase));
     if (phase == PH_DONE) break;
