@@ -134,7 +134,7 @@ template <class R> egpe_status Engine<R>::apply_params(const egpe_params& p) {
   // interpolated LHY sums and the nodes left to exact evaluation
   const LhyTableHost T = lhy_interp_table_cached<R>(p);
   static_assert(TabSpec<R>::deg + 1 == LhyTabDim<R>::coef, "table layout");
-  std::vector<R> tab(T.coef.begin(), T.coef.end());
+  const std::vector<R> tab = lhy_pack_table<R>(T);
   if (tab_ && tab_elems_ != tab.size()) {
     cudaFree(tab_);
     tab_ = nullptr;

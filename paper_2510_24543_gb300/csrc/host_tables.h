@@ -382,6 +382,34 @@ template <class R> inline LhyTableHost lhy_interp_table(const egpe_params& p) {
   return best;
 }
 
+// The device's records (lhy.cuh) of the tables, 16-byte aligned: per half and
+// interval the coefficients of the kTabFun functions, FP32 as they are, FP64 as
+// 64-bit fixed point with 61 - E fractional bits, sum_k |c_k| <= 2^E, followed by
+// the five exponents E (32-bit) and padding.
+template <class R> inline std::vector<R> lhy_pack_table(const LhyTableHost& T) {
+  return std::vector<R>(T.coef.begin(), T.coef.end());
+}
+template <> inline std::vector<double> lhy_pack_table<double>(const LhyTableHost& T) {
+  const int NC = T.deg + 1, REC = kTabFun * NC + 4;
+  std::vector<double> out((size_t)2 * T.ni * REC);
+  for (int r = 0; r < 2 * T.ni; ++r) {
+    const long double* c = &T.coef[(size_t)r * kTabFun * NC];
+    std::vector<long long> w(REC, 0);
+    int ex[8] = {};
+    for (int f = 0; f < kTabFun; ++f) {
+      long double sum = 0;
+      for (int k = 0; k < NC; ++k) sum += fabsl(c[f * NC + k]);
+      int e = 0;
+      if (sum > 0) frexpl(sum, &e);  // sum < 2^e
+      ex[f] = e;
+      for (int k = 0; k < NC; ++k) w[f * NC + k] = llroundl(ldexpl(c[f * NC + k], 61 - e));
+    }
+    std::memcpy(&w[kTabFun * NC], ex, sizeof(ex));
+    std::memcpy((void*)&out[(size_t)r * REC], w.data(), REC * sizeof(long long));
+  }
+  return out;
+}
+
 // The tables of one parameter set and field type, built once per process
 // (repeated handles share the build); returned by value, so a later eviction
 // cannot invalidate a caller's copy.

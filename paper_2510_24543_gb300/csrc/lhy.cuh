@@ -14,6 +14,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "fft.cuh"
 
 namespace egpe {
 
@@ -484,7 +485,7 @@ __device__ __forceinline__ void lhy_eta_sums(const LhyNode<R>* __restrict__ nd, 
 // Coefficients per function: degree 11 for FP64 fields, degree 7 for FP32.
 template <class R> struct LhyTabDim;
 template <> struct LhyTabDim<double> {
-  static constexpr int coef = 12, rec = 5 * coef;
+  static constexpr int coef = 12, rec = 5 * coef + 4;  // fixed point, with exponents (host_tables.h)
 };
 template <> struct LhyTabDim<float> {
   static constexpr int coef = 8, rec = 5 * coef;
@@ -510,50 +511,67 @@ __device__ __forceinline__ float horner_tab(const float* c, float x) {
   p = fmaf(p, x, a.y);
   return fmaf(p, x, a.x);
 }
-__device__ __forceinline__ double horner_tab(const double* c, double x) {
-  const double2* v = reinterpret_cast<const double2*>(c);
-  double2 k[6];
+// FP64: 64-bit fixed point, x = (h 2^32 + l) 2^-62 and 61 - E fractional bits; a step
+// is twelve integer instructions for one on the FP64 pipe (16 clocks per warp and
+// SM), and keeps eight more bits.
+struct FixedX {
+  int h, l;
+};
+__device__ __forceinline__ double horner_tab(const double* rec, int f, FixedX x) {
+  const longlong2* v = reinterpret_cast<const longlong2*>(rec + f * 12);
+  longlong2 k[6];
 #pragma unroll
   for (int i = 0; i < 6; ++i) k[i] = __ldg(v + i);
-  double p = k[5].y;
-  p = fma(p, x, k[5].x);
+  const int E = __ldg(reinterpret_cast<const int*>(rec + 60) + f);
+__device__ __forceinline__ float horner_tab(const float* rec, int f, float x) { return horner_tab(rec + f * 8, x); }
+template <class R> struct TabX {
+  using T = R;
+};
+template <> struct TabX<double> {
+  using T = FixedX;
+};
+  long long p = k[5].y;
+  p = k[5].x + mulq(p, x.h, x.l);
 #pragma unroll
   for (int i = 4; i >= 0; --i) {
-    p = fma(p, x, k[i].y);
-    p = fma(p, x, k[i].x);
+    p = k[i].y + mulq(p, x.h, x.l);
+    p = k[i].x + mulq(p, x.h, x.l);
   }
-  return p;
+  return from_fixed(p, LineScale{1024 + E, -1, 0});
 }
 
 // Interval record of (n1, n2) and its local coordinate x; rs = 1/sqrt(n) (1
 // where n = 0, whose terms vanish with their n-power prefactor).
 template <class R>
-__device__ __forceinline__ const R* lhy_tab_locate(const LhyTab<R>& t, R n1, R n2, R& x, R& rs) {
+__device__ __forceinline__ const R* lhy_tab_locate(const LhyTab<R>& t, R n1, R n2, typename TabX<R>::T& x, R& rs) {
   const R n = n1 + n2;
   const bool h = n1 > n2;
   if constexpr (std::is_same<R, double>::value) {
     // interval index by adding 1.5 2^52 (round to nearest of the coordinate less
     // 1/2), which leaves it in the low word: no conversions on the FP64 pipe
     rs = rsqrt_(n > 1e-300 ? n : 1.0);
+    const LimbQ xl = limbs(to_fixed(d, LineScale{1022, -1, 0}));  // 2 d in 62 fractional bits
+    x.h = xl.h;
+    x.l = xl.l;
+    return t.tab + (size_t)((h ? t.ni : 0) + i) * LhyTabDim<R>::rec;
+  } else {
+    rs = rsqrt_(n > R(0) ? n : R(1));
+    const R a = sqrt_pos(h ? n2 : n1) * rs;
+    const R tt = a * t.tscale;
+    int i = (int)tt;  // a <= 1/sqrt(2) up to rounding: clamp to the last interval (NaN converts to 0)
+    i = i < 0 ? 0 : (i < t.ni - 1 ? i : t.ni - 1);
+    x = R(2) * (tt - (R)i) - R(1);
     const double tt = fma(sqrt_pos(h ? n2 : n1) * rs, t.tscale, -0.5);
     const double g = tt + 6755399441055744.0;
-    const double d = tt - (g - 6755399441055744.0);
-    x = d + d;
+    double d = tt - (g - 6755399441055744.0);  // x/2
     int i = __double2loint(g);
     if (i > t.ni - 1) {  // a = 1/sqrt(2) up to rounding
-      x += (double)(2 * (i - (t.ni - 1)));
+      d += (double)(i - (t.ni - 1));
       i = t.ni - 1;
     }
     i = i < 0 ? 0 : i;
     return t.tab + (size_t)((h ? t.ni : 0) + i) * LhyTabDim<R>::rec;
   }
-  rs = rsqrt_(n > R(0) ? n : R(1));
-  const R a = sqrt_pos(h ? n2 : n1) * rs;
-  const R tt = a * t.tscale;
-  int i = (int)tt;  // a <= 1/sqrt(2) up to rounding: clamp to the last interval (NaN converts to 0)
-  i = i < 0 ? 0 : (i < t.ni - 1 ? i : t.ni - 1);
-  x = R(2) * (tt - (R)i) - R(1);
-  return t.tab + (size_t)((h ? t.ni : 0) + i) * LhyTabDim<R>::rec;
 }
 
 // The table's part of mu_LHY,1 and mu_LHY,2 at NP points.
@@ -562,12 +580,13 @@ __device__ __forceinline__ void lhy_tab_mu(const LhyTab<R>& t, const R (&n1)[NP]
                                            R (&m2)[NP]) {
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
-    R x, rs;
+    typename TabX<R>::T x;
+    R rs;
     const R* c = lhy_tab_locate(t, n1[j], n2[j], x, rs);
     const R n = n1[j] + n2[j];
     const R n32 = n * n * rs;
-    m1[j] = n32 * horner_tab(c, x);
-    m2[j] = n32 * horner_tab(c + LhyTabDim<R>::coef, x);
+    m1[j] = n32 * horner_tab(c, 0, x);
+    m2[j] = n32 * horner_tab(c, 1, x);
   }
 }
 
@@ -577,12 +596,13 @@ __device__ __forceinline__ void lhy_tab_hess(const LhyTab<R>& t, const R (&n1)[N
                                              const R (&n1p)[NP], const R (&n2p)[NP], R (&H)[NP]) {
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
-    R x, rs;
+    typename TabX<R>::T x;
+    R rs;
     const R* c = lhy_tab_locate(t, n1[j], n2[j], x, rs);
     const R n = n1[j] + n2[j];
-    const R h11 = horner_tab(c + 2 * LhyTabDim<R>::coef, x);
-    const R h12 = horner_tab(c + 3 * LhyTabDim<R>::coef, x);
-    const R h22 = horner_tab(c + 4 * LhyTabDim<R>::coef, x);
+    const R h11 = horner_tab(c, 2, x);
+    const R h12 = horner_tab(c, 3, x);
+    const R h22 = horner_tab(c, 4, x);
     H[j] = n * rs * (n1p[j] * (h11 * n1p[j] + R(2) * h12 * n2p[j]) + h22 * n2p[j] * n2p[j]);
   }
 }
