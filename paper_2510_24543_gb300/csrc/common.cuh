@@ -58,7 +58,7 @@ enum LczSlot { LCZ_TPP1 = 0, LCZ_TPP2, LCZ_NS };
 enum RtSlot { RT_P1 = 0, RT_P2, RT_PSIP1, RT_PSIP2, RT_PSI1, RT_PSI2, RT_NS };
 enum PgSlot {  // parameter-derivative sums (x dV later)
   PG_N11 = 0, PG_N12, PG_N22, PG_K11, PG_K12, PG_K22, PG_X2, PG_Y2, PG_Z2,
-  PG_F, PG_L11, PG_L22, PG_L12, PG_M11, PG_M22, PG_M12, PG_NS
+  PG_L11, PG_L22, PG_L12, PG_M11, PG_M22, PG_M12, PG_NS
 };
 // Default row width in bytes of a column-pass tile (one cache line); the
 // autotuner may pick 64 or 256 for the power-of-two lengths.

@@ -215,14 +215,18 @@ template <class R> egpe_status Engine<R>::param_grad(const C* psi, double out[EG
   EGPE_TRY(read_state(hs));
   const double* s = hs.pg;
   const double kap = prm_.lhy_kappa, eta = prm_.lhy_eta_scale;
+  // the LHY density is of degree 5/2 in the entries of eta = g + gdd w as well
+  // (V_+- are of degree 1), so F = (2/5) sum_ij eta_ij dF/deta_ij (Euler)
+  const double F = 0.4 * (prm_.g[0][0] * s[PG_L11] + prm_.g[1][1] * s[PG_L22] + prm_.g[0][1] * s[PG_L12] +
+                          prm_.gdd[0][0] * s[PG_M11] + prm_.gdd[1][1] * s[PG_M22] + prm_.gdd[0][1] * s[PG_M12]);
   out[EGPE_P_G11] = dV * (0.5 * s[PG_N11] + s[PG_L11]);
   out[EGPE_P_G12] = dV * (s[PG_N12] + s[PG_L12]);
   out[EGPE_P_G22] = dV * (0.5 * s[PG_N22] + s[PG_L22]);
   out[EGPE_P_GDD11] = dV * (0.5 * s[PG_K11] + s[PG_M11]);
   out[EGPE_P_GDD12] = dV * (s[PG_K12] + s[PG_M12]);
   out[EGPE_P_GDD22] = dV * (0.5 * s[PG_K22] + s[PG_M22]);
-  out[EGPE_P_KAPPA] = kap != 0.0 ? dV * s[PG_F] / kap : std::numeric_limits<double>::quiet_NaN();
-  out[EGPE_P_ETA_S] = -2.5 * dV * s[PG_F] / eta;
+  out[EGPE_P_KAPPA] = kap != 0.0 ? dV * F / kap : std::numeric_limits<double>::quiet_NaN();
+  out[EGPE_P_ETA_S] = -2.5 * dV * F / eta;
   out[EGPE_P_TRAP_X] = prm_.trap[0] * dV * s[PG_X2];
   out[EGPE_P_TRAP_Y] = prm_.trap[1] * dV * s[PG_Y2];
   out[EGPE_P_TRAP_Z] = prm_.trap[2] * dV * s[PG_Z2];

@@ -1709,7 +1709,7 @@ template <class R_, int L_> struct ZPg {
 template <class R_, int L_> struct XInvPG {
   using R = R_;
   using C = C2<R>;
-  static constexpr int PTS = 1, MAXT = 128;
+  static constexpr int PTS = 2, MAXT = 128;
   static constexpr const char* NAME = "x-inv parameter sums";
   static double alg_bytes(const KArgs<R>& a) { return 3.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 1, NS = PG_NS;
@@ -1727,32 +1727,30 @@ template <class R_, int L_> struct XInvPG {
                                 const LhyNode<R>* nodes) {
     const C* ps = pick(a.psi, u.cur);
     const LhyCoef<R> cf = lhy_coef(a);
+    R n1[NP], n2[NP], lh[NP][6];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
-      const size_t idx = pt[j].idx;
-      const int row = (int)(idx / a.nx), y = row % a.ny, z = row / a.ny;
-      const R X = -a.Lx + (R)pt[j].x * a.hx, Y = -a.Ly + (R)y * a.hy, Z = -a.Lz + (R)z * a.hz;
-      const R n1 = cabs2(ps[idx]), n2 = cabs2(ps[(size_t)a.N + idx]);
+      n1[j] = cabs2(ps[pt[j].idx]);
+      n2[j] = cabs2(ps[(size_t)a.N + pt[j].idx]);
+    }
+    lhy_eta_sums<R, NP>(nodes, a.Q, a.Qm, cf, n1, n2, lh);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const int row = (int)(pt[j].idx / L), y = row % a.ny, z = row / a.ny;
+      const R X = fma_((R)pt[j].x, a.hx, -a.Lx), Y = fma_((R)y, a.hy, -a.Ly), Z = fma_((R)z, a.hz, -a.Lz);
       const C K = pt[j].out(0);
-      const R nt = n1 + n2;
-      R lh[7];
-      lhy_eta_sums<R>(nodes, a.Q, cf, n1, n2, lh);
-      s[PG_N11] += n1 * n1;
-      s[PG_N12] += n1 * n2;
-      s[PG_N22] += n2 * n2;
-      s[PG_K11] += n1 * K.x;
-      s[PG_K12] += n1 * K.y;
-      s[PG_K22] += n2 * K.y;
-      s[PG_X2] += X * X * nt;
-      s[PG_Y2] += Y * Y * nt;
-      s[PG_Z2] += Z * Z * nt;
-      s[PG_F] += lh[0];
-      s[PG_L11] += lh[1];
-      s[PG_L22] += lh[2];
-      s[PG_L12] += lh[3];
-      s[PG_M11] += lh[4];
-      s[PG_M22] += lh[5];
-      s[PG_M12] += lh[6];
+      const R nt = n1[j] + n2[j];
+      s[PG_N11] = fma_(n1[j], n1[j], s[PG_N11]);
+      s[PG_N12] = fma_(n1[j], n2[j], s[PG_N12]);
+      s[PG_N22] = fma_(n2[j], n2[j], s[PG_N22]);
+      s[PG_K11] = fma_(n1[j], K.x, s[PG_K11]);
+      s[PG_K12] = fma_(n1[j], K.y, s[PG_K12]);
+      s[PG_K22] = fma_(n2[j], K.y, s[PG_K22]);
+      s[PG_X2] = fma_(X * X, nt, s[PG_X2]);
+      s[PG_Y2] = fma_(Y * Y, nt, s[PG_Y2]);
+      s[PG_Z2] = fma_(Z * Z, nt, s[PG_Z2]);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) s[PG_L11 + k] += lh[j][k];
     }
   }
   static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->pg; }

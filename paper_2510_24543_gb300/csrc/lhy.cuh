@@ -164,17 +164,20 @@ template <class R> __device__ __forceinline__ LhyPt<R> lhy_pt(const LhyCoef<R>& 
   return p;
 }
 
-// F = sum_q W_q sum_+- max(V,0)^{5/2};  mu_i = dF/dn_i
-//   = sum_q W_q (5/2) sum_+- max(V,0)^{3/2} (eta_ii +- sigma_i/s),
-// sigma_1 = eta11 delta + 2 eta12^2 n2, sigma_2 = -eta22 delta + 2 eta12^2 n1
-// (the paper's mu_LHY, Sec. II).  With S_k = sum W w^k (V+^{3/2} + V-^{3/2}) and
-// T_k = sum W w^k (V+^{3/2} - V-^{3/2})/s, and sigma_i(w) quadratic in w:
-//   mu_i = 5/2 (g_ii S_0 + gdd_ii S_1 + sigma_i0 T_0 + sigma_i1 T_1 + sigma_i2 T_2).
+// The node sums every first derivative of F = sum_q W_q sum_+- max(V,0)^{5/2} is
+// made of:
+//   S_k = sum_q W w^k (V+^{3/2} + V-^{3/2}),  T_k = sum_q W w^k (V+^{3/2} - V-^{3/2})/s.
 // W_q already includes kappa eta_s^{-5/2}.  NP points are evaluated together
 // (independent dependency chains per node).
 template <class R, int NP>
-__device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, int Q, int Qm, const LhyCoef<R>& c,
-                                           const R (&n1)[NP], const R (&n2)[NP], R (&mu1)[NP], R (&mu2)[NP]) {
+__device__ __forceinline__ void lhy_moments(const LhyNode<R>* __restrict__ nd, int Q, int Qm, const LhyCoef<R>& c,
+                                            const R (&n1)[NP], const R (&n2)[NP], LhyPt<R> (&p)[NP], R (&S0)[NP],
+                                            R (&S1)[NP], R (&T0)[NP], R (&T1)[NP], R (&T2)[NP]) {
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    p[j] = lhy_pt(c, n1[j], n2[j]);
+    S0[j] = S1[j] = T0[j] = T1[j] = T2[j] = R(0);
+  }
   if constexpr (std::is_same<R, double>::value) {
     // every term below FP64 rounding (see LhyCoef::nskip).  FP64 only: the FP32
     // transforms leave a round-off floor of ~1e-7 in amplitude everywhere, so
@@ -182,18 +185,7 @@ __device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, in
     bool any = false;
 #pragma unroll
     for (int j = 0; j < NP; ++j) any |= n1[j] + n2[j] > c.nskip;
-    if (!any) {
-#pragma unroll
-      for (int j = 0; j < NP; ++j) mu1[j] = mu2[j] = R(0);
-      return;
-    }
-  }
-  LhyPt<R> p[NP];
-  R S0[NP], S1[NP], T0[NP], T1[NP], T2[NP];
-#pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    p[j] = lhy_pt(c, n1[j], n2[j]);
-    S0[j] = S1[j] = T0[j] = T1[j] = T2[j] = R(0);
+    if (!any) return;
   }
   // nodes [0, Qm): det eta > 0, both branches; [Qm, Q): det eta <= 0, where
   // V+ V- = 4 n1 n2 det(eta) <= 0 makes max(V-, 0) = 0 at every point.  With
@@ -286,6 +278,18 @@ __device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, in
 #pragma unroll 2
     for (int k = Qm; k < Q; ++k) node(nd[k], std::false_type{});
   }
+}
+
+// mu_i = dF/dn_i = sum_q W_q (5/2) sum_+- max(V,0)^{3/2} (eta_ii +- sigma_i/s),
+// sigma_1 = eta11 delta + 2 eta12^2 n2, sigma_2 = -eta22 delta + 2 eta12^2 n1
+// (the paper's mu_LHY, Sec. II); sigma_i(w) is quadratic in w:
+//   mu_i = 5/2 (g_ii S_0 + gdd_ii S_1 + sigma_i0 T_0 + sigma_i1 T_1 + sigma_i2 T_2).
+template <class R, int NP>
+__device__ __forceinline__ void lhy_points(const LhyNode<R>* __restrict__ nd, int Q, int Qm, const LhyCoef<R>& c,
+                                           const R (&n1)[NP], const R (&n2)[NP], R (&mu1)[NP], R (&mu2)[NP]) {
+  LhyPt<R> p[NP];
+  R S0[NP], S1[NP], T0[NP], T1[NP], T2[NP];
+  lhy_moments<R, NP>(nd, Q, Qm, c, n1, n2, p, S0, S1, T0, T1, T2);
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
     // sigma_1(w) = (g11 + d11 w)(D0 + D1 w) + 2 n2 (g12 + d12 w)^2, sigma_2 likewise
@@ -433,43 +437,30 @@ __device__ __forceinline__ void lhy_hess(const LhyNode<R>* __restrict__ nd, int 
   for (int j = 0; j < NP; ++j) H[j] = R(2.5) * h[j];
 }
 
-// F and its partial derivatives with respect to the entries of
-// eta(u) = g + gdd (3u^2 - 1), summed over the u-rule (one point; the
-// parameter-derivative pass):  o[0] = F,  o[1..3] = dF/d(g11, g22, g12),
-// o[4..6] = dF/d(gdd11, gdd22, gdd12).  With V_+- = A +- s and f_+- =
-// (5/2) max(V_+-,0)^{3/2}:  dV_+-/deta11 = n1 +- delta n1/s,
+// Partial derivatives of F with respect to the entries of eta(u) = g + gdd w,
+// w = 3u^2 - 1, summed over the u-rule at NP points (the parameter-derivative
+// pass):  o[0..2] = dF/d(g11, g22, g12),  o[3..5] = dF/d(gdd11, gdd22, gdd12).
+// With f_+- = (5/2) max(V_+-,0)^{3/2}:  dV_+-/deta11 = n1 +- delta n1/s,
 // dV_+-/deta22 = n2 -+ delta n2/s, dV_+-/deta12 = +-4 eta12 n1 n2/s (g12 = g21
-// moved together); terms / s are 0 where s = 0.
-template <class R>
-__device__ __forceinline__ void lhy_eta_sums(const LhyNode<R>* __restrict__ nd, int Q, const LhyCoef<R>& c, R n1,
-                                             R n2, R (&o)[7]) {
+// moved together), so with delta = D0 + D1 w and eta12 = g12 + gdd12 w they are
+// combinations of the node sums of lhy_moments.  (A loop of its own with both square
+// roots, V^{5/2} and six accumulators took 590 us for 256 x 256 x 128 points in FP32.)
+template <class R, int NP>
+__device__ __forceinline__ void lhy_eta_sums(const LhyNode<R>* __restrict__ nd, int Q, int Qm, const LhyCoef<R>& c,
+                                             const R (&n1)[NP], const R (&n2)[NP], R (&o)[NP][6]) {
+  LhyPt<R> p[NP];
+  R S0[NP], S1[NP], T0[NP], T1[NP], T2[NP];
+  lhy_moments<R, NP>(nd, Q, Qm, c, n1, n2, p, S0, S1, T0, T1, T2);
 #pragma unroll
-  for (int k = 0; k < 7; ++k) o[k] = R(0);
-  if constexpr (std::is_same<R, double>::value)
-    if (!(n1 + n2 > c.nskip)) return;
-  const LhyPt<R> p = lhy_pt(c, n1, n2);
-  for (int q = 0; q < Q; ++q) {
-    const LhyNode<R>& e = nd[q];
-    const R A = p.A0 + p.A1 * e.w;
-    const R d = p.D0 + p.D1 * e.w;
-    const R s2 = d * d + e.e12sq * p.q4;
-    R rs, s;
-    inv_s(s2, rs, s);
-    const R e12 = c.g12 + c.d12 * e.w;
-    const R vp = fmax(A + s, R(0)), vm = fmax(A - s, R(0));
-    const R rp = sqrt_pos(vp), rm = sqrt_pos(vm);
-    const R fp = R(2.5) * vp * rp, fm = R(2.5) * vm * rm;
-    o[0] += e.W * (vp * vp * rp + vm * vm * rm);
-    const R sum = fp + fm, dif = fp - fm;
-    const R t11 = sum * n1 + dif * d * n1 * rs;
-    const R t22 = sum * n2 - dif * d * n2 * rs;
-    const R t12 = dif * R(4) * e12 * n1 * n2 * rs;
-    o[1] += e.W * t11;
-    o[2] += e.W * t22;
-    o[3] += e.W * t12;
-    o[4] += e.Ww * t11;
-    o[5] += e.Ww * t22;
-    o[6] += e.Ww * t12;
+  for (int j = 0; j < NP; ++j) {
+    const R dt0 = fma_(p[j].D1, T1[j], p[j].D0 * T0[j]), dt1 = fma_(p[j].D1, T2[j], p[j].D0 * T1[j]);
+    const R a1 = R(2.5) * n1[j], a2 = R(2.5) * n2[j], a12 = R(4) * a1 * n2[j];
+    o[j][0] = a1 * (S0[j] + dt0);
+    o[j][1] = a2 * (S0[j] - dt0);
+    o[j][2] = a12 * fma_(c.d12, T1[j], c.g12 * T0[j]);
+    o[j][3] = a1 * (S1[j] + dt1);
+    o[j][4] = a2 * (S1[j] - dt1);
+    o[j][5] = a12 * fma_(c.d12, T2[j], c.g12 * T1[j]);
   }
 }
 
@@ -523,13 +514,6 @@ __device__ __forceinline__ double horner_tab(const double* rec, int f, FixedX x)
 #pragma unroll
   for (int i = 0; i < 6; ++i) k[i] = __ldg(v + i);
   const int E = __ldg(reinterpret_cast<const int*>(rec + 60) + f);
-__device__ __forceinline__ float horner_tab(const float* rec, int f, float x) { return horner_tab(rec + f * 8, x); }
-template <class R> struct TabX {
-  using T = R;
-};
-template <> struct TabX<double> {
-  using T = FixedX;
-};
   long long p = k[5].y;
   p = k[5].x + mulq(p, x.h, x.l);
 #pragma unroll
@@ -539,6 +523,13 @@ template <> struct TabX<double> {
   }
   return from_fixed(p, LineScale{1024 + E, -1, 0});
 }
+__device__ __forceinline__ float horner_tab(const float* rec, int f, float x) { return horner_tab(rec + f * 8, x); }
+template <class R> struct TabX {
+  using T = R;
+};
+template <> struct TabX<double> {
+  using T = FixedX;
+};
 
 // Interval record of (n1, n2) and its local coordinate x; rs = 1/sqrt(n) (1
 // where n = 0, whose terms vanish with their n-power prefactor).
@@ -550,6 +541,15 @@ __device__ __forceinline__ const R* lhy_tab_locate(const LhyTab<R>& t, R n1, R n
     // interval index by adding 1.5 2^52 (round to nearest of the coordinate less
     // 1/2), which leaves it in the low word: no conversions on the FP64 pipe
     rs = rsqrt_(n > 1e-300 ? n : 1.0);
+    const double tt = fma(sqrt_pos(h ? n2 : n1) * rs, t.tscale, -0.5);
+    const double g = tt + 6755399441055744.0;
+    double d = tt - (g - 6755399441055744.0);  // x/2
+    int i = __double2loint(g);
+    if (i > t.ni - 1) {  // a = 1/sqrt(2) up to rounding
+      d += (double)(i - (t.ni - 1));
+      i = t.ni - 1;
+    }
+    i = i < 0 ? 0 : i;
     const LimbQ xl = limbs(to_fixed(d, LineScale{1022, -1, 0}));  // 2 d in 62 fractional bits
     x.h = xl.h;
     x.l = xl.l;
@@ -561,15 +561,6 @@ __device__ __forceinline__ const R* lhy_tab_locate(const LhyTab<R>& t, R n1, R n
     int i = (int)tt;  // a <= 1/sqrt(2) up to rounding: clamp to the last interval (NaN converts to 0)
     i = i < 0 ? 0 : (i < t.ni - 1 ? i : t.ni - 1);
     x = R(2) * (tt - (R)i) - R(1);
-    const double tt = fma(sqrt_pos(h ? n2 : n1) * rs, t.tscale, -0.5);
-    const double g = tt + 6755399441055744.0;
-    double d = tt - (g - 6755399441055744.0);  // x/2
-    int i = __double2loint(g);
-    if (i > t.ni - 1) {  // a = 1/sqrt(2) up to rounding
-      d += (double)(i - (t.ni - 1));
-      i = t.ni - 1;
-    }
-    i = i < 0 ? 0 : i;
     return t.tab + (size_t)((h ? t.ni : 0) + i) * LhyTabDim<R>::rec;
   }
 }
