@@ -16,9 +16,9 @@
 //   output position (j div Ns) Ns r + (j mod Ns) + q Ns
 // Thread t of a line owns butterflies j = t + b L/8 (b < 8/r).
 //
-// Lengths 48, 80 and 96 (a power of two times 3 or 5) use the same register
-// interface with a mixed-radix plan (radix 8, then 3/5 and 2/4 passes in
-// shared memory) and natural entry/exit layouts; see fft_mixed.
+// Lengths 48, 80 and 96 (8 times 6, 10 and 12) use the same register interface
+// with a radix-8 pass, one pass of radix L/8 and natural entry/exit layouts; see
+// fft_mixed.
 #pragma once
 #include <type_traits>
 
@@ -30,16 +30,11 @@ template <int L> struct IsPow2 {
   static constexpr bool v = L > 0 && (L & (L - 1)) == 0;
 };
 
-// Radix sequence of the mixed-radix lengths (a multiple of 8 times 3 or 5):
-// radix 8 first, then the remaining factors.
+// The other lengths are 8 times 6, 10 or 12: a radix-8 pass and one pass of radix
+// L/8, which is as many values as the line has threads.
 template <int L> struct MixedPlan {
   static constexpr int TPL = L / 8;
-  static constexpr int P = (L == 48) ? 3 : (L == 80) ? 3 : (L == 96) ? 3 : -1;
-  static_assert(P > 0, "unsupported FFT length");
-  __host__ __device__ static constexpr int rad(int p) {
-    return p == 0 ? 8 : (L == 48 ? (p == 1 ? 3 : 2) : L == 80 ? (p == 1 ? 5 : 2) : (p == 1 ? 4 : 3));
-  }
-  __host__ __device__ static constexpr int ns(int p) { return p == 0 ? 1 : ns(p - 1) * rad(p - 1); }
+  static_assert(TPL == 6 || TPL == 10 || TPL == 12, "unsupported FFT length");
   // natural layout on entry and exit, in both directions
   __device__ static __forceinline__ int entry_pos(bool, int t, int e) { return t + e * TPL; }
   __device__ static __forceinline__ int exit_pos(bool, int t, int e) { return t + e * TPL; }
@@ -465,58 +460,39 @@ __device__ __forceinline__ void fft_passes(C (&v)[NF][8], C* sm, int fstride, co
   }
 }
 
-// Mixed-radix passes p >= 1 through shared memory: the L/r butterflies of a
-// pass are spread over the line's L/8 threads (some threads idle when they do
-// not divide evenly); each thread reads all inputs of its butterflies before
-// the block synchronises and the outputs overwrite them in place.
-template <class C, int L, bool INV, int NF, int p, class SI, class TW>
-__device__ __forceinline__ void fft_mixed_passes(C* sm, int fstride, const TW* __restrict__ tw, int t, const SI& si) {
-  using PL = MixedPlan<L>;
-  constexpr int r = PL::rad(p);
-  constexpr int Ns = PL::ns(p);
-  constexpr int NBF = L / r;                       // butterflies in this pass
-  constexpr int NB = (NBF + PL::TPL - 1) / PL::TPL;  // per thread (upper bound)
-  constexpr int STW = L / (Ns * r);
+// DFT of 6 = 2 x 3, 10 = 2 x 5 or 12 = 4 x 3 points by the prime-factor algorithm
+// (Good, Thomas): with n = NB na + NA nb and k = ka mod NA, kb mod NB the transform
+// is NB DFTs of NA points and NA DFTs of NB points without twiddles.
+template <int N, bool INV, class C> __device__ __forceinline__ void dft_pfa(C (&x)[N]) {
+  constexpr int NA = N == 12 ? 4 : 2, NB = N / NA;
+  C u[NA][NB];
 #pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    C w[NB][r];
+  for (int b = 0; b < NB; ++b) {
+    C a[NA];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int j = t + b * PL::TPL;
-      if (j < NBF) {
+    for (int q = 0; q < NA; ++q) a[q] = x[(NB * q + NA * b) % N];
+    dft_r<NA, INV>(a);
 #pragma unroll
-        for (int q = 0; q < r; ++q) w[b][q] = sm[f * fstride + si(j + q * NBF)];
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int j = t + b * PL::TPL;
-      if (j < NBF) {
-        const int k = j % Ns;
-#pragma unroll
-        for (int q = 1; q < r; ++q) {
-          const TW tq = tw[q * k * STW];
-          w[b][q] = INV ? cmulc(w[b][q], tq) : cmul(w[b][q], tq);
-        }
-        dft_r<r, INV>(w[b]);
-        const int base = (j / Ns) * Ns * r + k;
-#pragma unroll
-        for (int q = 0; q < r; ++q) sm[f * fstride + si(base + q * Ns)] = w[b][q];
-      }
-    }
-    __syncthreads();
+    for (int q = 0; q < NA; ++q) u[q][b] = a[q];
   }
-  if constexpr (p + 1 < PL::P) fft_mixed_passes<C, L, INV, NF, p + 1, SI, TW>(sm, fstride, tw, t, si);
+#pragma unroll
+  for (int q = 0; q < NA; ++q) dft_r<NB, INV>(u[q]);
+#pragma unroll
+  for (int k = 0; k < N; ++k) x[k] = u[k % NA][k % NB];
 }
 
-// Mixed-radix line transform with natural entry and exit layouts (register e
-// of thread t holds position t + e L/8): the radix-8 first pass runs on the
-// registers as loaded, the later passes in shared memory, and the result is
-// read back in the same layout.
+// Mixed-radix line transform with natural entry and exit layouts (register e of
+// thread t holds position t + e L/8).  Input n = t + (L/8) e and output
+// k = k1 + 8 k2: thread t's radix-8 DFT over e, the twiddle W_L^{t k1}, and for each
+// k1 a DFT over t, taken in place at slots 8 t + k1, which become the outputs
+// 8 k2 + k1 in natural order.  Two trips through shared memory and three barriers;
+// plans of radix 8 and two more passes took three trips and six (FP32, 96^3: see
+// kernels.cuh for the passes).  The eight DFTs go to the line's first eight threads
+// (a second round for six); column lines keep whole warps busy or idle.
 template <class C, int L, bool INV, int NF, class SI, class TW>
 __device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, const TW* __restrict__ tw, int t,
                                           const SI& si) {
+  constexpr int N2 = MixedPlan<L>::TPL;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     dft8<INV>(v[f]);
@@ -524,11 +500,31 @@ __device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, con
     for (int q = 0; q < 8; ++q) sm[f * fstride + si(8 * t + q)] = v[f][q];
   }
   __syncthreads();
-  fft_mixed_passes<C, L, INV, NF, 1, SI, TW>(sm, fstride, tw, t, si);
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+#pragma unroll
+    for (int r = 0; r < (8 + N2 - 1) / N2; ++r) {
+      const int k1 = t + r * N2;
+      if (k1 < 8) {
+        C w[N2];
+#pragma unroll
+        for (int n = 0; n < N2; ++n) w[n] = sm[f * fstride + si(8 * n + k1)];
+#pragma unroll
+        for (int n = 1; n < N2; ++n) {
+          const TW q = tw[n * k1];
+          w[n] = INV ? cmulc(w[n], q) : cmul(w[n], q);
+        }
+        dft_pfa<N2, INV>(w);
+#pragma unroll
+        for (int n = 0; n < N2; ++n) sm[f * fstride + si(8 * n + k1)] = w[n];
+      }
+    }
+  }
+  __syncthreads();
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[f][e] = sm[f * fstride + si(t + e * MixedPlan<L>::TPL)];
+    for (int e = 0; e < 8; ++e) v[f][e] = sm[f * fstride + si(t + e * N2)];
   __syncthreads();  // callers may reuse the buffer
 }
 
