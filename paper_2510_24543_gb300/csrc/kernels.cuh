@@ -43,7 +43,8 @@ template <class R> struct KArgs {
   const C* twz;
   C* psi[2];                 // psi buffers (2 fields each)
   C* hp[2];                  // H psi buffers
-  C* ax[2];                  // aux: field 0 = (Phi1, Phi2), field 1 = (muL1, muL2)
+  C* ax[2];                  // aux: field 0 = (Phi1, Phi2), field 1 = (B1, B2), B_i = V + sum_j g_ij n_j + mu_LHY,i:
+                             // P_V, the line search and the ITE step need mu_LHY only in this sum
   C* rb[2];                  // residual buffers (current / previous by parity of n)
   C* pb[2];                  // direction buffers (current / previous)
   C* z;                      // preconditioned residual
@@ -406,6 +407,12 @@ template <class Op> struct ColDefaultM {
   static constexpr int M0 = IsPow2<Op::L>::v ? (MB < 512 / TPL ? MB : 512 / TPL) : MB;
   static constexpr int v = M0 > whole_warp_rows(Op::L) ? M0 : whole_warp_rows(Op::L);
 };
+// FP64: threads per SM the passes ask for (registers 65536 / this).  The fixed-point
+// lines wait on integer chains, which more warps hide.
+#ifndef EGPE_COL64
+#define EGPE_COL64 512
+#endif
+constexpr int COL64 = EGPE_COL64;
 // Launch bounds of a column kernel: the run-time width keeps ColMaxThreads; a
 // compile-time width MC has exactly MC L/8 threads, and the FP32 plain y/z
 // passes (the ColPlain op, small epilogue) of up to 256 threads ask for three
@@ -414,7 +421,8 @@ template <class Op> struct ColDefaultM {
 // pass takes 24 us with three blocks of 192 and 33 us with two.
 template <class Op> struct ColMinB {
   static constexpr int threads = ColDefaultM<Op>::v * (Op::L / 8);
-  static constexpr int v = sizeof(typename Op::R) == 4 && !IsPow2<Op::L>::v ? 576 / threads : 1;
+  static constexpr int want = sizeof(typename Op::R) == 8 ? COL64 : !IsPow2<Op::L>::v ? 576 : 0;
+  static constexpr int v = want > threads ? want / threads : 1;
 };
 template <class Op, int MC> struct ColBounds {
   static constexpr int threads = MC > 0 ? MC * (Op::L / 8) : ColMaxThreads<Op>::v;
@@ -929,12 +937,12 @@ template <class R_, int L_> struct XInvEG {
       const C T1 = pt[j].out(0), T2 = pt[j].out(1), PH = pt[j].out(2);
       const R phi1 = PH.x, phi2 = PH.y;
       const R c1 = fma_(a.g12, n2[j], a.g11 * n1[j]), c2 = fma_(a.g22, n2[j], a.g21 * n1[j]);
-      const R U1 = (V + c1) + (phi1 + m1[j]);
-      const R U2 = (V + c2) + (phi2 + m2[j]);
+      const R B1 = (V + c1) + m1[j], B2 = (V + c2) + m2[j];
+      const R U1 = B1 + phi1, U2 = B2 + phi2;
       hp[idx] = cmk<C>(fma_(U1, p1[j].x, T1.x), fma_(U1, p1[j].y, T1.y));
       hp[N + idx] = cmk<C>(fma_(U2, p2[j].x, T2.x), fma_(U2, p2[j].y, T2.y));
       ax[idx] = PH;
-      ax[N + idx] = cmk<C>(m1[j], m2[j]);
+      ax[N + idx] = cmk<C>(B1, B2);
       // the energies and mu_i are combinations of these (finalize_energy)
       s[EG_TRAP1] = fma_(V, n1[j], s[EG_TRAP1]);
       s[EG_TRAP2] = fma_(V, n2[j], s[EG_TRAP2]);
@@ -986,41 +994,31 @@ template <class R> __device__ __forceinline__ void pc_uniform(const KArgs<R>& a,
   }
 }
 
-// P_V,i of component i at a point (Sec. IV.B), with the floor.
-template <class R>
-__device__ __forceinline__ R pv_at(const KArgs<R>& a, const PcUni<R>& u, int i, R V, R n1, R n2, R ml) {
-  const R P = fma_(i ? a.g22 : a.g12, n2, fma_(i ? a.g21 : a.g11, n1, (pick(u.shift, i) + V) + ml));
-  const R fl = pick(u.floor_, i);
+// P_V,i of component i at a point (Sec. IV.B) from B_i, with the floor.
+template <class R> __device__ __forceinline__ R pv_at(const PcUni<R>& u, int i, R B) {
+  const R P = pick(u.shift, i) + B, fl = pick(u.floor_, i);
   return P > fl ? P : fl;
 }
 // r_i = H_i psi_i - mu_i psi_i (stored unless given) and w_i = P_V^{-1} r_i when
 // diag, at CH points: both components (NV = 2, i = 0) or component i alone.
 template <class R, int CH, int NV>
 __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u, int i, const size_t (&idx)[CH],
-                                            const R (&V)[CH], C2<R> (&w)[NV][CH]) {
+                                            C2<R> (&w)[NV][CH]) {
   using C = C2<R>;
   const size_t N = a.N;
-  C h[NV][CH], p[2][CH], ml[CH];  // NV = 1: p[0] is component i, p[1] the other
+  C h[NV][CH], p[NV][CH], bb[CH];
 #pragma unroll
   for (int j = 0; j < CH; ++j) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       const size_t q = (size_t)(i + k) * N + idx[j];
       h[k][j] = u.rgiven ? pick(a.rb, u.nsel)[q] : pick(a.hp, u.cur)[q];
-      if (a.diag || !u.rgiven) p[k][j] = pick(a.psi, u.cur)[q];
+      if (!u.rgiven) p[k][j] = pick(a.psi, u.cur)[q];
     }
-    if (a.diag) {
-      if constexpr (NV == 1) p[1][j] = pick(a.psi, u.cur)[(i ? 0 : N) + idx[j]];
-      ml[j] = pick(a.ax, u.cur)[N + idx[j]];
-    }
+    if (a.diag) bb[j] = pick(a.ax, u.cur)[N + idx[j]];
   }
 #pragma unroll
   for (int j = 0; j < CH; ++j) {
-    R nn[2];
-    if (a.diag) {
-      nn[0] = cabs2(p[0][j]);
-      nn[1] = cabs2(p[1][j]);
-    }
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       const int c = i + k;
@@ -1030,10 +1028,7 @@ __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u
         r = cmk<C>(fma_(-mu, p[k][j].x, r.x), fma_(-mu, p[k][j].y, r.y));
         pick(a.rb, u.nsel)[(size_t)c * N + idx[j]] = r;
       }
-      if (a.diag) {
-        const R n1 = NV == 1 && i ? nn[1] : nn[0], n2 = NV == 1 && i ? nn[0] : nn[1];
-        r = cscale(r, rcp_(pv_at(a, u, c, V[j], n1, n2, c ? ml[j].y : ml[j].x)));
-      }
+      if (a.diag) r = cscale(r, rcp_(pv_at(u, c, c ? bb[j].y : bb[j].x)));
       w[k][j] = r;
     }
   }
@@ -1094,20 +1089,14 @@ template <class R_, int L_> struct XFwdPC {
         for (int k = 0; k < NV; ++k) v[k][e] = cmk<C>(0, 0);
       return;
     }
-    const R vyz = trap_yz(a, row);
     constexpr int CH = ChunkW<R>::v;
 #pragma unroll
     for (int e0 = 0; e0 < 8; e0 += CH) {
       size_t idx[CH];
-      R V[CH];
       C w[NV][CH];
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const int x = Plan<L>::entry_pos(false, t, e0 + j);
-        idx[j] = (size_t)row * a.nx + x;
-        V[j] = trap_x(a, x) + vyz;
-      }
-      pc_residual<R, CH, NV>(a, u, f, idx, V, w);
+      for (int j = 0; j < CH; ++j) idx[j] = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
+      pc_residual<R, CH, NV>(a, u, f, idx, w);
 #pragma unroll
       for (int j = 0; j < CH; ++j)
 #pragma unroll
@@ -1183,11 +1172,8 @@ template <class R_, int L_> struct XInvPC {
       const size_t idx = pt[j].idx;
       C z1 = pt[j].out(0), z2 = pt[j].out(1);
       if (a.blend) {  // z = (1 - w) P_Delta^{-1} r + w P_V^{-1} r
-        const C ml = pick(a.ax, u.cur)[(size_t)a.N + idx];
-        const R V = trap_x(a, pt[j].x) + pt[j].vyz;
-        const R n1 = cabs2(in[j].p1), n2 = cabs2(in[j].p2);
-        const R wd = R(1) - u.wv;
-        const R w1 = u.wv * rcp_(pv_at(a, u, 0, V, n1, n2, ml.x)), w2 = u.wv * rcp_(pv_at(a, u, 1, V, n1, n2, ml.y));
+        const C bb = pick(a.ax, u.cur)[(size_t)a.N + idx];
+        const R wd = R(1) - u.wv, w1 = u.wv * rcp_(pv_at(u, 0, bb.x)), w2 = u.wv * rcp_(pv_at(u, 1, bb.y));
         z1 = cmk<C>(wd * z1.x + w1 * in[j].r1.x, wd * z1.y + w1 * in[j].r1.y);
         z2 = cmk<C>(wd * z2.x + w2 * in[j].r2.x, wd * z2.y + w2 * in[j].r2.y);
       }
@@ -1215,16 +1201,10 @@ __device__ __forceinline__ void pc_point_body(const KArgs<R>& a) {
   pc_uniform(a, u);
   PAcc<R> acc[PC_NS];
   const size_t N = a.N;
-  const size_t nxy = (size_t)a.nx * a.ny;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(idx % a.nx);
-    const int y = (int)((idx / a.nx) % a.ny);
-    const int z = (int)(idx / nxy);
-    const R V = trap_x(a, x) + (a.vt[a.nx + y] + a.vt[a.nx + a.ny + z]);
     C w[2][1];
     const size_t id[1] = {idx};
-    const R Vp[1] = {V};
-    pc_residual<R, 1, 2>(a, u, 0, id, Vp, w);
+    pc_residual<R, 1, 2>(a, u, 0, id, w);
     const C w1 = w[0][0], w2 = w[1][0];
     a.z[idx] = w1;
     a.z[N + idx] = w2;
@@ -1445,7 +1425,7 @@ template <class R_, int L_> struct XInvLC {
     const C* hp = pick(a.hp, u.cur);
     const C* ax = pick(a.ax, u.cur);
     R n1[NP], n2[NP], n1p[NP], n2p[NP], Hh[NP];
-    C p1[NP], p2[NP], q1[NP], q2[NP], h1[NP], h2[NP], phi[NP], ml[NP];
+    C p1[NP], p2[NP], q1[NP], q2[NP], h1[NP], h2[NP], phi[NP], bb[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
       const size_t idx = pt[j].idx;
@@ -1456,7 +1436,7 @@ template <class R_, int L_> struct XInvLC {
       h1[j] = hp[idx];
       h2[j] = hp[N + idx];
       phi[j] = ax[idx];
-      ml[j] = ax[N + idx];
+      bb[j] = ax[N + idx];
     }
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
@@ -1467,9 +1447,7 @@ template <class R_, int L_> struct XInvLC {
       n1p[j] = rho1 + rho1;
       n2p[j] = rho2 + rho2;
       const C PR = pt[j].out(0);
-      const R V = trap_x(a, pt[j].x) + pt[j].vyz;
-      const R U1 = fma_(a.g12, n2[j], fma_(a.g11, n1[j], (V + phi[j].x) + ml[j].x));
-      const R U2 = fma_(a.g22, n2[j], fma_(a.g21, n1[j], (V + phi[j].y) + ml[j].y));
+      const R U1 = phi[j].x + bb[j].x, U2 = phi[j].y + bb[j].y;
       s[LC_P1] += a1;
       s[LC_P2] += a2;
       s[LC_PSIP1] += rho1;
@@ -1526,23 +1504,13 @@ template <class R_, int L_> struct XFwdKin {
     load_rows<XFwdKin>(a, ps, f, row, valid, t, v);
     if (!a.flag || !valid) return;
     const C* ax = pick(a.ax, u.cur);
-    const R vyz = trap_yz(a, row);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int x = Plan<L>::entry_pos(false, t, e);
-      const size_t idx = (size_t)row * a.nx + x;
-      const R V = trap_x(a, x) + vyz;
-      const C phi = ax[idx], ml = ax[N + idx];
-      R n[2];  // NV = 1: component f, then the other
-      n[0] = cabs2(v[0][e]);
-      n[1] = cabs2(NV == 1 ? ps[(f ? 0 : N) + idx] : v[NV - 1][e]);
+      const size_t idx = (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e);
+      const C phi = ax[idx], bb = ax[N + idx];
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        const int c = f + k;
-        const R n1 = NV == 1 && f ? n[1] : n[0], n2 = NV == 1 && f ? n[0] : n[1];
-        const R U = fma_(c ? a.g22 : a.g12, n2, fma_(c ? a.g21 : a.g11, n1, V + ((c ? phi.y : phi.x) + (c ? ml.y : ml.x))));
-        v[k][e] = cscale(v[k][e], exp(-u.dtau * U));
-      }
+      for (int k = 0; k < NV; ++k)
+        v[k][e] = cscale(v[k][e], exp(-u.dtau * (f + k ? phi.y + bb.y : phi.x + bb.x)));
     }
   }
   template <int NV>
