@@ -199,7 +199,8 @@ typedef struct egpe_handle egpe_handle;
  * precision on the current CUDA device.  cuda_stream is a cudaStream_t, or
  * NULL for a stream owned by the handle and ordered against the legacy default
  * stream at every call (see Streams above).  Allocates every workspace up front (about 26
- * complex fields per instance and precision).  Errors: INVALID_ARG (bad sizes,
+ * complex fields per instance and precision); the first solve with a kinetic
+ * preconditioner adds 10 more to an FP64 engine where they fit.  Errors: INVALID_ARG (bad sizes,
  * non-symmetric couplings, L <= 0, Q out of range), OOM, CUDA. */
 egpe_status egpe_create(const egpe_grid* grids, const egpe_params* params, int n_inst,
                         egpe_precision prec, void* cuda_stream, egpe_handle** out);
@@ -282,7 +283,9 @@ egpe_status egpe_retract(egpe_handle* h, int inst, const void* psi, const void* 
 /* Unnormalised 3D DFT (inverse: sign +, no 1/N) of nfields consecutive complex
  * fields of the instance's grid with the library's own Stockham kernels.
  * in and out may alias.  Device pointers.  A diagnostic of the transform that
- * every other entry point uses. */
+ * every other entry point uses.  FP64 lines are transformed in 64-bit fixed point
+ * under a scale of their own: a line with a value of 2^1013 or more (or not
+ * finite) gives NaN, a line with none above 2^-960 gives 0. */
 egpe_status egpe_fft(egpe_handle* h, int inst, const void* in, void* out, int nfields, int inverse);
 
 /* Diagnostic: device time of every kernel of one solver attempt

@@ -41,6 +41,8 @@ template <class R> class BatchRunner {
     const int n = (int)eng_.size();
     runs.assign(n, SolveRun{});
     EGPE_TRY(alloc());
+    carried_ = true;
+    for (Engine<R>* e : eng_) carried_ = e->ensure_carry(o.precond) && carried_;
     egpe_solve_opts oo = o;
     oo.use_graph = 0;
     for (int i = 0; i < n; ++i)
@@ -51,17 +53,23 @@ template <class R> class BatchRunner {
     std::vector<int> active = live(phase);
     const int mode = o.precond;
     const int poll = std::max(1, o.poll_every);
-    const long long max_launch = (long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4;
+    const long long max_launch =
+        ((long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4) * (carried_ ? kRefreshEvery : 1);
     long long replays = 0, kernels = 0;
+    bool want_refresh = false;
     while (!active.empty() && replays < max_launch) {
       if (active != built_) EGPE_TRY(rebuild(active, mode));
       for (int k = attempts_ahead(poll, max_iter, replays); k > 0; --k) {
-        EGPE_CUDA(cudaGraphLaunch(graph_, stream_));
+        const bool refresh = attempt_kind(carried_, replays, want_refresh) == ATT_REFRESH;
+        want_refresh = false;
+        if (refresh && !refresh_) EGPE_TRY(build(active, mode, ATT_REFRESH, refresh_, per_refresh_));
+        EGPE_CUDA(cudaGraphLaunch(refresh ? refresh_ : graph_, stream_));
         ++replays;
-        kernels += per_replay_;
+        kernels += refresh ? per_refresh_ : per_replay_;
       }
       EGPE_TRY(gather(phase));
       active = live(phase);
+      for (int ph : phase) want_refresh |= ph == PH_DIRECT;
     }
     for (int i = 0; i < n; ++i) {
       Engine<R>& e = *eng_[i];
@@ -78,11 +86,12 @@ template <class R> class BatchRunner {
   std::vector<Engine<R>*> eng_;
   cudaStream_t stream_ = nullptr;
   bool concurrent_ = false;
+  bool carried_ = false;  // every instance has room for T psi and T p
   std::vector<cudaStream_t> branch_;  // forked capture streams, one per group (concurrent mode)
   std::vector<cudaEvent_t> join_;     // [0]: fork point, [1 + g]: end of group g's chain
-  cudaGraphExec_t graph_ = nullptr;
+  cudaGraphExec_t graph_ = nullptr, refresh_ = nullptr;
   std::vector<int> built_;
-  long long per_replay_ = 0;
+  long long per_replay_ = 0, per_refresh_ = 0;
   int builds_ = 0;
   DevState** d_sts_ = nullptr;
   int* d_phase_ = nullptr;
@@ -90,7 +99,8 @@ template <class R> class BatchRunner {
 
   void release() {
     if (graph_) cudaGraphExecDestroy(graph_);
-    graph_ = nullptr;
+    if (refresh_) cudaGraphExecDestroy(refresh_);
+    graph_ = refresh_ = nullptr;
     for (cudaStream_t b : branch_) cudaStreamDestroy(b);
     for (cudaEvent_t e : join_) cudaEventDestroy(e);
     branch_.clear();
@@ -136,6 +146,16 @@ template <class R> class BatchRunner {
   // records each one's attempt and captures one graph that launches every
   // pass once per chunk.
   egpe_status rebuild(const std::vector<int>& active, int mode) {
+    if (refresh_) cudaGraphExecDestroy(refresh_);  // built again when it is next due
+    refresh_ = nullptr;
+    EGPE_TRY(build(active, mode, attempt_kind(carried_, 0, false), graph_, per_replay_));
+    built_ = active;
+    ++builds_;
+    return EGPE_OK;
+  }
+
+  egpe_status build(const std::vector<int>& active, int mode, AttemptKind kind, cudaGraphExec_t& graph,
+                    long long& per_replay) {
     std::map<std::tuple<int, int, int>, std::vector<int>> groups;
     for (int i : active) groups[std::make_tuple(eng_[i]->nx, eng_[i]->ny, eng_[i]->nz)].push_back(i);
     struct Launch {
@@ -158,7 +178,7 @@ template <class R> class BatchRunner {
         const int nc = (int)std::min<size_t>(KB_MAX, ids.size() - c0);
         recs.assign(nc, {});
         args.assign(nc, {});
-        for (int c = 0; c < nc; ++c) EGPE_TRY(eng_[ids[c0 + c]]->record_attempt(mode, recs[c], args[c]));
+        for (int c = 0; c < nc; ++c) EGPE_TRY(eng_[ids[c0 + c]]->record_attempt(mode, kind, recs[c], args[c]));
         for (int c = 1; c < nc; ++c)
           if (recs[c].size() != recs[0].size()) {
             set_error_msg("batched solve: instances recorded different launch sequences");
@@ -212,8 +232,8 @@ template <class R> class BatchRunner {
         join_.push_back(e);
       }
     }
-    if (graph_) cudaGraphExecDestroy(graph_);
-    graph_ = nullptr;
+    if (graph) cudaGraphExecDestroy(graph);
+    graph = nullptr;
     cudaGraph_t g = nullptr;
     EGPE_CUDA(cudaStreamBeginCapture(stream_, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
@@ -240,16 +260,14 @@ template <class R> class BatchRunner {
       set_error(le != cudaSuccess ? "batched launch" : "cudaStreamEndCapture", le != cudaSuccess ? le : ce);
       return EGPE_ERR_CUDA;
     }
-    cudaError_t ie = cudaGraphInstantiate(&graph_, g, 0);
+    cudaError_t ie = cudaGraphInstantiate(&graph, g, 0);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) {
-      graph_ = nullptr;
+      graph = nullptr;
       set_error("cudaGraphInstantiate", ie);
       return EGPE_ERR_CUDA;
     }
-    per_replay_ = (long long)launches.size();
-    built_ = active;
-    ++builds_;
+    per_replay = (long long)launches.size();
     return EGPE_OK;
   }
 };

@@ -43,7 +43,9 @@ template <class C> __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x) {
 enum EgSlot {  // pointwise part of one energy/gradient evaluation (x dV later):
   // int of n_i V, n_i sum_j g_ij n_j, n_i Phi_i, n_i mu_LHY,i, n_i
   EG_TRAP1 = 0, EG_TRAP2, EG_CON1, EG_CON2, EG_NPHI1, EG_NPHI2,
-  EG_NMUL1, EG_NMUL2, EG_NORM1, EG_NORM2, EG_NS
+  EG_NMUL1, EG_NMUL2, EG_NORM1, EG_NORM2,
+  EG_KIN1, EG_KIN2,  // <psi_i, T psi_i> where T psi is carried along (else Parseval, EgzSlot)
+  EG_NS
 };
 enum EgzSlot { EGZ_KIN1 = 0, EGZ_KIN2, EGZ_NS };  // Parseval sums of the z pass
 enum PcaSlot { PCA_RR1 = 0, PCA_RR2, PCA_NS };     // residual norms (first pass)
@@ -54,7 +56,7 @@ enum PcSlot {  // preconditioned residual / beta sums
 enum LcSlot {  // line-coefficient sums
   LC_P1 = 0, LC_P2, LC_PSIP1, LC_PSIP2, LC_PH1, LC_PH2, LC_UPP1, LC_UPP2, LC_SRHO, LC_HLHY, LC_NS
 };
-enum LczSlot { LCZ_TPP1 = 0, LCZ_TPP2, LCZ_NS };
+enum LczSlot { LCZ_TPP1 = 0, LCZ_TPP2, LCZ_NS };  // <p_i, T p_i>: Parseval sums, or from T p where it is carried along
 enum RtSlot { RT_P1 = 0, RT_P2, RT_PSIP1, RT_PSIP2, RT_PSI1, RT_PSI2, RT_NS };
 enum PgSlot {  // parameter-derivative sums (x dV later)
   PG_N11 = 0, PG_N12, PG_N22, PG_K11, PG_K12, PG_K22, PG_X2, PG_Y2, PG_Z2,
@@ -67,9 +69,24 @@ static constexpr int MAX_NS = 16;
 static_assert(PG_NS <= MAX_NS, "reduction slots");
 
 // Phases of the on-device solver state machine.
-enum Phase { PH_NEW_ITER = 0, PH_TRIAL = 1, PH_DONE = 2 };
-// Launch gates: which phases a kernel runs in.
-enum Gate { GATE_ALWAYS = 0, GATE_NEW_ITER = 1, GATE_ACTIVE = 2 };
+// PH_DIRECT: the iteration waits for an attempt that transforms its direction
+// (T p cannot be carried along, see AttemptKind).
+enum Phase { PH_NEW_ITER = 0, PH_TRIAL = 1, PH_DONE = 2, PH_DIRECT = 3 };
+// Launch gates: which phases a kernel runs in.  REFRESH_*: the passes of a refresh
+// attempt; CARRIED_TRIAL: trial evaluations that need T p.
+enum Gate {
+  GATE_ALWAYS = 0, GATE_NEW_ITER = 1, GATE_ACTIVE = 2, GATE_REFRESH_PC = 3, GATE_REFRESH_CARRIED = 4,
+  GATE_REFRESH_DIRECT = 5, GATE_CARRIED_TRIAL = 6
+};
+// How an attempt obtains the kinetic terms.  FULL: by transforms of the direction
+// and of the trial state.  CARRIED (kinetic preconditioners): T is linear, and
+// P_Delta z = (alpha + T) z = w gives T z = w - alpha z without a transform, so
+// T p = -T z + beta T p_prev - c T psi and T psi' = a T psi + b T p are carried along
+// beside p and psi: 8 transforms per iteration instead of 14.  REFRESH: as CARRIED,
+// with the trial state transformed, which removes what rounding has accumulated in
+// T psi; it also takes the directions whose T is not known (the residual fallback,
+// and the next conjugate one), by transform.
+enum AttemptKind { ATT_FULL = 0, ATT_CARRIED = 1, ATT_REFRESH = 2 };
 
 struct SolveOptsDev {
   int precond, restart_period, max_iter, armijo_max, trace_cap, fp32_phase, beta_rule, stall_iters;
@@ -95,7 +112,8 @@ struct DevState {
   // flow control
   int phase, status, n, attempts, restarts, armijo_total, armijo_k, kind;
   int cur, fallback, trace_len, restart_flag;
-  int rgiven, pgiven, timeout, pad1;  // timeout: a device wait ran out of its poll budget
+  int direct_lc, tp_bad, timeout, pad1;  // timeout: a device wait ran out of its poll budget;
+                                         // direct_lc: this direction is transformed; tp_bad: its T p is not known
   SolveOptsDev opt;
   // current point (slot cur)
   double E, mu[2], shift[2], nmuL[2], norm2[2];

@@ -104,9 +104,13 @@ __device__ inline bool ctrl_timed_out(DevState* st) {
   return true;
 }
 
-__device__ inline void load_point(DevState* st, int slot) {
+// Kinetic sums of an evaluation: carried along (lin) or by Parseval.
+__device__ inline const double* kin_sums(const DevState* st, int slot, int lin) {
+  return lin ? st->eg[slot] + EG_KIN1 : st->egz[slot];
+}
+__device__ inline void load_point(DevState* st, int slot, int lin) {
   EnergyOut o;
-  finalize_energy(st->eg[slot], st->egz[slot], st->dV, o);
+  finalize_energy(st->eg[slot], kin_sums(st, slot, lin), st->dV, o);
   st->E = o.E;
   for (int i = 0; i < 2; ++i) {
     st->mu[i] = o.mu[i];
@@ -121,17 +125,17 @@ __device__ inline void load_point(DevState* st, int slot) {
 
 // After an energy/gradient evaluation.  mode 0: evaluation of the current
 // point (start of a solve, or a standalone call); mode 1: trial point.
-static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, TraceDev* trace) {
+static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, int lin, TraceDev* trace) {
   if (ctrl_timed_out(st)) return;
   if (mode == 0) {
-    load_point(st, st->cur);
+    load_point(st, st->cur, lin);
     st->phase = finite_(st->E) ? PH_NEW_ITER : PH_DONE;
     if (!finite_(st->E)) st->status = 4;  // EGPE_ERR_NONFINITE
     return;
   }
   const int slot = st->cur ^ 1;
   EnergyOut o;
-  finalize_energy(st->eg[slot], st->egz[slot], st->dV, o);
+  finalize_energy(st->eg[slot], kin_sums(st, slot, lin), st->dV, o);
   st->attempts += 1;
   st->E_trial = o.E;
   const SolveOptsDev& op = st->opt;
@@ -166,7 +170,7 @@ static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, TraceD
     const double Eold = st->E;
     st->rz_prev = st->rz;
     st->cur = slot;
-    load_point(st, slot);
+    load_point(st, slot, lin);
     st->dE_last = st->E - Eold;
     st->alpha_prev = st->alpha;
     st->n += 1;
@@ -194,7 +198,7 @@ static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, TraceD
 static __device__ __noinline__ void ctrl_after_ite(DevState* st) {
   if (ctrl_timed_out(st)) return;
   const double Eold = st->E;
-  load_point(st, st->cur);
+  load_point(st, st->cur, 0);
   st->dE_last = st->E - Eold;
   st->n += 1;
   if (!finite_(st->E)) {
@@ -211,7 +215,7 @@ static __device__ __noinline__ void ctrl_after_ite(DevState* st) {
 
 // After the preconditioned residual and its sums: convergence test, beta,
 // projection coefficients, restart rules.
-static __device__ __noinline__ void ctrl_after_pc(DevState* st) {
+static __device__ __noinline__ void ctrl_after_pc(DevState* st, int kind) {
   if (ctrl_timed_out(st)) return;
   const double* pc = st->pc;
   const double dV = st->dV;
@@ -267,12 +271,21 @@ static __device__ __noinline__ void ctrl_after_pc(DevState* st) {
       descent += -pc[PC_ZR1 + i] - c[i] * pc[PC_PSIR1 + i];
     }
   }
-  st->fallback = 0;
-  if (descent >= 0.0) {
+  const int fallback = descent >= 0.0 ? 1 : 0;
+  if (fallback) {
     // p = -(r - Re<r,psi> psi): c_i = Re<-r_i, psi_i>
-    st->fallback = 1;
     for (int i = 0; i < 2; ++i) c[i] = -pc[PC_PSIR1 + i];
   }
+  if (kind != ATT_FULL) {
+    const int direct = (fallback || (beta != 0.0 && st->tp_bad)) ? 1 : 0;
+    if (direct && kind == ATT_CARRIED) {  // left to the next refresh attempt
+      st->phase = PH_DIRECT;
+      return;
+    }
+    st->direct_lc = st->tp_bad = direct;
+    st->phase = PH_NEW_ITER;
+  }
+  st->fallback = fallback;
   st->beta = beta;
   st->restart_flag = (beta == 0.0) ? 1 : 0;
   if (beta == 0.0) st->restarts += 1;

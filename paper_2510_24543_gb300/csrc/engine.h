@@ -69,6 +69,19 @@ inline int attempts_ahead(int poll, int max_iter, long long launched) {
   return left > 0 && left < poll ? (int)left : poll;
 }
 
+// FP64 engines with a preconditioner whose z comes from P_Delta alone carry T psi and
+// T p along, and every kRefreshEvery-th attempt transforms the trial state instead
+// (a refresh costs about a sixth of an attempt more).  FP32 engines do not: the carried
+// T psi does not see the rounding of psi itself, which the transformed one feeds back into
+// the residual, and 12 iterations at 128^3 ended 9e-7 from the FP64 iterates instead of
+// 2e-7 (and were 6% faster).
+inline bool carried_mode(int mode) { return mode == 1 || mode == 3; }
+constexpr int kRefreshEvery = 8;
+inline AttemptKind attempt_kind(bool carried, long long launched, bool want_refresh) {
+  if (!carried) return ATT_FULL;
+  return want_refresh || launched % kRefreshEvery == kRefreshEvery - 1 ? ATT_REFRESH : ATT_CARRIED;
+}
+
 template <class R> class Engine {
  public:
   using C = C2<R>;
@@ -78,6 +91,9 @@ template <class R> class Engine {
   ~Engine() { destroy(); }
 
   egpe_status create(const egpe_grid& g, const egpe_params& p, cudaStream_t stream);
+  // Whether attempts of this mode carry T psi and T p along: allocates their 10 fields
+  // at the first solve that does; where they do not fit, every attempt is ATT_FULL.
+  bool ensure_carry(int mode);
   void destroy();
 
   // Standalone evaluations (synchronous; device pointers of this precision).
@@ -137,7 +153,7 @@ template <class R> class Engine {
   // Captured graphs hold launch shapes: drop them when the shapes change.
   void drop_graphs();
   // Records (instead of launching) the kernels of one solver attempt.
-  egpe_status record_attempt(int mode, std::vector<LaunchRec<R>>& recs, std::vector<KArgs<R>>& args);
+  egpe_status record_attempt(int mode, AttemptKind kind, std::vector<LaunchRec<R>>& recs, std::vector<KArgs<R>>& args);
   C* current_psi();  // valid after solve (device)
   C* psi_slot0();    // psi buffer 0 (start of a solve)
 
@@ -147,10 +163,15 @@ template <class R> class Engine {
   double dV = 0.0;
 
  private:
-  egpe_status enq_eg(int trial, int gate, int ctrl);
-  egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven);
-  egpe_status enq_lc(int gate, int ctrl, int pgiven);
-  egpe_status enq_attempt(int mode);
+  // att: whether T psi is stored for attempts that carry it along (not ATT_FULL)
+  egpe_status enq_eg(int trial, int gate, int ctrl, AttemptKind att = ATT_FULL);
+  egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att = ATT_FULL);
+  egpe_status enq_lc(int gate, int ctrl, int pgiven, AttemptKind att = ATT_FULL);
+  egpe_status enq_dipolar(const KArgs<R>& a);
+  egpe_status enq_eg_carried(int gate, int ctrl);
+  egpe_status enq_lc_carried(int mode, int gate, int ctrl);
+  egpe_status enq_attempt(int mode, AttemptKind kind);
+  egpe_status capture_attempt(int mode, AttemptKind kind, cudaGraphExec_t& out, int& kernels);
   egpe_status enq_kin(int potential, int gate);
   egpe_status enq_pg(int gate);
   egpe_status apply_params(const egpe_params& p);
@@ -215,6 +236,8 @@ template <class R> class Engine {
   egpe_grid grid_{};
   egpe_params prm_{};
   void* arena_ = nullptr;
+  void* carry_ = nullptr;  // tb, tp, wz
+  bool carry_failed_ = false;
   C* twx_ = nullptr;
   C* twy_ = nullptr;
   C* twz_ = nullptr;
@@ -235,6 +258,10 @@ template <class R> class Engine {
   long long kernels_ = 0;
   std::unordered_map<unsigned long long, int> occ_;
   cudaGraphExec_t graph_[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  cudaGraphExec_t refresh_[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // refresh attempts, by mode
+  int refresh_kernels_[5] = {0, 0, 0, 0, 0};
+  bool run_carried_ = false;
+  bool want_refresh_ = false;  // the last look found an iteration waiting for one
   int run_mode_ = 0, run_graph_ = 1;
   long long run_k0_ = 0, run_launches_ = 0, per_attempt_ = 0;
   int graph_max_iter_[5] = {0, 0, 0, 0, 0};

@@ -44,3 +44,12 @@
   template egpe_status Engine<R>::plain_x_##SFX(int, const KArgs<R>&);                                   \
   template egpe_status Engine<R>::plain_col_##SFX(int, int, const KArgs<R>&, const CUtensorMap*);        \
   }
+
+// The passes of attempts that carry T psi and T p along (FP64 engines).
+#define EGPE_EXT_INSTANTIATE_CARRIED(SFX)                                                   \
+  namespace egpe {                                                                          \
+  template egpe_status Engine<double>::dispatch_x_##SFX<XFwdLL>(int, const KArgs<double>&); \
+  template egpe_status Engine<double>::dispatch_x_##SFX<XInvLL>(int, const KArgs<double>&); \
+  template egpe_status Engine<double>::dispatch_x_##SFX<XFwdEL>(int, const KArgs<double>&); \
+  template egpe_status Engine<double>::dispatch_x_##SFX<XInvEL>(int, const KArgs<double>&); \
+  }

@@ -83,7 +83,7 @@ template <class Op> cudaError_t noalloc_launch_x(egpe::KArgs<double> a, int rows
                       mx * row_pass_bytes<Op>() + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
   const int groups = (rows + mx - 1) / mx;
   const int grid = std::min(groups, (int)kNoAllocBlocks);
-  xpass_kernel<Op><<<grid, mx * RowGroups<Op>::v * L / 8, smem, s>>>(a);
+  xpass_kernel<Op><<<grid, mx * row_groups<Op>(mx, rows, kNoAllocSMs) * L / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -319,28 +319,43 @@ template <class R> void Engine<R>::set_wait_limit(long long polls) {
 }
 
 template <class R> void Engine<R>::drop_graphs() {
-  for (auto& gx : graph_)
-    if (gx) {
-      cudaGraphExecDestroy(gx);
-      gx = nullptr;
-    }
+  for (auto* set : {graph_, refresh_})
+    for (int m = 0; m < 5; ++m)
+      if (set[m]) {
+        cudaGraphExecDestroy(set[m]);
+        set[m] = nullptr;
+      }
   if (graph_ite_) cudaGraphExecDestroy(graph_ite_);
   graph_ite_ = nullptr;
 }
 
+template <class R> bool Engine<R>::ensure_carry(int mode) {
+  if (sizeof(R) != 8 || !carried_mode(mode) || carry_failed_) return false;
+  if (carry_) return true;
+  // tb[2], tp[2], wz: every value is written before it is read
+  if (cudaMalloc(&carry_, 10 * N * sizeof(C)) != cudaSuccess) {
+    cudaGetLastError();
+    carry_ = nullptr;
+    carry_failed_ = true;
+    return false;
+  }
+  C* c = reinterpret_cast<C*>(carry_);
+  for (int b = 0; b < 2; ++b) base_->tb[b] = c + 2 * b * N;
+  for (int b = 0; b < 2; ++b) base_->tp[b] = c + (4 + 2 * b) * N;
+  base_->wz = c + 8 * N;
+  return true;
+}
+
 template <class R> void Engine<R>::destroy() {
+  if (carry_) cudaFree(carry_);
+  carry_ = nullptr;
+  carry_failed_ = false;
   for (auto& k : tlog_) {
     cudaEventDestroy(k.a);
     cudaEventDestroy(k.b);
   }
   tlog_.clear();
-  for (auto& gx : graph_)
-    if (gx) {
-      cudaGraphExecDestroy(gx);
-      gx = nullptr;
-    }
-  if (graph_ite_) cudaGraphExecDestroy(graph_ite_);
-  graph_ite_ = nullptr;
+  drop_graphs();
   if (kin_tab_) cudaFree(kin_tab_);
   kin_tab_ = nullptr;
   if (arena_) cudaFree(arena_);
@@ -433,7 +448,8 @@ egpe_status Engine<R>::profile_attempt(const C* psi, int precond, int reps, std:
   EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(reset_state(&o, sizeof(R) == 4, 1 << 30, 0.0, sizeof(R) == 4 ? 1e-6 : 1e-13));
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1));
+  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0, false);
+  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   EGPE_CUDA(cudaStreamSynchronize(stream));
   names.clear();
   ms.clear();
@@ -441,7 +457,7 @@ egpe_status Engine<R>::profile_attempt(const C* psi, int precond, int reps, std:
   timing_ = true;
   for (int r = 0; r < reps; ++r) {
     tpos_ = 0;
-    egpe_status s = enq_attempt(o.precond);
+    egpe_status s = enq_attempt(o.precond, kind);
     if (s != EGPE_OK) {
       timing_ = false;
       return s;
@@ -486,12 +502,13 @@ egpe_status Engine<R>::record(const KArgs<R>& a, const CUtensorMap* tm, const vo
 }
 
 template <class R>
-egpe_status Engine<R>::record_attempt(int mode, std::vector<LaunchRec<R>>& recs, std::vector<KArgs<R>>& args) {
+egpe_status Engine<R>::record_attempt(int mode, AttemptKind kind, std::vector<LaunchRec<R>>& recs,
+                                      std::vector<KArgs<R>>& args) {
   recs.clear();
   args.clear();
   rec_ = &recs;
   rec_args_ = &args;
-  const egpe_status s = enq_attempt(mode);
+  const egpe_status s = enq_attempt(mode, kind);
   rec_ = nullptr;
   rec_args_ = nullptr;
   return s;
@@ -521,14 +538,15 @@ egpe_status Engine<R>::autotune(const C* psi, int precond, int reps, std::vector
   EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(reset_state(&o, sizeof(R) == 4, 1 << 30, 0.0, sizeof(R) == 4 ? 1e-6 : 1e-13));
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1));
-  EGPE_TRY(enq_attempt(o.precond));  // realistic coefficients in the state
+  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0, false);
+  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
+  EGPE_TRY(enq_attempt(o.precond, kind));  // realistic coefficients in the state
   EGPE_CUDA(cudaStreamSynchronize(stream));
   tune_.clear();
   set_col_bytes(EGPE_COL_BYTES);
   std::vector<LaunchRec<R>> recs;
   std::vector<KArgs<R>> args;
-  EGPE_TRY(record_attempt(o.precond, recs, args));
+  EGPE_TRY(record_attempt(o.precond, kind, recs, args));
   cudaEvent_t e0, e1;
   EGPE_CUDA(cudaEventCreate(&e0));
   EGPE_CUDA(cudaEventCreate(&e1));
@@ -650,7 +668,7 @@ egpe_status Engine<R>::autotune(const C* psi, int precond, int reps, std::vector
       set_col_bytes(w);
       std::vector<LaunchRec<R>> wr;
       std::vector<KArgs<R>> wa;
-      st = record_attempt(o.precond, wr, wa);
+      st = record_attempt(o.precond, kind, wr, wa);
       if (st != EGPE_OK) break;
       const double t = time_seq(wr, wa);
       if (st != EGPE_OK) break;
@@ -687,13 +705,13 @@ egpe_status Engine<R>::launch_point(void (*kern)(KArgs<R>), void (*kern_b)(KBatc
 }
 
 template <class R> template <class Op> egpe_status Engine<R>::launch_x(KArgs<R> a) {
-  // TPL: threads of one row
-  constexpr int L = Op::L, NS = Op::NS, TPL = RowGroups<Op>::v * L / 8;
+  constexpr int L = Op::L, NS = Op::NS;
   const size_t rowbytes = row_pass_bytes<Op>();
   const size_t smem_fixed =
       L * sizeof(C) + (Op::USES_LHY ? lhy_stage_bytes<R>(a.Q) : 0) + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
   const int rows = ny * nz;
   const int mx_default = default_rows<Op>(rows, nsm_);
+  const int TPL = row_groups<Op>(mx_default, rows, nsm_) * L / 8;  // threads of one row
   int mx = mx_default;
   if (!tune_.empty()) {
     auto it = tune_.find(typeid(Op).name());
@@ -864,8 +882,9 @@ egpe_status Engine<R>::plain_col(int axis, int inverse, const KArgs<R>& a, const
 }
 
 // Energy / gradient pipeline: 6 complex 3D transforms.
-template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl) {
+template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl, AttemptKind att) {
   KArgs<R> a = *base_;
+  a.att = att;
   a.gate = gate;
   a.flag = trial;
   a.ctrl = 0;
@@ -883,8 +902,9 @@ template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl) 
 }
 
 // Preconditioner pipeline: 4 transforms for the kinetic modes, none otherwise.
-template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, int rgiven) {
+template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att) {
   KArgs<R> a = *base_;
+  a.att = att;
   a.gate = gate;
   a.flag = rgiven;
   a.diag = (mode == 2 || mode == 3) ? 1 : 0;
@@ -909,8 +929,9 @@ template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, i
 }
 
 // Line-search pipeline: forward transforms of p_1, p_2 and one packed pair.
-template <class R> egpe_status Engine<R>::enq_lc(int gate, int ctrl, int pgiven) {
+template <class R> egpe_status Engine<R>::enq_lc(int gate, int ctrl, int pgiven, AttemptKind att) {
   KArgs<R> a = *base_;
+  a.att = att;
   a.gate = gate;
   a.flag = pgiven;
   a.ctrl = 0;
@@ -929,7 +950,67 @@ template <class R> egpe_status Engine<R>::enq_lc(int gate, int ctrl, int pgiven)
   return dispatch_x<XInvLC>(nx, a);
 }
 
-template <class R> egpe_status Engine<R>::enq_attempt(int mode) {
+// Field 0 of the workspace through the rest of the dipolar convolution.
+template <class R> egpe_status Engine<R>::enq_dipolar(const KArgs<R>& a) {
+  KArgs<R> y = a;
+  y.gin = a.W;
+  y.gout = a.W;
+  EGPE_TRY(plain_col(1, 0, y, tmy()));
+  EGPE_TRY(dispatch_col<ZPg>(nz, a, tmz()));
+  return plain_col(1, 1, y, tmy());
+}
+
+// Line-search and trial pipelines with T psi and T p carried along: one packed
+// transform pair each (the dipolar convolutions of rho and of the trial densities).
+template <class R> egpe_status Engine<R>::enq_lc_carried(int mode, int gate, int ctrl) {
+  KArgs<R> a = *base_;
+  a.att = ATT_CARRIED;
+  a.gate = gate;
+  a.flag = 0;
+  a.ctrl = 0;
+  a.diag = mode == 3 ? 1 : 0;
+  a.nf = 1;
+  a.f0 = 0;
+  if constexpr (sizeof(R) == 8) {
+    EGPE_TRY(dispatch_x<XFwdLL>(nx, a));
+    EGPE_TRY(enq_dipolar(a));
+    a.ctrl = ctrl;
+    return dispatch_x<XInvLL>(nx, a);
+  }
+  return EGPE_ERR_UNSUPPORTED;
+}
+
+template <class R> egpe_status Engine<R>::enq_eg_carried(int gate, int ctrl) {
+  KArgs<R> a = *base_;
+  a.att = ATT_CARRIED;
+  a.gate = gate;
+  a.flag = 1;
+  a.ctrl = 0;
+  a.nf = 1;
+  a.f0 = 0;
+  if constexpr (sizeof(R) == 8) {
+    EGPE_TRY(dispatch_x<XFwdEL>(nx, a));
+    EGPE_TRY(enq_dipolar(a));
+    a.ctrl = ctrl;
+    return dispatch_x<XInvEL>(nx, a);
+  }
+  return EGPE_ERR_UNSUPPORTED;
+}
+
+template <class R> egpe_status Engine<R>::enq_attempt(int mode, AttemptKind kind) {
+  if constexpr (sizeof(R) == 8) {
+    if (kind == ATT_CARRIED) {
+      EGPE_TRY(enq_pc(mode, GATE_NEW_ITER, 1, 0, kind));
+      EGPE_TRY(enq_lc_carried(mode, GATE_NEW_ITER, 1));
+      return enq_eg_carried(GATE_CARRIED_TRIAL, 1);
+    }
+    if (kind == ATT_REFRESH) {
+      EGPE_TRY(enq_pc(mode, GATE_REFRESH_PC, 1, 0, kind));
+      EGPE_TRY(enq_lc_carried(mode, GATE_REFRESH_CARRIED, 1));
+      EGPE_TRY(enq_lc(GATE_REFRESH_DIRECT, 1, 0, kind));
+      return enq_eg(1, GATE_ACTIVE, 1, kind);
+    }
+  }
   EGPE_TRY(enq_pc(mode, GATE_NEW_ITER, 1, 0));
   EGPE_TRY(enq_lc(GATE_NEW_ITER, 1, 0));
   return enq_eg(1, GATE_ACTIVE, 1);
@@ -1106,11 +1187,7 @@ egpe_status Engine<R>::solve_begin(const egpe_solve_opts& o, int fp32_phase, int
   if (want_trace && trace_cap > trace_alloc_) {
     // the trace buffer is captured by the graphs: allocate once, generously
     const int want = std::max(trace_cap, 65536);
-    for (auto& gx : graph_)
-      if (gx) {
-        cudaGraphExecDestroy(gx);
-        gx = nullptr;
-      }
+    drop_graphs();
     if (trace_) cudaFree(trace_);
     trace_ = nullptr;
     EGPE_CUDA(cudaMalloc(&trace_, (size_t)want * sizeof(TraceDev)));
@@ -1123,39 +1200,47 @@ egpe_status Engine<R>::solve_begin(const egpe_solve_opts& o, int fp32_phase, int
   EGPE_TRY(reset_state(&oo, fp32_phase, max_iter, tol_res, accept_rtol));
   // r and p history start at zero (beta = 0 at n = 0 reads them)
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1));
+  run_carried_ = ensure_carry(mode);
+  const AttemptKind kind = attempt_kind(run_carried_, 0, false);
+  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   run_k0_ = kernels_;
   run_ite_ = false;
   run_mode_ = mode;
   run_graph_ = o.use_graph ? 1 : 0;
   run_launches_ = 0;
   per_attempt_ = 0;
+  want_refresh_ = false;
   if (run_graph_) {
-    if (!graph_[mode]) {
-      cudaGraph_t g = nullptr;
-      EGPE_CUDA(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-      const long long kb = kernels_;
-      egpe_status s = enq_attempt(mode);
-      cudaError_t ce = cudaStreamEndCapture(stream, &g);
-      if (s != EGPE_OK) {
-        if (g) cudaGraphDestroy(g);
-        return s;
-      }
-      if (ce != cudaSuccess) {
-        set_error("cudaStreamEndCapture", ce);
-        return EGPE_ERR_CUDA;
-      }
-      graph_max_iter_[mode] = (int)(kernels_ - kb);
-      cudaError_t ie = cudaGraphInstantiate(&graph_[mode], g, 0);
-      cudaGraphDestroy(g);
-      if (ie != cudaSuccess) {
-        set_error("cudaGraphInstantiate", ie);
-        graph_[mode] = nullptr;
-        return EGPE_ERR_CUDA;
-      }
-      kernels_ = kb;
-    }
+    if (!graph_[mode]) EGPE_TRY(capture_attempt(mode, kind, graph_[mode], graph_max_iter_[mode]));
     per_attempt_ = graph_max_iter_[mode];
+  }
+  return EGPE_OK;
+}
+
+// Captures one attempt into an executable graph and counts its kernels.
+template <class R>
+egpe_status Engine<R>::capture_attempt(int mode, AttemptKind kind, cudaGraphExec_t& out, int& kernels) {
+  cudaGraph_t g = nullptr;
+  EGPE_CUDA(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
+  const long long kb = kernels_;
+  egpe_status s = enq_attempt(mode, kind);
+  cudaError_t ce = cudaStreamEndCapture(stream, &g);
+  kernels = (int)(kernels_ - kb);
+  kernels_ = kb;
+  if (s != EGPE_OK) {
+    if (g) cudaGraphDestroy(g);
+    return s;
+  }
+  if (ce != cudaSuccess) {
+    set_error("cudaStreamEndCapture", ce);
+    return EGPE_ERR_CUDA;
+  }
+  cudaError_t ie = cudaGraphInstantiate(&out, g, 0);
+  cudaGraphDestroy(g);
+  if (ie != cudaSuccess) {
+    set_error("cudaGraphInstantiate", ie);
+    out = nullptr;
+    return EGPE_ERR_CUDA;
   }
   return EGPE_OK;
 }
@@ -1271,11 +1356,20 @@ template <class R> egpe_status Engine<R>::solve_launch(int attempts) {
       } else {
         EGPE_TRY(enq_ite_step(GATE_ACTIVE));
       }
-    } else if (run_graph_) {
-      EGPE_CUDA(cudaGraphLaunch(graph_[run_mode_], stream));
-      kernels_ += per_attempt_;
     } else {
-      EGPE_TRY(enq_attempt(run_mode_));
+      const AttemptKind kind = attempt_kind(run_carried_, run_launches_, want_refresh_);
+      want_refresh_ = false;
+      if (!run_graph_) {
+        EGPE_TRY(enq_attempt(run_mode_, kind));
+      } else if (kind == ATT_REFRESH) {
+        if (!refresh_[run_mode_])
+          EGPE_TRY(capture_attempt(run_mode_, kind, refresh_[run_mode_], refresh_kernels_[run_mode_]));
+        EGPE_CUDA(cudaGraphLaunch(refresh_[run_mode_], stream));
+        kernels_ += refresh_kernels_[run_mode_];
+      } else {
+        EGPE_CUDA(cudaGraphLaunch(graph_[run_mode_], stream));
+        kernels_ += per_attempt_;
+      }
     }
     ++run_launches_;
   }
@@ -1286,6 +1380,7 @@ template <class R> egpe_status Engine<R>::solve_poll(int& phase) {
   EGPE_CUDA(cudaMemcpyAsync(&st_host_->phase, &st_->phase, sizeof(int), cudaMemcpyDeviceToHost, stream));
   EGPE_CUDA(cudaStreamSynchronize(stream));
   phase = st_host_->phase;
+  want_refresh_ = phase == PH_DIRECT;
   return EGPE_OK;
 }
 
@@ -1347,7 +1442,8 @@ egpe_status Engine<R>::solve(const egpe_solve_opts& o, int fp32_phase, int max_i
                              int trace_offset) {
   EGPE_TRY(solve_begin(o, fp32_phase, max_iter, tol_res, accept_rtol, trace_out != nullptr, trace_cap));
   const int poll = std::max(1, o.poll_every);
-  const long long max_launch = (long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4;
+  const long long max_launch =
+      ((long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4) * (run_carried_ ? kRefreshEvery : 1);
   while (run_launches_ < max_launch) {
     EGPE_TRY(solve_launch(attempts_ahead(poll, max_iter, run_launches_)));
     int phase = 0;

@@ -2,3 +2,4 @@
 #include "engine_ext.cuh"
 EGPE_EXT_DEFINE(mr, 48, 96)
 EGPE_EXT_INSTANTIATE(double, mr)
+EGPE_EXT_INSTANTIATE_CARRIED(mr)

@@ -49,6 +49,9 @@ template <class R> struct KArgs {
   C* pb[2];                  // direction buffers (current / previous)
   C* z;                      // preconditioned residual
   C* W;                      // transform workspace, 3 fields
+  C* tb[2];                  // T psi of the psi buffers (attempts that carry it along)
+  C* tp[2];                  // T p of the direction buffers
+  C* wz;                     // P_V^{-1} r, where T z = wz - alpha z
   const C* gin;              // generic in/out of the plain passes
   C* gout;
   double* partials;
@@ -62,13 +65,22 @@ template <class R> struct KArgs {
   int ctrl;                  // run the controller step in the last block
   int diag;                  // P_V part of the preconditioner
   int blend;                 // weighted P_V / P_Delta combination (mode 4)
+  int att;                   // AttemptKind
   long long wait_polls;      // poll budget of a TMA tile wait before the pass reports a timeout
 };
 
 template <class R> __device__ __forceinline__ bool gate_open(const KArgs<R>& a) {
   if (a.gate == GATE_ALWAYS) return true;
   const int ph = __ldcg(&a.st->phase);
-  return a.gate == GATE_NEW_ITER ? (ph == PH_NEW_ITER) : (ph != PH_DONE);
+  const bool on = ph == PH_NEW_ITER || ph == PH_TRIAL;
+  switch (a.gate) {
+    case GATE_NEW_ITER: return ph == PH_NEW_ITER;
+    case GATE_REFRESH_PC: return ph == PH_NEW_ITER || ph == PH_DIRECT;
+    case GATE_REFRESH_CARRIED: return ph == PH_NEW_ITER && !__ldcg(&a.st->direct_lc);
+    case GATE_REFRESH_DIRECT: return ph == PH_NEW_ITER && __ldcg(&a.st->direct_lc);
+    case GATE_CARRIED_TRIAL: return on && !__ldcg(&a.st->tp_bad);
+  }
+  return on;
 }
 
 // Batched launches: one launch runs the same pass for up to KB_MAX instances
@@ -166,10 +178,16 @@ template <class Op> struct MaxThreadsWant<Op, std::void_t<decltype(Op::MAXT)>> {
 template <class Op> struct RowGroups {
   static constexpr int v = sizeof(typename Op::R) == 8 ? Op::NF : 1;
 };
+// FP64 epilogues of one field (power-of-two lengths, whose transforms need no block
+// barrier) may be launched with two groups more that only take points (row_groups).
+template <class Op> struct ExtraGroups {
+  static constexpr int v = sizeof(typename Op::R) == 8 && Op::NF == 1 && Op::POINTS && IsPow2<Op::L>::v ? 3 : 1;
+};
 template <class Op> struct MaxThreads {
   static constexpr int G = whole_warp_rows(Op::L) * (Op::L / 8) * RowGroups<Op>::v;
   static constexpr int W = MaxThreadsWant<Op>::v;
-  static constexpr int v = W >= G ? W - W % G : G;
+  static constexpr int v0 = W >= G ? W - W % G : G;
+  static constexpr int v = v0 > G * ExtraGroups<Op>::v ? v0 : G * ExtraGroups<Op>::v;
 };
 
 // Minimum resident blocks per SM a row-pass op asks the compiler to allow for
@@ -251,7 +269,7 @@ template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typen
   double* vrow = reinterpret_cast<double*>(buf + NF * a.MX * LP);  // trap terms of the rows (block-wide epilogues)
   RedSmem<NSR>* red = reinterpret_cast<RedSmem<NSR>*>(vrow + a.MX);
   const int tid = threadIdx.x;
-  const int g = G > 1 ? tid / (a.MX * TPL) : 0;
+  const int g = G > 1 || ExtraGroups<Op>::v > 1 ? tid / (a.MX * TPL) : 0;
   const int rt = tid - g * a.MX * TPL;
   const int mrow = rt / TPL, t = rt - mrow * TPL;
   const int fs = a.MX * LP;  // a field's rows in buf
@@ -273,14 +291,16 @@ template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typen
     const int row = grp * a.MX + mrow;
     const bool valid = row < rows;
     C v[NV][8];
-    Op::load(a, u, f, row, valid, t, v);
-    fft_line<C, L, Op::INV, NV>(v, line, fs, tw, t, si);
+    if (ExtraGroups<Op>::v == 1 || g < NF) {
+      Op::load(a, u, f, row, valid, t, v);
+      fft_line<C, L, Op::INV, NV>(v, line, fs, tw, t, si);
+    }
     if constexpr (!Op::POINTS) {
       Op::store(a, u, f, row, valid, t, v, acc);
       if constexpr (G > 1 && !Op::INV) f = f + 1 < G ? f + 1 : 0;
     } else {
       constexpr bool ST = StageOut<Op>::v;
-      if constexpr (ST) {
+      if (ST && (ExtraGroups<Op>::v == 1 || g < NF)) {
 #pragma unroll
         for (int k = 0; k < NV; ++k)
 #pragma unroll
@@ -356,6 +376,14 @@ template <class Op> inline int default_rows(int rows, int nsm) {
          (sizeof(typename Op::R) == 4 || rows >= mx * 2 * nsm))
     mx *= 2;
   return mx;
+}
+
+// Thread groups of a launch: the extra ones where each SM has at most two row groups
+// (at 32^3 the energy epilogue takes 26 us instead of 40, the line epilogue 33 instead
+// of 48; at 128^3 they cost 12%).
+template <class Op> inline int row_groups(int mx, int rows, int nsm) {
+  return ExtraGroups<Op>::v > 1 && mx == whole_warp_rows(Op::L) && rows <= mx * 2 * nsm ? ExtraGroups<Op>::v
+                                                                                         : RowGroups<Op>::v;
 }
 
 // Row-pass entry points.  A min-blocks bound is given only when the op asks for
@@ -677,13 +705,13 @@ template <class R> struct EgUni {
 
 // Controller step after an energy/gradient evaluation (last block, one thread):
 // ctrl 1 = NCG (start point or trial), ctrl 2 = end of an imaginary-time step.
-template <class R> __device__ __forceinline__ void eg_ctrl(const KArgs<R>& a) {
+template <class R> __device__ __forceinline__ void eg_ctrl(const KArgs<R>& a, int lin) {
   if (a.ctrl == 2) {
     a.st->ffts += 20;  // two kinetic half steps (8) and two evaluations (12)
     ctrl_after_ite(a.st);
   } else if (a.ctrl) {
-    a.st->ffts += 6;
-    ctrl_after_eg(a.st, a.flag ? 1 : 0, a.trace);
+    a.st->ffts += lin ? 2 : 6;
+    ctrl_after_eg(a.st, a.flag ? 1 : 0, lin, a.trace);
   }
 }
 
@@ -896,22 +924,22 @@ __device__ __forceinline__ void lhy_second(const KArgs<R>& a, const LhyNode<R>* 
   }
 }
 
-template <class R_, int L_> struct XInvEG {
+template <class R_, int L_, bool LIN> struct XInvEGT {
   using R = R_;
   using C = C2<R>;
   // FP32: 128 threads, 4 blocks per SM (128 registers; the mixed-radix lengths 3, which
   // spill at 4); FP64: three groups of 32 threads
-  static constexpr int PTS = 4, MAXT = sizeof(R_) == 4 ? 128 : 96, MINB = sizeof(R_) == 4 ? (IsPow2<L_>::v ? 4 : 3) : 1;
+  static constexpr int PTS = 4, MAXT = sizeof(R_) == 4 ? 128 : LIN ? 64 : 96, MINB = sizeof(R_) == 4 ? (IsPow2<L_>::v ? 4 : 3) : 1;
   static constexpr bool STAGE_OUT = true;
   static constexpr const char* NAME = "x-inv energy+LHY";
-  static double alg_bytes(const KArgs<R>& a) { return 9.0 * a.N * sizeof(C); }
-  static constexpr int L = L_, NF = 3, NS = EG_NS;
+  static double alg_bytes(const KArgs<R>& a) { return (LIN || a.att == ATT_FULL ? 9.0 : 11.0) * a.N * sizeof(C); }
+  static constexpr int L = L_, NF = LIN ? 1 : 3, NS = EG_NS;
   static constexpr bool INV = true, USES_LHY = true, LHY_TAB = true, POINTS = true;
   using Uni = EgUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { XFwdEG<R, L>::uniform(a, u); }
   template <int NV>
   static __device__ void load(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8]) {
-    load_rows<XInvEG>(a, a.W, f, row, valid, t, v);
+    load_rows<XInvEGT>(a, a.W, f, row, valid, t, v);
   }
   template <int NP, bool ST>
   static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[EG_NS],
@@ -919,13 +947,18 @@ template <class R_, int L_> struct XInvEG {
     const C* ps = pick(a.psi, u.slot);
     C* hp = pick(a.hp, u.slot);
     C* ax = pick(a.ax, u.slot);
+    C* tb = pick(a.tb, u.slot);
     const size_t N = a.N;
-    C p1[NP], p2[NP];
+    C p1[NP], p2[NP], k1[NP], k2[NP];
     R n1[NP], n2[NP], m1[NP], m2[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
       p1[j] = ps[pt[j].idx];
       p2[j] = ps[N + pt[j].idx];
+      if constexpr (LIN) {
+        k1[j] = tb[pt[j].idx];
+        k2[j] = tb[N + pt[j].idx];
+      }
       n1[j] = cabs2(p1[j]);
       n2[j] = cabs2(p2[j]);
     }
@@ -934,7 +967,15 @@ template <class R_, int L_> struct XInvEG {
     for (int j = 0; j < NP; ++j) {
       const size_t idx = pt[j].idx;
       const R V = trap_x(a, pt[j].x) + pt[j].vyz;
-      const C T1 = pt[j].out(0), T2 = pt[j].out(1), PH = pt[j].out(2);
+      const C T1 = LIN ? k1[j] : pt[j].out(0), T2 = LIN ? k2[j] : pt[j].out(NF > 1 ? 1 : 0);
+      const C PH = pt[j].out(NF - 1);
+      if constexpr (LIN) {
+        cdot_add(s[EG_KIN1], p1[j], T1);
+        cdot_add(s[EG_KIN2], p2[j], T2);
+      } else if (a.att != ATT_FULL) {
+        tb[idx] = T1;
+        tb[N + idx] = T2;
+      }
       const R phi1 = PH.x, phi2 = PH.y;
       const R c1 = fma_(a.g12, n2[j], a.g11 * n1[j]), c2 = fma_(a.g22, n2[j], a.g21 * n1[j]);
       const R B1 = (V + c1) + m1[j], B2 = (V + c2) + m2[j];
@@ -957,8 +998,10 @@ template <class R_, int L_> struct XInvEG {
     }
   }
   static __device__ double* out(const KArgs<R>& a, Uni& u) { return a.st->eg[u.slot]; }
-  static __device__ void finish(const KArgs<R>& a, Uni&) { eg_ctrl(a); }
+  static __device__ void finish(const KArgs<R>& a, Uni&) { eg_ctrl(a, LIN); }
 };
+template <class R, int L> struct XInvEG : XInvEGT<R, L, false> {};
+template <class R, int L> struct XInvEL : XInvEGT<R, L, true> {};
 
 // ----------------------------------------------------------------------------
 // Preconditioner pipeline (Sec. IV.B): r = H psi - mu psi, z = P^{-1} r with
@@ -1028,7 +1071,10 @@ __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u
         r = cmk<C>(fma_(-mu, p[k][j].x, r.x), fma_(-mu, p[k][j].y, r.y));
         pick(a.rb, u.nsel)[(size_t)c * N + idx[j]] = r;
       }
-      if (a.diag) r = cscale(r, rcp_(pv_at(u, c, c ? bb[j].y : bb[j].x)));
+      if (a.diag) {
+        r = cscale(r, rcp_(pv_at(u, c, c ? bb[j].y : bb[j].x)));
+        if (a.att != ATT_FULL) a.wz[(size_t)c * N + idx[j]] = r;
+      }
       w[k][j] = r;
     }
   }
@@ -1186,7 +1232,7 @@ template <class R_, int L_> struct XInvPC {
   static __device__ void finish(const KArgs<R>& a, Uni&) {
     if (a.ctrl) {
       a.st->ffts += 4;
-      ctrl_after_pc(a.st);
+      ctrl_after_pc(a.st, a.att);
     }
   }
 };
@@ -1218,7 +1264,7 @@ __device__ __forceinline__ void pc_point_body(const KArgs<R>& a) {
     for (int k = 0; k < PC_NS; ++k) acc[k].add(s[k]);
   }
   if (reduce_blocks<PC_NS>(acc, a.partials, a.counter, a.st->pc, red)) {
-    if (threadIdx.x == 0 && a.ctrl) ctrl_after_pc(a.st);
+    if (threadIdx.x == 0 && a.ctrl) ctrl_after_pc(a.st, a.att);
   }
 }
 template <class R> __global__ void __launch_bounds__(256) pc_point_kernel(KArgs<R> a) { pc_point_body(a); }
@@ -1402,7 +1448,7 @@ template <class R_, int L_> struct ZLc {
   static __device__ void finish(const KArgs<R>&, Uni&) {}
 };
 
-template <class R_, int L_> struct XInvLC {
+template <class R_, int L_, bool LIN> struct XInvLCT {
   using R = R_;
   using C = C2<R>;
   static constexpr int PTS = 4, MAXT = sizeof(R_) == 4 ? 256 : 64, MINB = sizeof(R_) == 4 ? 2 : 1;
@@ -1414,7 +1460,7 @@ template <class R_, int L_> struct XInvLC {
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { lc_uniform(a, u); }
   template <int NV>
   static __device__ void load(const KArgs<R>& a, Uni&, int, int row, bool valid, int t, C (&v)[NV][8]) {
-    load_rows<XInvLC>(a, a.W, 2, row, valid, t, v);
+    load_rows<XInvLCT>(a, a.W, LIN ? 0 : 2, row, valid, t, v);
   }
   template <int NP, bool ST>
   static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[LC_NS],
@@ -1467,10 +1513,155 @@ template <class R_, int L_> struct XInvLC {
   static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->lc; }
   static __device__ void finish(const KArgs<R>& a, Uni&) {
     if (a.ctrl) {
-      a.st->ffts += 4;
+      a.st->ffts += LIN ? 2 : 4;
       ctrl_after_lc(a.st);
     }
   }
+};
+template <class R, int L> struct XInvLC : XInvLCT<R, L, false> {};
+template <class R, int L> struct XInvLL : XInvLCT<R, L, true> {};
+
+// Direction of an attempt that carries T psi and T p along: p and T p from their
+// terms (T z = w - alpha z, w = P_V^{-1} r or r), and the forward rows of the packed
+// source of rho alone.
+template <class R_, int L_> struct XFwdLL {
+  using R = R_;
+  using C = C2<R>;
+  static constexpr int MAXT = 64;
+  static constexpr const char* NAME = "x-fwd line dir";
+  static double alg_bytes(const KArgs<R>& a) { return 17.0 * a.N * sizeof(C); }
+  static constexpr int L = L_, NF = 1, NS = LCZ_NS;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
+  struct Uni : LcUni<R> {
+    R shift[2], tpp[2];  // tpp: <p_i, T p_i> over the thread's points of a row
+  };
+  static __device__ void uniform(const KArgs<R>& a, Uni& u) {
+    lc_uniform(a, u);
+    load_uniforms<R, 2>({&a.st->shift[0], &a.st->shift[1]}, u.shift);
+  }
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int, int row, bool valid, int t, C (&v)[NV][8]) {
+    u.tpp[0] = u.tpp[1] = R(0);
+    const size_t N = a.N;
+    const C* ps = pick(a.psi, u.cur);
+    const C* ts = pick(a.tb, u.cur);
+    const C* pp = pick(a.pb, u.nsel ^ 1);
+    const C* tpp = pick(a.tp, u.nsel ^ 1);
+    const C* ws = a.diag ? a.wz : pick(a.rb, u.nsel);
+    C* pd = pick(a.pb, u.nsel);
+    C* td = pick(a.tp, u.nsel);
+    const bool usepp = u.beta != R(0);
+    constexpr int CH = 2;
+#pragma unroll
+    for (int e0 = 0; e0 < 8; e0 += CH) {
+      C p[2][CH], z[2][CH], w[2][CH], k[2][CH], d[2][CH], td1[2][CH];
+#pragma unroll
+      for (int j = 0; j < CH; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const size_t q = valid ? (size_t)i * N + (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j) : 0;
+          p[i][j] = ps[q];
+          z[i][j] = a.z[q];
+          w[i][j] = ws[q];
+          k[i][j] = ts[q];
+          if (usepp) {
+            d[i][j] = pp[q];
+            td1[i][j] = tpp[q];
+          }
+        }
+#pragma unroll
+      for (int j = 0; j < CH; ++j) {
+        R rho[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const R c = u.c[i], al = u.shift[i];
+          C q = cmk<C>(fma_(-c, p[i][j].x, -z[i][j].x), fma_(-c, p[i][j].y, -z[i][j].y));
+          C tq = cmk<C>(fma_(-c, k[i][j].x, fma_(al, z[i][j].x, -w[i][j].x)),
+                        fma_(-c, k[i][j].y, fma_(al, z[i][j].y, -w[i][j].y)));
+          if (usepp) {
+            q = cmk<C>(fma_(u.beta, d[i][j].x, q.x), fma_(u.beta, d[i][j].y, q.y));
+            tq = cmk<C>(fma_(u.beta, td1[i][j].x, tq.x), fma_(u.beta, td1[i][j].y, tq.y));
+          }
+          if (valid) {
+            const size_t o = (size_t)i * N + (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
+            pd[o] = q;
+            td[o] = tq;
+            cdot_add(u.tpp[i], q, tq);
+          }
+          rho[i] = valid ? cdot(p[i][j], q) : R(0);
+        }
+        v[0][e0 + j] = cmk<C>(fma_(a.d12, rho[1], a.d11 * rho[0]), fma_(a.d22, rho[1], a.d21 * rho[0]));
+      }
+    }
+  }
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>* acc) {
+    store_rows<XFwdLL>(a, a.W, f, row, valid, t, v);
+    acc[0].add(u.tpp[0]);
+    acc[1].add(u.tpp[1]);
+  }
+  static __device__ double* out(const KArgs<R>& a, Uni&) { return a.st->lcz; }
+  static __device__ void finish(const KArgs<R>&, Uni&) {}
+};
+
+// Trial point of such an attempt: psi' = a psi + b p and T psi' = a T psi + b T p, and
+// the forward rows of the packed dipolar source alone.
+template <class R_, int L_> struct XFwdEL {
+  using R = R_;
+  using C = C2<R>;
+  static constexpr const char* NAME = "x-fwd energy";
+  static double alg_bytes(const KArgs<R>& a) { return 13.0 * a.N * sizeof(C); }
+  static constexpr int L = L_, NF = 1, NS = 0;
+  static constexpr bool INV = false, USES_LHY = false, POINTS = false;
+  using Uni = EgUni<R>;
+  static __device__ void uniform(const KArgs<R>& a, Uni& u) { XFwdEG<R, L>::uniform(a, u); }
+  template <int NV>
+  static __device__ void load(const KArgs<R>& a, Uni& u, int, int row, bool valid, int t, C (&v)[NV][8]) {
+    const size_t N = a.N;
+    const C* ps = pick(a.psi, u.cur);
+    const C* ts = pick(a.tb, u.cur);
+    const C* pd = pick(a.pb, u.nsel);
+    const C* td = pick(a.tp, u.nsel);
+    C* po = pick(a.psi, u.slot);
+    C* to = pick(a.tb, u.slot);
+    constexpr int CH = ChunkW<R>::v;
+#pragma unroll
+    for (int e0 = 0; e0 < 8; e0 += CH) {
+      C p[2][CH], k[2][CH], q[2][CH], tq[2][CH];
+#pragma unroll
+      for (int j = 0; j < CH; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const size_t o = valid ? (size_t)i * N + (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j) : 0;
+          p[i][j] = ps[o];
+          k[i][j] = ts[o];
+          q[i][j] = pd[o];
+          tq[i][j] = td[o];
+        }
+#pragma unroll
+      for (int j = 0; j < CH; ++j) {
+        R n[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const R ca = u.ca[i], cb = u.cb[i];
+          const C x = cmk<C>(fma_(cb, q[i][j].x, ca * p[i][j].x), fma_(cb, q[i][j].y, ca * p[i][j].y));
+          if (valid) {
+            const size_t o = (size_t)i * N + (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
+            po[o] = x;
+            to[o] = cmk<C>(fma_(cb, tq[i][j].x, ca * k[i][j].x), fma_(cb, tq[i][j].y, ca * k[i][j].y));
+          }
+          n[i] = valid ? cabs2(x) : R(0);
+        }
+        v[0][e0 + j] = cmk<C>(fma_(a.d12, n[1], a.d11 * n[0]), fma_(a.d22, n[1], a.d21 * n[0]));
+      }
+    }
+  }
+  template <int NV>
+  static __device__ void store(const KArgs<R>& a, Uni&, int f, int row, bool valid, int t, C (&v)[NV][8], PAcc<R>*) {
+    store_rows<XFwdEL>(a, a.W, f, row, valid, t, v);
+  }
+  static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
+  static __device__ void finish(const KArgs<R>&, Uni&) {}
 };
 
 // ----------------------------------------------------------------------------
