@@ -164,8 +164,14 @@ template <class R> class Engine {
 
  private:
   // att: whether T psi is stored for attempts that carry it along (not ATT_FULL)
-  egpe_status enq_eg(int trial, int gate, int ctrl, AttemptKind att = ATT_FULL);
-  egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att = ATT_FULL);
+  // in, out: the caller's psi and gradient of a standalone evaluation (element-aligned)
+  egpe_status enq_eg(int trial, int gate, int ctrl, AttemptKind att = ATT_FULL, const C* in = nullptr,
+                     C* out = nullptr);
+  // A standalone evaluation of psi without waiting for it; hp and aux as after a trial.
+  egpe_status enq_evaluation(const C* psi, C* grad);
+  static bool element_aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % sizeof(C) == 0; }
+  void energy_out(const DevState& hs, egpe_energy_terms& out) const;
+  egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att = ATT_FULL, C* z = nullptr);
   egpe_status enq_lc(int gate, int ctrl, int pgiven, AttemptKind att = ATT_FULL);
   egpe_status enq_dipolar(const KArgs<R>& a);
   egpe_status enq_eg_carried(int gate, int ctrl);
@@ -173,7 +179,7 @@ template <class R> class Engine {
   egpe_status enq_attempt(int mode, AttemptKind kind);
   egpe_status capture_attempt(int mode, AttemptKind kind, cudaGraphExec_t& out, int& kernels);
   egpe_status enq_kin(int potential, int gate);
-  egpe_status enq_pg(int gate);
+  egpe_status enq_pg(int gate, const C* in);
   egpe_status apply_params(const egpe_params& p);
   egpe_status enq_ite_step(int gate);
   egpe_status reset_state(const egpe_solve_opts* o, int fp32_phase, int max_iter, double tol_res,

@@ -190,8 +190,9 @@ template <class R> egpe_status Engine<R>::set_params(const egpe_params& p) {
 
 // Parameter-derivative pass: one packed density field through the dipolar
 // kernel (4 transform passes) and the sums of the last row pass.
-template <class R> egpe_status Engine<R>::enq_pg(int gate) {
+template <class R> egpe_status Engine<R>::enq_pg(int gate, const C* in) {
   KArgs<R> a = *base_;
+  a.gin = in;
   a.gate = gate;
   a.flag = 0;
   a.ctrl = 0;
@@ -209,8 +210,10 @@ template <class R> egpe_status Engine<R>::enq_pg(int gate) {
 
 template <class R> egpe_status Engine<R>::param_grad(const C* psi, double out[EGPE_NPARAM]) {
   EGPE_TRY(reset_state(nullptr, 0, 0, 0.0, 0.0));
-  EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
-  EGPE_TRY(enq_pg(GATE_ALWAYS));
+  const bool direct = element_aligned(psi);
+  if (!direct)
+    EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  EGPE_TRY(enq_pg(GATE_ALWAYS, direct ? psi : nullptr));
   DevState hs;
   EGPE_TRY(read_state(hs));
   const double* s = hs.pg;
@@ -882,9 +885,12 @@ egpe_status Engine<R>::plain_col(int axis, int inverse, const KArgs<R>& a, const
 }
 
 // Energy / gradient pipeline: 6 complex 3D transforms.
-template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl, AttemptKind att) {
+template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl, AttemptKind att, const C* in,
+                                                       C* out) {
   KArgs<R> a = *base_;
   a.att = att;
+  a.gin = in;
+  a.gout = out;
   a.gate = gate;
   a.flag = trial;
   a.ctrl = 0;
@@ -902,9 +908,10 @@ template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl, 
 }
 
 // Preconditioner pipeline: 4 transforms for the kinetic modes, none otherwise.
-template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att) {
+template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att, C* z) {
   KArgs<R> a = *base_;
   a.att = att;
+  if (z) a.z = z;
   a.gate = gate;
   a.flag = rgiven;
   a.diag = (mode == 2 || mode == 3) ? 1 : 0;
@@ -1063,38 +1070,51 @@ template <class R> egpe_status Engine<R>::read_state(DevState& hs, bool report_t
   return EGPE_OK;
 }
 
-template <class R> egpe_status Engine<R>::energy_grad(const C* psi, egpe_energy_terms* out, C* grad) {
+// The first pass reads psi from the caller's buffer and leaves it in the psi buffer
+// (the later passes read it there, so grad may be psi), the last one writes H psi to
+// both: no copies of their own.  Buffers that are not element-aligned are copied.
+template <class R> egpe_status Engine<R>::enq_evaluation(const C* psi, C* grad) {
   EGPE_TRY(reset_state(nullptr, 0, 0, 0.0, 0.0));
-  EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
-  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1));
-  if (grad) EGPE_CUDA(cudaMemcpyAsync(grad, base_->hp[0], 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  const bool din = element_aligned(psi), dout = element_aligned(grad);
+  if (!din) EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, ATT_FULL, din ? psi : nullptr, dout ? grad : nullptr));
+  if (grad && !dout)
+    EGPE_CUDA(cudaMemcpyAsync(grad, base_->hp[0], 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  return EGPE_OK;
+}
+
+template <class R> void Engine<R>::energy_out(const DevState& hs, egpe_energy_terms& out) const {
+  EnergyOut o;
+  finalize_energy(hs.eg[0], hs.egz[0], hs.dV, o);
+  out.E = o.E;
+  for (int i = 0; i < 2; ++i) {
+    out.kin[i] = o.kin[i];
+    out.mu[i] = o.mu[i];
+    out.norm2[i] = o.norm2[i];
+    out.shift[i] = o.shift[i];
+  }
+  out.trap = o.trap;
+  out.contact = o.contact;
+  out.dipolar = o.dipolar;
+  out.lhy = o.lhy;
+}
+
+template <class R> egpe_status Engine<R>::energy_grad(const C* psi, egpe_energy_terms* out, C* grad) {
+  EGPE_TRY(enq_evaluation(psi, grad));
   DevState hs;
   EGPE_TRY(read_state(hs));
-  if (out) {
-    EnergyOut o;
-    finalize_energy(hs.eg[0], hs.egz[0], hs.dV, o);
-    out->E = o.E;
-    for (int i = 0; i < 2; ++i) {
-      out->kin[i] = o.kin[i];
-      out->mu[i] = o.mu[i];
-      out->norm2[i] = o.norm2[i];
-      out->shift[i] = o.shift[i];
-    }
-    out->trap = o.trap;
-    out->contact = o.contact;
-    out->dipolar = o.dipolar;
-    out->lhy = o.lhy;
-  }
+  if (out) energy_out(hs, *out);
   return EGPE_OK;
 }
 
 template <class R> egpe_status Engine<R>::line_coeffs(const C* psi, const C* p, double coeffs[3]) {
-  egpe_energy_terms t;
-  EGPE_TRY(energy_grad(psi, &t, nullptr));
+  EGPE_TRY(enq_evaluation(psi, nullptr));
   EGPE_CUDA(cudaMemcpyAsync(base_->pb[0], p, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(enq_lc(GATE_ALWAYS, 0, 1));
   DevState hs;
   EGPE_TRY(read_state(hs));
+  egpe_energy_terms t;
+  energy_out(hs, t);
   LineOut o;
   finalize_line(hs.lc, hs.lcz, hs.mu, hs.dV, o);
   coeffs[0] = t.E;
@@ -1104,12 +1124,13 @@ template <class R> egpe_status Engine<R>::line_coeffs(const C* psi, const C* p, 
 }
 
 template <class R> egpe_status Engine<R>::precondition(int mode, const C* psi, const C* r, C* z) {
-  EGPE_TRY(energy_grad(psi, nullptr, nullptr));
+  EGPE_TRY(enq_evaluation(psi, nullptr));
   if (r) EGPE_CUDA(cudaMemcpyAsync(base_->rb[0], r, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
-  EGPE_TRY(enq_pc(mode, GATE_ALWAYS, 0, r ? 1 : 0));
-  EGPE_CUDA(cudaMemcpyAsync(z, base_->z, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
-  EGPE_CUDA(cudaStreamSynchronize(stream));
-  return EGPE_OK;
+  const bool dz = element_aligned(z);
+  EGPE_TRY(enq_pc(mode, GATE_ALWAYS, 0, r ? 1 : 0, ATT_FULL, dz ? z : nullptr));
+  if (!dz) EGPE_CUDA(cudaMemcpyAsync(z, base_->z, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  DevState hs;
+  return read_state(hs);
 }
 
 template <class R> egpe_status Engine<R>::retract(const C* psi, const C* p, const double theta[2], C* out) {

@@ -52,8 +52,8 @@ template <class R> struct KArgs {
   C* tb[2];                  // T psi of the psi buffers (attempts that carry it along)
   C* tp[2];                  // T p of the direction buffers
   C* wz;                     // P_V^{-1} r, where T z = wz - alpha z
-  const C* gin;              // generic in/out of the plain passes
-  C* gout;
+  const C* gin;              // generic in/out of the plain passes; standalone evaluations: the caller's psi
+  C* gout;                   // (copied to the psi buffer on the way) and gradient
   double* partials;
   unsigned* counter;
   DevState* st;
@@ -719,7 +719,7 @@ template <class R_, int L_> struct XFwdEG {
   using R = R_;
   using C = C2<R>;
   static constexpr const char* NAME = "x-fwd energy";
-  static double alg_bytes(const KArgs<R>& a) { return (a.flag ? 9.0 : 5.0) * a.N * sizeof(C); }
+  static double alg_bytes(const KArgs<R>& a) { return (a.flag ? 9.0 : a.gin ? 7.0 : 5.0) * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 3, NS = 0;
   static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   using Uni = EgUni<R>;
@@ -742,7 +742,7 @@ template <class R_, int L_> struct XFwdEG {
     return cmk<C>(fma_(a.d12, n2, a.d11 * n1), fma_(a.d22, n2, a.d21 * n1));
   }
   static __device__ C point(const KArgs<R>& a, const Uni& u, int i, size_t idx) {
-    const C p = pick(a.psi, u.cur)[(size_t)i * a.N + idx];
+    const C p = (a.gin ? a.gin : pick(a.psi, u.cur))[(size_t)i * a.N + idx];
     if (!a.flag) return p;
     const C q = pick(a.pb, u.nsel)[(size_t)i * a.N + idx];
     return cmk<C>(fma_(pick(u.cb, i), q.x, pick(u.ca, i) * p.x), fma_(pick(u.cb, i), q.y, pick(u.ca, i) * p.y));
@@ -761,7 +761,7 @@ template <class R_, int L_> struct XFwdEG {
       if (f < 2) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[0][e] = point(a, u, f, base + Plan<L>::entry_pos(false, t, e));
-        if (a.flag) {
+        if (a.flag || a.gin) {
           C* dst = pick(a.psi, u.slot) + (size_t)f * N + base;
 #pragma unroll
           for (int e = 0; e < 8; ++e) dst[Plan<L>::entry_pos(false, t, e)] = v[0][e];
@@ -776,7 +776,7 @@ template <class R_, int L_> struct XFwdEG {
     } else {
       // both components at once, the loads of a chunk before its arithmetic
       constexpr int CH = ChunkW<R>::v;
-      const C* src = pick(a.psi, u.cur);
+      const C* src = a.gin ? a.gin : pick(a.psi, u.cur);
       const C* pd = pick(a.pb, u.nsel);
       C* dst = pick(a.psi, u.slot);
 #pragma unroll
@@ -798,11 +798,13 @@ template <class R_, int L_> struct XFwdEG {
           if (a.flag) {
             p1 = cmk<C>(fma_(u.cb[0], q1[j].x, u.ca[0] * p1.x), fma_(u.cb[0], q1[j].y, u.ca[0] * p1.y));
             p2 = cmk<C>(fma_(u.cb[1], q2[j].x, u.ca[1] * p2.x), fma_(u.cb[1], q2[j].y, u.ca[1] * p2.y));
+            v[0][e0 + j] = p1;
+            v[1][e0 + j] = p2;
+          }
+          if (a.flag || a.gin) {
             const size_t idx = base + Plan<L>::entry_pos(false, t, e0 + j);
             dst[idx] = p1;
             dst[N + idx] = p2;
-            v[0][e0 + j] = p1;
-            v[1][e0 + j] = p2;
           }
           v[2][e0 + j] = source(a, p1, p2);
         }
@@ -980,8 +982,14 @@ template <class R_, int L_, bool LIN> struct XInvEGT {
       const R c1 = fma_(a.g12, n2[j], a.g11 * n1[j]), c2 = fma_(a.g22, n2[j], a.g21 * n1[j]);
       const R B1 = (V + c1) + m1[j], B2 = (V + c2) + m2[j];
       const R U1 = B1 + phi1, U2 = B2 + phi2;
-      hp[idx] = cmk<C>(fma_(U1, p1[j].x, T1.x), fma_(U1, p1[j].y, T1.y));
-      hp[N + idx] = cmk<C>(fma_(U2, p2[j].x, T2.x), fma_(U2, p2[j].y, T2.y));
+      const C H1 = cmk<C>(fma_(U1, p1[j].x, T1.x), fma_(U1, p1[j].y, T1.y));
+      const C H2 = cmk<C>(fma_(U2, p2[j].x, T2.x), fma_(U2, p2[j].y, T2.y));
+      hp[idx] = H1;
+      hp[N + idx] = H2;
+      if (!LIN && a.gout) {
+        a.gout[idx] = H1;
+        a.gout[N + idx] = H2;
+      }
       ax[idx] = PH;
       ax[N + idx] = cmk<C>(B1, B2);
       // the energies and mu_i are combinations of these (finalize_energy)
@@ -1820,12 +1828,17 @@ template <class R_, int L_> struct XFwdPG {
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { u.cur = __ldcg(&a.st->cur); }
   template <int NV>
   static __device__ void load(const KArgs<R>& a, Uni& u, int, int row, bool valid, int t, C (&v)[NV][8]) {
-    const C* ps = pick(a.psi, u.cur);
+    const C* ps = a.gin ? a.gin : pick(a.psi, u.cur);
+    C* dst = pick(a.psi, u.cur);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const size_t idx = valid ? (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e) : 0;
       const C p1 = ps[idx], p2 = ps[(size_t)a.N + idx];
       v[0][e] = valid ? cmk<C>(cabs2(p1), cabs2(p2)) : cmk<C>(0, 0);
+      if (a.gin && valid) {
+        dst[idx] = p1;
+        dst[(size_t)a.N + idx] = p2;
+      }
     }
   }
   template <int NV>
