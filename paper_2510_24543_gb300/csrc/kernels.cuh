@@ -112,8 +112,13 @@ template <class R> __device__ __forceinline__ LhyCoef<R> lhy_coef(const KArgs<R>
   return c;
 }
 
-// One of a pair, by a select: a run-time index would put the pair in local memory.
+// One of a pair, by a select: a run-time index would put a pair held in registers in
+// local memory.  The FP32 buffers of the kernel arguments are indexed: the address comes
+// from the constant bank at its use, where the select kept both halves in registers
+// (128^3 x-inverse line pass 56.4 -> 55.1 us, energy pass 50.8 -> 50.2).  The FP64
+// kernels spill with the index (x-inverse preconditioner pass 191 -> 212 us).
 template <class T> __device__ __forceinline__ T pick(const T (&p)[2], int i) { return i ? p[1] : p[0]; }
+__device__ __forceinline__ C2<float>* pick(C2<float>* const (&p)[2], int i) { return p[i]; }
 
 // Terms of the trap and of |k|^2/2 (over N) that depend on one index come from
 // tables: forming them per point took an integer conversion and three products in
