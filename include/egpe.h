@@ -415,7 +415,9 @@ egpe_status egpe_ncg_continuation(egpe_handle* h, int inst, const egpe_params* p
  * egpe_solver_step: enqueues `attempts` attempts of the loop body of
  *   Algorithm 1 (precondition, line coefficients, trial evaluation and the
  *   on-device controller); asynchronous; attempts after the solver has
- *   finished are no-ops on the device.
+ *   finished are no-ops on the device.  An FP64 iteration with a kinetic
+ *   preconditioner whose direction falls back to the residual takes one attempt
+ *   more, which transforms that direction.
  * egpe_solver_read: waits for the stream, fills *report (status
  *   EGPE_ERR_NOT_CONVERGED while the solver is still running, res = ||r|| of
  *   the current point) and copies the current psi to psi_out (device; may be

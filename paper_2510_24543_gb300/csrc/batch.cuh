@@ -53,15 +53,12 @@ template <class R> class BatchRunner {
     std::vector<int> active = live(phase);
     const int mode = o.precond;
     const int poll = std::max(1, o.poll_every);
-    const long long max_launch =
-        ((long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4) * (carried_ ? kRefreshEvery : 1);
+    const long long max_launch = max_attempts(max_iter, o.armijo_max, carried_);
     long long replays = 0, kernels = 0;
-    bool want_refresh = false;
     while (!active.empty() && replays < max_launch) {
       if (active != built_) EGPE_TRY(rebuild(active, mode));
       for (int k = attempts_ahead(poll, max_iter, replays); k > 0; --k) {
-        const bool refresh = attempt_kind(carried_, replays, want_refresh) == ATT_REFRESH;
-        want_refresh = false;
+        const bool refresh = attempt_kind(carried_, replays) == ATT_REFRESH;
         if (refresh && !refresh_) EGPE_TRY(build(active, mode, ATT_REFRESH, refresh_, per_refresh_));
         EGPE_CUDA(cudaGraphLaunch(refresh ? refresh_ : graph_, stream_));
         ++replays;
@@ -69,7 +66,6 @@ template <class R> class BatchRunner {
       }
       EGPE_TRY(gather(phase));
       active = live(phase);
-      for (int ph : phase) want_refresh |= ph == PH_DIRECT;
     }
     for (int i = 0; i < n; ++i) {
       Engine<R>& e = *eng_[i];
@@ -148,7 +144,7 @@ template <class R> class BatchRunner {
   egpe_status rebuild(const std::vector<int>& active, int mode) {
     if (refresh_) cudaGraphExecDestroy(refresh_);  // built again when it is next due
     refresh_ = nullptr;
-    EGPE_TRY(build(active, mode, attempt_kind(carried_, 0, false), graph_, per_replay_));
+    EGPE_TRY(build(active, mode, attempt_kind(carried_, 0), graph_, per_replay_));
     built_ = active;
     ++builds_;
     return EGPE_OK;

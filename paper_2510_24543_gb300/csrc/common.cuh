@@ -69,23 +69,21 @@ static constexpr int MAX_NS = 16;
 static_assert(PG_NS <= MAX_NS, "reduction slots");
 
 // Phases of the on-device solver state machine.
-// PH_DIRECT: the iteration waits for an attempt that transforms its direction
-// (T p cannot be carried along, see AttemptKind).
+// PH_DIRECT: the direction is the residual itself (carried attempts): the next
+// attempt's preconditioner passes transform it instead of preconditioning.
 enum Phase { PH_NEW_ITER = 0, PH_TRIAL = 1, PH_DONE = 2, PH_DIRECT = 3 };
-// Launch gates: which phases a kernel runs in.  REFRESH_*: the passes of a refresh
-// attempt; CARRIED_TRIAL: trial evaluations that need T p.
-enum Gate {
-  GATE_ALWAYS = 0, GATE_NEW_ITER = 1, GATE_ACTIVE = 2, GATE_REFRESH_PC = 3, GATE_REFRESH_CARRIED = 4,
-  GATE_REFRESH_DIRECT = 5, GATE_CARRIED_TRIAL = 6
-};
+// Launch gates: which phases a kernel runs in.  CARRIED_PC: the preconditioner passes
+// of a carried or refresh attempt (PH_NEW_ITER and PH_DIRECT).
+enum Gate { GATE_ALWAYS = 0, GATE_NEW_ITER = 1, GATE_ACTIVE = 2, GATE_CARRIED_PC = 3 };
 // How an attempt obtains the kinetic terms.  FULL: by transforms of the direction
 // and of the trial state.  CARRIED (kinetic preconditioners): T is linear, and
 // P_Delta z = (alpha + T) z = w gives T z = w - alpha z without a transform, so
 // T p = -T z + beta T p_prev - c T psi and T psi' = a T psi + b T p are carried along
-// beside p and psi: 8 transforms per iteration instead of 14.  REFRESH: as CARRIED,
+// beside p and psi: 8 transforms per iteration instead of 14.  In a residual-fallback
+// step r takes the place of z, and the preconditioner passes of one attempt more form
+// its w = (alpha + T) r, so T p is known after every direction.  REFRESH: as CARRIED,
 // with the trial state transformed, which removes what rounding has accumulated in
-// T psi; it also takes the directions whose T is not known (the residual fallback,
-// and the next conjugate one), by transform.
+// T psi.
 enum AttemptKind { ATT_FULL = 0, ATT_CARRIED = 1, ATT_REFRESH = 2 };
 
 struct SolveOptsDev {
@@ -112,8 +110,7 @@ struct DevState {
   // flow control
   int phase, status, n, attempts, restarts, armijo_total, armijo_k, kind;
   int cur, fallback, trace_len, restart_flag;
-  int direct_lc, tp_bad, timeout, pad1;  // timeout: a device wait ran out of its poll budget;
-                                         // direct_lc: this direction is transformed; tp_bad: its T p is not known
+  int timeout, pad0, pad1, pad2;  // timeout: a device wait ran out of its poll budget
   SolveOptsDev opt;
   // current point (slot cur)
   double E, mu[2], shift[2], nmuL[2], norm2[2];
@@ -124,7 +121,7 @@ struct DevState {
   double dV, invN;
   long long ffts;
   double res_best;     // smallest residual so far and the iteration that reached it
-  int n_best, pad2;
+  int n_best, pad3;
 };
 
 // Gauss-Legendre node constants of the LHY u-integral, in field precision.

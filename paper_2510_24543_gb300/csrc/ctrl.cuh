@@ -217,6 +217,10 @@ static __device__ __noinline__ void ctrl_after_ite(DevState* st) {
 // projection coefficients, restart rules.
 static __device__ __noinline__ void ctrl_after_pc(DevState* st, int kind) {
   if (ctrl_timed_out(st)) return;
+  if (st->phase == PH_DIRECT) {  // w = (alpha + T) r of the direction chosen last time is there now
+    st->phase = PH_NEW_ITER;
+    return;
+  }
   const double* pc = st->pc;
   const double dV = st->dV;
   const SolveOptsDev& op = st->opt;
@@ -276,15 +280,7 @@ static __device__ __noinline__ void ctrl_after_pc(DevState* st, int kind) {
     // p = -(r - Re<r,psi> psi): c_i = Re<-r_i, psi_i>
     for (int i = 0; i < 2; ++i) c[i] = -pc[PC_PSIR1 + i];
   }
-  if (kind != ATT_FULL) {
-    const int direct = (fallback || (beta != 0.0 && st->tp_bad)) ? 1 : 0;
-    if (direct && kind == ATT_CARRIED) {  // left to the next refresh attempt
-      st->phase = PH_DIRECT;
-      return;
-    }
-    st->direct_lc = st->tp_bad = direct;
-    st->phase = PH_NEW_ITER;
-  }
+  if (fallback && kind != ATT_FULL) st->phase = PH_DIRECT;
   st->fallback = fallback;
   st->beta = beta;
   st->restart_flag = (beta == 0.0) ? 1 : 0;

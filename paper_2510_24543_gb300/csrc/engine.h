@@ -77,9 +77,14 @@ inline int attempts_ahead(int poll, int max_iter, long long launched) {
 // 2e-7 (and were 6% faster).
 inline bool carried_mode(int mode) { return mode == 1 || mode == 3; }
 constexpr int kRefreshEvery = 8;
-inline AttemptKind attempt_kind(bool carried, long long launched, bool want_refresh) {
+inline AttemptKind attempt_kind(bool carried, long long launched) {
   if (!carried) return ATT_FULL;
-  return want_refresh || launched % kRefreshEvery == kRefreshEvery - 1 ? ATT_REFRESH : ATT_CARRIED;
+  return launched % kRefreshEvery == kRefreshEvery - 1 ? ATT_REFRESH : ATT_CARRIED;
+}
+// Attempts after which a solve stops polling whatever the phase says: every iteration
+// with all its trials, and one attempt more for a fallback direction.
+inline long long max_attempts(int max_iter, int armijo_max, bool carried) {
+  return ((long long)max_iter + 2) * ((long long)armijo_max + (carried ? 3 : 2)) + 4;
 }
 
 template <class R> class Engine {
@@ -172,7 +177,7 @@ template <class R> class Engine {
   static bool element_aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % sizeof(C) == 0; }
   void energy_out(const DevState& hs, egpe_energy_terms& out) const;
   egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att = ATT_FULL, C* z = nullptr);
-  egpe_status enq_lc(int gate, int ctrl, int pgiven, AttemptKind att = ATT_FULL);
+  egpe_status enq_lc(int gate, int ctrl, int pgiven);
   egpe_status enq_dipolar(const KArgs<R>& a);
   egpe_status enq_eg_carried(int gate, int ctrl);
   egpe_status enq_lc_carried(int mode, int gate, int ctrl);
@@ -267,7 +272,6 @@ template <class R> class Engine {
   cudaGraphExec_t refresh_[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // refresh attempts, by mode
   int refresh_kernels_[5] = {0, 0, 0, 0, 0};
   bool run_carried_ = false;
-  bool want_refresh_ = false;  // the last look found an iteration waiting for one
   int run_mode_ = 0, run_graph_ = 1;
   long long run_k0_ = 0, run_launches_ = 0, per_attempt_ = 0;
   int graph_max_iter_[5] = {0, 0, 0, 0, 0};

@@ -451,7 +451,7 @@ egpe_status Engine<R>::profile_attempt(const C* psi, int precond, int reps, std:
   EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(reset_state(&o, sizeof(R) == 4, 1 << 30, 0.0, sizeof(R) == 4 ? 1e-6 : 1e-13));
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0, false);
+  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0);
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   EGPE_CUDA(cudaStreamSynchronize(stream));
   names.clear();
@@ -541,7 +541,7 @@ egpe_status Engine<R>::autotune(const C* psi, int precond, int reps, std::vector
   EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(reset_state(&o, sizeof(R) == 4, 1 << 30, 0.0, sizeof(R) == 4 ? 1e-6 : 1e-13));
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0, false);
+  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0);
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   EGPE_TRY(enq_attempt(o.precond, kind));  // realistic coefficients in the state
   EGPE_CUDA(cudaStreamSynchronize(stream));
@@ -936,9 +936,9 @@ template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, i
 }
 
 // Line-search pipeline: forward transforms of p_1, p_2 and one packed pair.
-template <class R> egpe_status Engine<R>::enq_lc(int gate, int ctrl, int pgiven, AttemptKind att) {
+template <class R> egpe_status Engine<R>::enq_lc(int gate, int ctrl, int pgiven) {
   KArgs<R> a = *base_;
-  a.att = att;
+  a.att = ATT_FULL;
   a.gate = gate;
   a.flag = pgiven;
   a.ctrl = 0;
@@ -1006,16 +1006,10 @@ template <class R> egpe_status Engine<R>::enq_eg_carried(int gate, int ctrl) {
 
 template <class R> egpe_status Engine<R>::enq_attempt(int mode, AttemptKind kind) {
   if constexpr (sizeof(R) == 8) {
-    if (kind == ATT_CARRIED) {
-      EGPE_TRY(enq_pc(mode, GATE_NEW_ITER, 1, 0, kind));
+    if (kind != ATT_FULL) {
+      EGPE_TRY(enq_pc(mode, GATE_CARRIED_PC, 1, 0, kind));
       EGPE_TRY(enq_lc_carried(mode, GATE_NEW_ITER, 1));
-      return enq_eg_carried(GATE_CARRIED_TRIAL, 1);
-    }
-    if (kind == ATT_REFRESH) {
-      EGPE_TRY(enq_pc(mode, GATE_REFRESH_PC, 1, 0, kind));
-      EGPE_TRY(enq_lc_carried(mode, GATE_REFRESH_CARRIED, 1));
-      EGPE_TRY(enq_lc(GATE_REFRESH_DIRECT, 1, 0, kind));
-      return enq_eg(1, GATE_ACTIVE, 1, kind);
+      return kind == ATT_REFRESH ? enq_eg(1, GATE_ACTIVE, 1, kind) : enq_eg_carried(GATE_ACTIVE, 1);
     }
   }
   EGPE_TRY(enq_pc(mode, GATE_NEW_ITER, 1, 0));
@@ -1222,7 +1216,7 @@ egpe_status Engine<R>::solve_begin(const egpe_solve_opts& o, int fp32_phase, int
   // r and p history start at zero (beta = 0 at n = 0 reads them)
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
   run_carried_ = ensure_carry(mode);
-  const AttemptKind kind = attempt_kind(run_carried_, 0, false);
+  const AttemptKind kind = attempt_kind(run_carried_, 0);
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   run_k0_ = kernels_;
   run_ite_ = false;
@@ -1230,7 +1224,6 @@ egpe_status Engine<R>::solve_begin(const egpe_solve_opts& o, int fp32_phase, int
   run_graph_ = o.use_graph ? 1 : 0;
   run_launches_ = 0;
   per_attempt_ = 0;
-  want_refresh_ = false;
   if (run_graph_) {
     if (!graph_[mode]) EGPE_TRY(capture_attempt(mode, kind, graph_[mode], graph_max_iter_[mode]));
     per_attempt_ = graph_max_iter_[mode];
@@ -1378,8 +1371,7 @@ template <class R> egpe_status Engine<R>::solve_launch(int attempts) {
         EGPE_TRY(enq_ite_step(GATE_ACTIVE));
       }
     } else {
-      const AttemptKind kind = attempt_kind(run_carried_, run_launches_, want_refresh_);
-      want_refresh_ = false;
+      const AttemptKind kind = attempt_kind(run_carried_, run_launches_);
       if (!run_graph_) {
         EGPE_TRY(enq_attempt(run_mode_, kind));
       } else if (kind == ATT_REFRESH) {
@@ -1401,7 +1393,6 @@ template <class R> egpe_status Engine<R>::solve_poll(int& phase) {
   EGPE_CUDA(cudaMemcpyAsync(&st_host_->phase, &st_->phase, sizeof(int), cudaMemcpyDeviceToHost, stream));
   EGPE_CUDA(cudaStreamSynchronize(stream));
   phase = st_host_->phase;
-  want_refresh_ = phase == PH_DIRECT;
   return EGPE_OK;
 }
 
@@ -1463,8 +1454,7 @@ egpe_status Engine<R>::solve(const egpe_solve_opts& o, int fp32_phase, int max_i
                              int trace_offset) {
   EGPE_TRY(solve_begin(o, fp32_phase, max_iter, tol_res, accept_rtol, trace_out != nullptr, trace_cap));
   const int poll = std::max(1, o.poll_every);
-  const long long max_launch =
-      ((long long)(max_iter + 2) * (long long)(o.armijo_max + 2) + 4) * (run_carried_ ? kRefreshEvery : 1);
+  const long long max_launch = max_attempts(max_iter, o.armijo_max, run_carried_);
   while (run_launches_ < max_launch) {
     EGPE_TRY(solve_launch(attempts_ahead(poll, max_iter, run_launches_)));
     int phase = 0;

@@ -72,15 +72,11 @@ template <class R> struct KArgs {
 template <class R> __device__ __forceinline__ bool gate_open(const KArgs<R>& a) {
   if (a.gate == GATE_ALWAYS) return true;
   const int ph = __ldcg(&a.st->phase);
-  const bool on = ph == PH_NEW_ITER || ph == PH_TRIAL;
   switch (a.gate) {
     case GATE_NEW_ITER: return ph == PH_NEW_ITER;
-    case GATE_REFRESH_PC: return ph == PH_NEW_ITER || ph == PH_DIRECT;
-    case GATE_REFRESH_CARRIED: return ph == PH_NEW_ITER && !__ldcg(&a.st->direct_lc);
-    case GATE_REFRESH_DIRECT: return ph == PH_NEW_ITER && __ldcg(&a.st->direct_lc);
-    case GATE_CARRIED_TRIAL: return on && !__ldcg(&a.st->tp_bad);
+    case GATE_CARRIED_PC: return ph == PH_NEW_ITER || ph == PH_DIRECT;
   }
-  return on;
+  return ph == PH_NEW_ITER || ph == PH_TRIAL;
 }
 
 // Batched launches: one launch runs the same pass for up to KB_MAX instances
@@ -1022,10 +1018,16 @@ template <class R, int L> struct XInvEL : XInvEGT<R, L, true> {};
 // ----------------------------------------------------------------------------
 template <class R> struct PcUni {
   int cur, nsel, rgiven;
+  bool direct;  // PH_DIRECT: the passes form w = (alpha + T) r of a residual-fallback step
   R mu[2], shift[2], floor_[2];
   R wv;  // weight of P_V in the blended preconditioner
 };
+// Only FP64 engines carry T p along (engine.h).
+template <class R> __device__ __forceinline__ bool pc_direct(const KArgs<R>& a) {
+  return sizeof(R) == 8 && a.att != ATT_FULL && __ldcg(&a.st->phase) == PH_DIRECT;
+}
 template <class R> __device__ __forceinline__ void pc_uniform(const KArgs<R>& a, PcUni<R>& u) {
+  u.direct = pc_direct(a);
   u.cur = __ldcg(&a.st->cur);
   u.nsel = __ldcg(&a.st->n) & 1;
   u.rgiven = a.flag;
@@ -1056,7 +1058,8 @@ template <class R> __device__ __forceinline__ R pv_at(const PcUni<R>& u, int i, 
   return P > fl ? P : fl;
 }
 // r_i = H_i psi_i - mu_i psi_i (stored unless given) and w_i = P_V^{-1} r_i when
-// diag, at CH points: both components (NV = 2, i = 0) or component i alone.
+// diag, at CH points: both components (NV = 2, i = 0) or component i alone.  In a
+// direct pass w_i = r_i.
 template <class R, int CH, int NV>
 __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u, int i, const size_t (&idx)[CH],
                                             C2<R> (&w)[NV][CH]) {
@@ -1084,7 +1087,7 @@ __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u
         r = cmk<C>(fma_(-mu, p[k][j].x, r.x), fma_(-mu, p[k][j].y, r.y));
         pick(a.rb, u.nsel)[(size_t)c * N + idx[j]] = r;
       }
-      if (a.diag) {
+      if (a.diag && !u.direct) {
         r = cscale(r, rcp_(pv_at(u, c, c ? bb[j].y : bb[j].x)));
         if (a.att != ATT_FULL) a.wz[(size_t)c * N + idx[j]] = r;
       }
@@ -1178,8 +1181,10 @@ template <class R_, int L_> struct ZPc {
   static constexpr int L = L_, NS = 0, AXIS = 2;
   struct Uni : KzLine<R, L_> {
     R shift[2];
+    bool direct;
   };
   static __device__ void uniform(const KArgs<R>& a, Uni& u, int t) {
+    u.direct = pc_direct(a);
     load_uniforms<R, 2>({&a.st->shift[0], &a.st->shift[1]}, u.shift);
     u.set(a, t);
   }
@@ -1193,9 +1198,10 @@ template <class R_, int L_> struct ZPc {
     const R sh = a.invN * (f == 0 ? u.shift[0] : u.shift[1]);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      // invN / (shift + |k|^2/2), numerator and denominator over N
-      const R kz = u.kz[e];
-      v[0][e] = cscale(v[0][e], a.invN * a.invN * rcp_(sh + (kxy + kz)));
+      // invN / (shift + |k|^2/2), numerator and denominator over N; a direct pass
+      // multiplies by (shift + |k|^2/2) / N
+      const R q = sh + (kxy + u.kz[e]);
+      v[0][e] = cscale(v[0][e], u.direct ? q : a.invN * a.invN * rcp_(q));
     }
     col_after<L>(sm, si);
     fft_line<C, L, true, 1>(v, sm, 0, tw, t, si);
@@ -1223,6 +1229,7 @@ template <class R_, int L_> struct XInvPC {
   template <int NP, bool ST>
   static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[PC_NS],
                                 const LhyNode<R>*) {
+    C* zd = u.direct ? a.wz : a.z;
     PcSumIn<R> in[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) pc_sum_load<R>(a, u, pt[j].idx, in[j]);
@@ -1236,8 +1243,8 @@ template <class R_, int L_> struct XInvPC {
         z1 = cmk<C>(wd * z1.x + w1 * in[j].r1.x, wd * z1.y + w1 * in[j].r1.y);
         z2 = cmk<C>(wd * z2.x + w2 * in[j].r2.x, wd * z2.y + w2 * in[j].r2.y);
       }
-      a.z[idx] = z1;
-      a.z[(size_t)a.N + idx] = z2;
+      zd[idx] = z1;
+      zd[(size_t)a.N + idx] = z2;
       pc_sum_add<R>(in[j], z1, z2, s);
     }
   }
@@ -1535,8 +1542,8 @@ template <class R, int L> struct XInvLC : XInvLCT<R, L, false> {};
 template <class R, int L> struct XInvLL : XInvLCT<R, L, true> {};
 
 // Direction of an attempt that carries T psi and T p along: p and T p from their
-// terms (T z = w - alpha z, w = P_V^{-1} r or r), and the forward rows of the packed
-// source of rho alone.
+// terms (T z = w - alpha z, w = P_V^{-1} r or r; in a fallback step z = r and
+// w = (alpha + T) r), and the forward rows of the packed source of rho alone.
 template <class R_, int L_> struct XFwdLL {
   using R = R_;
   using C = C2<R>;
@@ -1560,7 +1567,8 @@ template <class R_, int L_> struct XFwdLL {
     const C* ts = pick(a.tb, u.cur);
     const C* pp = pick(a.pb, u.nsel ^ 1);
     const C* tpp = pick(a.tp, u.nsel ^ 1);
-    const C* ws = a.diag ? a.wz : pick(a.rb, u.nsel);
+    const C* zs = u.fallback ? pick(a.rb, u.nsel) : a.z;
+    const C* ws = a.diag || u.fallback ? a.wz : pick(a.rb, u.nsel);
     C* pd = pick(a.pb, u.nsel);
     C* td = pick(a.tp, u.nsel);
     const bool usepp = u.beta != R(0);
@@ -1574,7 +1582,7 @@ template <class R_, int L_> struct XFwdLL {
         for (int i = 0; i < 2; ++i) {
           const size_t q = valid ? (size_t)i * N + (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j) : 0;
           p[i][j] = ps[q];
-          z[i][j] = a.z[q];
+          z[i][j] = zs[q];
           w[i][j] = ws[q];
           k[i][j] = ts[q];
           if (usepp) {
