@@ -742,11 +742,17 @@ template <class R_, int L_> struct XFwdEG {
     const R n1 = cabs2(p1), n2 = cabs2(p2);
     return cmk<C>(fma_(a.d12, n2, a.d11 * n1), fma_(a.d22, n2, a.d21 * n1));
   }
+  // ca p + cb q.  The large term is the exact product inside the FMA: rounded on its
+  // own, ca p (ca within a few units of 1 near convergence) is off in one direction
+  // at nearly every point, and the FP32 norms after a solve drift with it.
+  static __device__ C trial(R ca, C p, R cb, C q) {
+    return cmk<C>(fma_(ca, p.x, cb * q.x), fma_(ca, p.y, cb * q.y));
+  }
   static __device__ C point(const KArgs<R>& a, const Uni& u, int i, size_t idx) {
     const C p = (a.gin ? a.gin : pick(a.psi, u.cur))[(size_t)i * a.N + idx];
     if (!a.flag) return p;
     const C q = pick(a.pb, u.nsel)[(size_t)i * a.N + idx];
-    return cmk<C>(fma_(pick(u.cb, i), q.x, pick(u.ca, i) * p.x), fma_(pick(u.cb, i), q.y, pick(u.ca, i) * p.y));
+    return trial(pick(u.ca, i), p, pick(u.cb, i), q);
   }
   template <int NV>
   static __device__ void load(const KArgs<R>& a, Uni& u, int f, int row, bool valid, int t, C (&v)[NV][8]) {
@@ -797,8 +803,8 @@ template <class R_, int L_> struct XFwdEG {
         for (int j = 0; j < CH; ++j) {
           C p1 = v[0][e0 + j], p2 = v[1][e0 + j];
           if (a.flag) {
-            p1 = cmk<C>(fma_(u.cb[0], q1[j].x, u.ca[0] * p1.x), fma_(u.cb[0], q1[j].y, u.ca[0] * p1.y));
-            p2 = cmk<C>(fma_(u.cb[1], q2[j].x, u.ca[1] * p2.x), fma_(u.cb[1], q2[j].y, u.ca[1] * p2.y));
+            p1 = trial(u.ca[0], p1, u.cb[0], q1[j]);
+            p2 = trial(u.ca[1], p2, u.cb[1], q2[j]);
             v[0][e0 + j] = p1;
             v[1][e0 + j] = p2;
           }
@@ -1664,12 +1670,11 @@ template <class R_, int L_> struct XFwdEL {
         R n[2];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-          const R ca = u.ca[i], cb = u.cb[i];
-          const C x = cmk<C>(fma_(cb, q[i][j].x, ca * p[i][j].x), fma_(cb, q[i][j].y, ca * p[i][j].y));
+          const C x = XFwdEG<R, L>::trial(u.ca[i], p[i][j], u.cb[i], q[i][j]);
           if (valid) {
             const size_t o = (size_t)i * N + (size_t)row * a.nx + Plan<L>::entry_pos(false, t, e0 + j);
             po[o] = x;
-            to[o] = cmk<C>(fma_(cb, tq[i][j].x, ca * k[i][j].x), fma_(cb, tq[i][j].y, ca * k[i][j].y));
+            to[o] = XFwdEG<R, L>::trial(u.ca[i], k[i][j], u.cb[i], tq[i][j]);
           }
           n[i] = valid ? cabs2(x) : R(0);
         }
