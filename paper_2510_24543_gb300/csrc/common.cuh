@@ -44,7 +44,7 @@ enum EgSlot {  // pointwise part of one energy/gradient evaluation (x dV later):
   // int of n_i V, n_i sum_j g_ij n_j, n_i Phi_i, n_i mu_LHY,i, n_i
   EG_TRAP1 = 0, EG_TRAP2, EG_CON1, EG_CON2, EG_NPHI1, EG_NPHI2,
   EG_NMUL1, EG_NMUL2, EG_NORM1, EG_NORM2,
-  EG_KIN1, EG_KIN2,  // <psi_i, T psi_i> where T psi is carried along (else Parseval, EgzSlot)
+  EG_KIN1, EG_KIN2,  // <psi_i, T psi_i> where T psi is carried along (else Parseval, EgzSlot, and no such sums)
   EG_NS
 };
 enum EgzSlot { EGZ_KIN1 = 0, EGZ_KIN2, EGZ_NS };  // Parseval sums of the z pass

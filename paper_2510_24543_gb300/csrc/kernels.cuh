@@ -942,7 +942,7 @@ template <class R_, int L_, bool LIN> struct XInvEGT {
   static constexpr bool STAGE_OUT = true;
   static constexpr const char* NAME = "x-inv energy+LHY";
   static double alg_bytes(const KArgs<R>& a) { return (LIN || a.att == ATT_FULL ? 9.0 : 11.0) * a.N * sizeof(C); }
-  static constexpr int L = L_, NF = LIN ? 1 : 3, NS = EG_NS;
+  static constexpr int L = L_, NF = LIN ? 1 : 3, NS = LIN ? EG_NS : EG_KIN1;
   static constexpr bool INV = true, USES_LHY = true, LHY_TAB = true, POINTS = true;
   using Uni = EgUni<R>;
   static __device__ void uniform(const KArgs<R>& a, Uni& u) { XFwdEG<R, L>::uniform(a, u); }
@@ -951,7 +951,7 @@ template <class R_, int L_, bool LIN> struct XInvEGT {
     load_rows<XInvEGT>(a, a.W, f, row, valid, t, v);
   }
   template <int NP, bool ST>
-  static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[EG_NS],
+  static __device__ void points(const KArgs<R>& a, Uni& u, const RowPt<R, NF, ST> (&pt)[NP], R (&s)[NS],
                                 const LhyNode<R>* nodes) {
     const C* ps = pick(a.psi, u.slot);
     C* hp = pick(a.hp, u.slot);
