@@ -120,12 +120,9 @@ __device__ inline void load_point(DevState* st, int slot, int lin) {
   }
 }
 
-// The controller steps are not inlined: one thread of the grid runs them, and
-// inside a pass their FP64 chains would set its register count.
-
 // After an energy/gradient evaluation.  mode 0: evaluation of the current
 // point (start of a solve, or a standalone call); mode 1: trial point.
-static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, int lin, TraceDev* trace) {
+__device__ inline void ctrl_after_eg(DevState* st, int mode, int lin, TraceDev* trace) {
   if (ctrl_timed_out(st)) return;
   if (mode == 0) {
     load_point(st, st->cur, lin);
@@ -195,7 +192,7 @@ static __device__ __noinline__ void ctrl_after_eg(DevState* st, int mode, int li
 
 // End of one imaginary-time step: the energy of the renormalised state, the
 // |E^{k+1} - E^k| < tol_dE stopping rule of the ITE comparison (Sec. VI.A).
-static __device__ __noinline__ void ctrl_after_ite(DevState* st) {
+__device__ inline void ctrl_after_ite(DevState* st) {
   if (ctrl_timed_out(st)) return;
   const double Eold = st->E;
   load_point(st, st->cur, 0);
@@ -215,7 +212,7 @@ static __device__ __noinline__ void ctrl_after_ite(DevState* st) {
 
 // After the preconditioned residual and its sums: convergence test, beta,
 // projection coefficients, restart rules.
-static __device__ __noinline__ void ctrl_after_pc(DevState* st, int kind) {
+__device__ inline void ctrl_after_pc(DevState* st, int kind) {
   if (ctrl_timed_out(st)) return;
   if (st->phase == PH_DIRECT) {  // w = (alpha + T) r of the direction chosen last time is there now
     st->phase = PH_NEW_ITER;
@@ -290,7 +287,7 @@ static __device__ __noinline__ void ctrl_after_pc(DevState* st, int kind) {
 }
 
 // After the line-search sums: E', E'', alpha, theta, retraction coefficients.
-static __device__ __noinline__ void ctrl_after_lc(DevState* st) {
+__device__ inline void ctrl_after_lc(DevState* st) {
   if (ctrl_timed_out(st)) return;
   LineOut o;
   finalize_line(st->lc, st->lcz, st->mu, st->dV, o);
@@ -320,6 +317,29 @@ static __device__ __noinline__ void ctrl_after_lc(DevState* st) {
   st->armijo_k = 0;
   set_retraction(st);
 }
+
+// How the passes of field precision R run the controller steps (one thread of the
+// grid does).  FP64 passes call them: inlined, their FP64 chains would set the pass's
+// register count.  FP32 passes inline them: the call cost the line pass 2 us and the
+// other two x-inverse passes 0.3 and 0.7 us at 128^3 (54.4 -> 52.3, 49.4 -> 49.1,
+// 48.0 -> 47.3).
+template <class R> struct Ctrl;
+template <> struct Ctrl<float> {
+  static __device__ __forceinline__ void after_eg(DevState* st, int mode, int lin, TraceDev* trace) {
+    ctrl_after_eg(st, mode, lin, trace);
+  }
+  static __device__ __forceinline__ void after_ite(DevState* st) { ctrl_after_ite(st); }
+  static __device__ __forceinline__ void after_pc(DevState* st, int kind) { ctrl_after_pc(st, kind); }
+  static __device__ __forceinline__ void after_lc(DevState* st) { ctrl_after_lc(st); }
+};
+template <> struct Ctrl<double> {
+  static __device__ __noinline__ void after_eg(DevState* st, int mode, int lin, TraceDev* trace) {
+    ctrl_after_eg(st, mode, lin, trace);
+  }
+  static __device__ __noinline__ void after_ite(DevState* st) { ctrl_after_ite(st); }
+  static __device__ __noinline__ void after_pc(DevState* st, int kind) { ctrl_after_pc(st, kind); }
+  static __device__ __noinline__ void after_lc(DevState* st) { ctrl_after_lc(st); }
+};
 #endif
 
 }  // namespace egpe

@@ -709,10 +709,10 @@ template <class R> struct EgUni {
 template <class R> __device__ __forceinline__ void eg_ctrl(const KArgs<R>& a, int lin) {
   if (a.ctrl == 2) {
     a.st->ffts += 20;  // two kinetic half steps (8) and two evaluations (12)
-    ctrl_after_ite(a.st);
+    Ctrl<R>::after_ite(a.st);
   } else if (a.ctrl) {
     a.st->ffts += lin ? 2 : 6;
-    ctrl_after_eg(a.st, a.flag ? 1 : 0, lin, a.trace);
+    Ctrl<R>::after_eg(a.st, a.flag ? 1 : 0, lin, a.trace);
   }
 }
 
@@ -1258,7 +1258,7 @@ template <class R_, int L_> struct XInvPC {
   static __device__ void finish(const KArgs<R>& a, Uni&) {
     if (a.ctrl) {
       a.st->ffts += 4;
-      ctrl_after_pc(a.st, a.att);
+      Ctrl<R>::after_pc(a.st, a.att);
     }
   }
 };
@@ -1290,7 +1290,7 @@ __device__ __forceinline__ void pc_point_body(const KArgs<R>& a) {
     for (int k = 0; k < PC_NS; ++k) acc[k].add(s[k]);
   }
   if (reduce_blocks<PC_NS>(acc, a.partials, a.counter, a.st->pc, red)) {
-    if (threadIdx.x == 0 && a.ctrl) ctrl_after_pc(a.st, a.att);
+    if (threadIdx.x == 0 && a.ctrl) Ctrl<R>::after_pc(a.st, a.att);
   }
 }
 template <class R> __global__ void __launch_bounds__(256) pc_point_kernel(KArgs<R> a) { pc_point_body(a); }
@@ -1540,7 +1540,7 @@ template <class R_, int L_, bool LIN> struct XInvLCT {
   static __device__ void finish(const KArgs<R>& a, Uni&) {
     if (a.ctrl) {
       a.st->ffts += LIN ? 2 : 4;
-      ctrl_after_lc(a.st);
+      Ctrl<R>::after_lc(a.st);
     }
   }
 };
