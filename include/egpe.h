@@ -178,7 +178,11 @@ typedef struct {
   int graph_launches;       /* graph replays (or attempt sequences) issued          */
   double E;                 /* final energy                                         */
   double mu[2];             /* final chemical potentials                            */
-  double res;               /* final ||r||                                          */
+  double res;               /* final ||r||.  FP64 runs with a kinetic preconditioner
+                               carry T psi along; one that ends as converged or
+                               stagnated has had its final state transformed, one
+                               cut at max_iter at most 7 iterations earlier (||r||
+                               may lack the rounding of psi, below eps |k|^2/2)     */
   double seconds;           /* wall time of the call                                */
   long long ffts;           /* complex 3D transforms executed                       */
   long long kernels;        /* kernel launches issued (including masked ones)       */
@@ -417,7 +421,8 @@ egpe_status egpe_ncg_continuation(egpe_handle* h, int inst, const egpe_params* p
  *   on-device controller); asynchronous; attempts after the solver has
  *   finished are no-ops on the device.  An FP64 iteration with a kinetic
  *   preconditioner whose direction falls back to the residual takes one attempt
- *   more, which transforms that direction.
+ *   more, which transforms that direction, and such a run that meets its
+ *   tolerance waits for egpe_solver_read to confirm it by transform.
  * egpe_solver_read: waits for the stream, fills *report (status
  *   EGPE_ERR_NOT_CONVERGED while the solver is still running, res = ||r|| of
  *   the current point) and copies the current psi to psi_out (device; may be

@@ -53,11 +53,17 @@ template <class R> class BatchRunner {
     std::vector<int> active = live(phase);
     const int mode = o.precond;
     const int poll = std::max(1, o.poll_every);
-    const long long max_launch = max_attempts(max_iter, o.armijo_max, carried_);
+    const long long max_launch = max_attempts(max_iter, o.armijo_max, poll, carried_);
     long long replays = 0, kernels = 0;
     while (!active.empty() && replays < max_launch) {
       if (active != built_) EGPE_TRY(rebuild(active, mode));
-      for (int k = attempts_ahead(poll, max_iter, replays); k > 0; --k) {
+      bool verify = false;
+      for (int i : active)
+        if (phase[i] == PH_VERIFY) {
+          EGPE_TRY(eng_[i]->enq_verify());
+          verify = true;
+        }
+      for (int k = attempts_ahead(poll, max_iter, replays, verify); k > 0; --k) {
         const bool refresh = attempt_kind(carried_, replays) == ATT_REFRESH;
         if (refresh && !refresh_) EGPE_TRY(build(active, mode, ATT_REFRESH, refresh_, per_refresh_));
         EGPE_CUDA(cudaGraphLaunch(refresh ? refresh_ : graph_, stream_));

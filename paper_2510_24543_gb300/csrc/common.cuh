@@ -71,10 +71,12 @@ static_assert(PG_NS <= MAX_NS, "reduction slots");
 // Phases of the on-device solver state machine.
 // PH_DIRECT: the direction is the residual itself (carried attempts): the next
 // attempt's preconditioner passes transform it instead of preconditioning.
-enum Phase { PH_NEW_ITER = 0, PH_TRIAL = 1, PH_DONE = 2, PH_DIRECT = 3 };
+// PH_VERIFY: a run with carried T psi is about to end on what it says; the host
+// enqueues one evaluation of the current point by transform, and goes on from that.
+enum Phase { PH_NEW_ITER = 0, PH_TRIAL = 1, PH_DONE = 2, PH_DIRECT = 3, PH_VERIFY = 4 };
 // Launch gates: which phases a kernel runs in.  CARRIED_PC: the preconditioner passes
 // of a carried or refresh attempt (PH_NEW_ITER and PH_DIRECT).
-enum Gate { GATE_ALWAYS = 0, GATE_NEW_ITER = 1, GATE_ACTIVE = 2, GATE_CARRIED_PC = 3 };
+enum Gate { GATE_ALWAYS = 0, GATE_NEW_ITER = 1, GATE_ACTIVE = 2, GATE_CARRIED_PC = 3, GATE_VERIFY = 4 };
 // How an attempt obtains the kinetic terms.  FULL: by transforms of the direction
 // and of the trial state.  CARRIED (kinetic preconditioners): T is linear, and
 // P_Delta z = (alpha + T) z = w gives T z = w - alpha z without a transform, so
@@ -110,7 +112,8 @@ struct DevState {
   // flow control
   int phase, status, n, attempts, restarts, armijo_total, armijo_k, kind;
   int cur, fallback, trace_len, restart_flag;
-  int timeout, pad0, pad1, pad2;  // timeout: a device wait ran out of its poll budget
+  int timeout, lin, pad0, pad1;  // timeout: a device wait ran out of its poll budget;
+                                 // lin: H psi of the current point comes from a carried T psi
   SolveOptsDev opt;
   // current point (slot cur)
   double E, mu[2], shift[2], nmuL[2], norm2[2];

@@ -111,6 +111,7 @@ __device__ inline const double* kin_sums(const DevState* st, int slot, int lin) 
 __device__ inline void load_point(DevState* st, int slot, int lin) {
   EnergyOut o;
   finalize_energy(st->eg[slot], kin_sums(st, slot, lin), st->dV, o);
+  st->lin = lin;
   st->E = o.E;
   for (int i = 0; i < 2; ++i) {
     st->mu[i] = o.mu[i];
@@ -120,14 +121,31 @@ __device__ inline void load_point(DevState* st, int slot, int lin) {
   }
 }
 
+// Ends the run as converged or stagnated.  A carried T psi does not see the rounding
+// of psi itself, which |k|^2/2 magnifies in ||r||: the current point is evaluated by
+// transform first (PH_VERIFY), and a run that does not meet its tolerance then goes on.
+__device__ inline void ctrl_end(DevState* st, int status) {
+  st->status = status;
+  st->phase = st->lin ? PH_VERIFY : PH_DONE;
+}
+
 // After an energy/gradient evaluation.  mode 0: evaluation of the current
-// point (start of a solve, or a standalone call); mode 1: trial point.
+// point (start of a solve, a standalone call, or PH_VERIFY); mode 1: trial point.
 __device__ inline void ctrl_after_eg(DevState* st, int mode, int lin, TraceDev* trace) {
   if (ctrl_timed_out(st)) return;
   if (mode == 0) {
+    const bool verify = st->phase == PH_VERIFY;
+    const double Eold = st->E;
     load_point(st, st->cur, lin);
     st->phase = finite_(st->E) ? PH_NEW_ITER : PH_DONE;
-    if (!finite_(st->E)) st->status = 4;  // EGPE_ERR_NONFINITE
+    if (!finite_(st->E)) {
+      st->status = 4;  // EGPE_ERR_NONFINITE
+    } else if (verify) {
+      st->dE_last += st->E - Eold;
+      const bool flat = st->status == 0 && st->opt.tol_dE > 0.0 && st->n > 0 && fabs(st->dE_last) < st->opt.tol_dE;
+      if (flat || st->status == 6) st->phase = PH_DONE;
+      else st->status = 5;  // ||r|| is for the next attempt's preconditioner passes to judge
+    }
     return;
   }
   const int slot = st->cur ^ 1;
@@ -172,16 +190,12 @@ __device__ inline void ctrl_after_eg(DevState* st, int mode, int lin, TraceDev* 
     st->alpha_prev = st->alpha;
     st->n += 1;
     st->phase = PH_NEW_ITER;
-    if (op.tol_dE > 0.0 && fabs(st->dE_last) < op.tol_dE) {
-      st->status = 0;
-      st->phase = PH_DONE;
-    }
+    if (op.tol_dE > 0.0 && fabs(st->dE_last) < op.tol_dE) ctrl_end(st, 0);
   } else {
     st->armijo_k += 1;
     st->armijo_total += 1;
     if (st->armijo_k > op.armijo_max) {
-      st->status = 6;  // EGPE_ERR_STAGNATED
-      st->phase = PH_DONE;
+      ctrl_end(st, 6);  // EGPE_ERR_STAGNATED
       return;
     }
     st->alpha = st->alpha0 / (double)(1ll << st->armijo_k);
@@ -228,8 +242,7 @@ __device__ inline void ctrl_after_pc(DevState* st, int kind) {
     return;
   }
   if (st->res < op.tol_res) {
-    st->status = 0;
-    st->phase = PH_DONE;
+    ctrl_end(st, 0);
     return;
   }
   if (st->n >= op.max_iter) {

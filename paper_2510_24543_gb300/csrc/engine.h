@@ -63,8 +63,10 @@ struct SolveRun {
 };
 
 // Attempts to enqueue before the next look at the phase: `poll`, but none beyond
-// the one that finds max_iter reached unless line-search retries used some up.
-inline int attempts_ahead(int poll, int max_iter, long long launched) {
+// the one that finds max_iter reached unless line-search retries used some up, and
+// one where the last look found a run to verify (most end there).
+inline int attempts_ahead(int poll, int max_iter, long long launched, bool verify) {
+  if (verify) return 1;
   const long long left = (long long)max_iter + 1 - launched;
   return left > 0 && left < poll ? (int)left : poll;
 }
@@ -82,9 +84,10 @@ inline AttemptKind attempt_kind(bool carried, long long launched) {
   return launched % kRefreshEvery == kRefreshEvery - 1 ? ATT_REFRESH : ATT_CARRIED;
 }
 // Attempts after which a solve stops polling whatever the phase says: every iteration
-// with all its trials, and one attempt more for a fallback direction.
-inline long long max_attempts(int max_iter, int armijo_max, bool carried) {
-  return ((long long)max_iter + 2) * ((long long)armijo_max + (carried ? 3 : 2)) + 4;
+// with all its trials, and one attempt more each for a fallback direction and for an
+// end that did not stand up to the transform (which waits for the host's next look).
+inline long long max_attempts(int max_iter, int armijo_max, int poll, bool carried) {
+  return ((long long)max_iter + 2) * ((long long)armijo_max + (carried ? 3ll + poll : 2ll)) + 4;
 }
 
 template <class R> class Engine {
@@ -182,6 +185,9 @@ template <class R> class Engine {
   egpe_status enq_eg_carried(int gate, int ctrl);
   egpe_status enq_lc_carried(int mode, int gate, int ctrl);
   egpe_status enq_attempt(int mode, AttemptKind kind);
+  // The current point of a run in PH_VERIFY by transform (nothing in other phases).
+  egpe_status enq_verify() { return enq_eg(0, GATE_VERIFY, 1, ATT_REFRESH); }
+  egpe_status enq_resnorm();
   egpe_status capture_attempt(int mode, AttemptKind kind, cudaGraphExec_t& out, int& kernels);
   egpe_status enq_kin(int potential, int gate);
   egpe_status enq_pg(int gate, const C* in);

@@ -1396,17 +1396,33 @@ template <class R> egpe_status Engine<R>::solve_poll(int& phase) {
   return EGPE_OK;
 }
 
+// ||r_i||^2 of the current point into st->pca.
+template <class R> egpe_status Engine<R>::enq_resnorm() {
+  KArgs<R> a = *base_;
+  const int grid = (int)std::min<size_t>((N + 255) / 256, (size_t)nsm_ * 8);
+  resnorm_kernel<R><<<grid, 256, 0, stream>>>(a);
+  ++kernels_;
+  EGPE_CUDA(cudaGetLastError());
+  return EGPE_OK;
+}
+
 template <class R>
 egpe_status Engine<R>::solve_finish(SolveRun& run, egpe_trace_entry* trace_out, int trace_cap, int trace_offset) {
-  {
-    KArgs<R> a = *base_;
-    const int grid = (int)std::min<size_t>((N + 255) / 256, (size_t)nsm_ * 8);
-    resnorm_kernel<R><<<grid, 256, 0, stream>>>(a);
-    ++kernels_;
-    EGPE_CUDA(cudaGetLastError());
-  }
+  EGPE_TRY(enq_resnorm());
   DevState hs;
   EGPE_TRY(read_state(hs, false));
+  if (hs.phase == PH_VERIFY) {  // a stepped run: its end is confirmed (or not) here
+    EGPE_TRY(enq_verify());
+    EGPE_TRY(enq_resnorm());
+    EGPE_TRY(read_state(hs, false));
+    if (hs.phase == PH_NEW_ITER && sqrt((hs.pca[0] + hs.pca[1]) * dV) < hs.opt.tol_res) {
+      hs.phase = st_host_->phase = PH_DONE;
+      hs.status = st_host_->status = EGPE_OK;
+      EGPE_CUDA(cudaMemcpyAsync(&st_->phase, &st_host_->phase, sizeof(int), cudaMemcpyHostToDevice, stream));
+      EGPE_CUDA(cudaMemcpyAsync(&st_->status, &st_host_->status, sizeof(int), cudaMemcpyHostToDevice, stream));
+      EGPE_CUDA(cudaStreamSynchronize(stream));  // the pinned mirror is free again
+    }
+  }
   run.status = (hs.phase == PH_DONE) ? hs.status : EGPE_ERR_NOT_CONVERGED;
   if (hs.timeout) run.status = EGPE_ERR_TIMEOUT;
   run.n = hs.n;
@@ -1454,12 +1470,12 @@ egpe_status Engine<R>::solve(const egpe_solve_opts& o, int fp32_phase, int max_i
                              int trace_offset) {
   EGPE_TRY(solve_begin(o, fp32_phase, max_iter, tol_res, accept_rtol, trace_out != nullptr, trace_cap));
   const int poll = std::max(1, o.poll_every);
-  const long long max_launch = max_attempts(max_iter, o.armijo_max, run_carried_);
-  while (run_launches_ < max_launch) {
-    EGPE_TRY(solve_launch(attempts_ahead(poll, max_iter, run_launches_)));
-    int phase = 0;
+  const long long max_launch = max_attempts(max_iter, o.armijo_max, poll, run_carried_);
+  int phase = PH_NEW_ITER;
+  while (run_launches_ < max_launch && phase != PH_DONE) {
+    if (phase == PH_VERIFY) EGPE_TRY(enq_verify());
+    EGPE_TRY(solve_launch(attempts_ahead(poll, max_iter, run_launches_, phase == PH_VERIFY)));
     EGPE_TRY(solve_poll(phase));
-    if (phase == PH_DONE) break;
   }
   return solve_finish(run, trace_out, trace_cap, trace_offset);
 }

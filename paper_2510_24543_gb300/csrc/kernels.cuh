@@ -75,6 +75,7 @@ template <class R> __device__ __forceinline__ bool gate_open(const KArgs<R>& a) 
   switch (a.gate) {
     case GATE_NEW_ITER: return ph == PH_NEW_ITER;
     case GATE_CARRIED_PC: return ph == PH_NEW_ITER || ph == PH_DIRECT;
+    case GATE_VERIFY: return ph == PH_VERIFY;
   }
   return ph == PH_NEW_ITER || ph == PH_TRIAL;
 }
