@@ -202,10 +202,13 @@ typedef struct egpe_handle egpe_handle;
 /* Create a handle for n_inst instances (grids[i], params[i]) of the given
  * precision on the current CUDA device.  cuda_stream is a cudaStream_t, or
  * NULL for a stream owned by the handle and ordered against the legacy default
- * stream at every call (see Streams above).  Allocates every workspace up front (about 26
- * complex fields per instance and precision); the first solve with a kinetic
- * preconditioner adds 10 more to an FP64 engine where they fit.  Errors: INVALID_ARG (bad sizes,
- * non-symmetric couplings, L <= 0, Q out of range), OOM, CUDA. */
+ * stream at every call (see Streams above).  Allocates every workspace up front: about 26
+ * complex fields per instance and precision, and 10 more per FP64 instance for
+ * what solves with a kinetic preconditioner carry along.  Those 10 are left out
+ * for the whole handle where they would take more than half of the memory still
+ * free; its solves then transform instead (slower, same results up to rounding).
+ * Errors: INVALID_ARG (bad sizes, non-symmetric couplings, L <= 0, Q out of
+ * range), OOM, CUDA. */
 egpe_status egpe_create(const egpe_grid* grids, const egpe_params* params, int n_inst,
                         egpe_precision prec, void* cuda_stream, egpe_handle** out);
 
@@ -320,7 +323,9 @@ egpe_status egpe_autotune(egpe_handle* h, int inst, int engine, const void* psi,
 /* Applies tuned shapes (key and choice of each entry; host array) to the
  * instance's engine, e.g. from a cache of an earlier egpe_autotune of the same
  * build, device and grid.  Entries whose key the engine never launches are
- * ignored; out-of-range choices fall back to the untuned shape. */
+ * ignored; out-of-range choices fall back to the untuned shape.  The key
+ * "carried kinetic terms" with choice 0 makes FP64 attempts with a kinetic
+ * preconditioner transform what they otherwise carry along (1, the default). */
 egpe_status egpe_set_tuning(egpe_handle* h, int inst, int engine, const egpe_tuning* t, int count);
 
 /* Diagnostic of the LHY interpolation tables that the energy/gradient and

@@ -42,12 +42,12 @@ template <class R> class BatchRunner {
     runs.assign(n, SolveRun{});
     EGPE_TRY(alloc());
     carried_ = true;
-    for (Engine<R>* e : eng_) carried_ = e->ensure_carry(o.precond) && carried_;
+    for (const Engine<R>* e : eng_) carried_ = carried_ && e->carries(o.precond);
     egpe_solve_opts oo = o;
     oo.use_graph = 0;
     for (int i = 0; i < n; ++i)
       EGPE_TRY(eng_[i]->solve_begin(oo, fp32_phase, max_iter, tol_res, accept_rtol, i == 0 && trace_out != nullptr,
-                                    trace_cap));
+                                    trace_cap, carried_));
     std::vector<int> phase;
     EGPE_TRY(gather(phase));
     std::vector<int> active = live(phase);
@@ -88,7 +88,7 @@ template <class R> class BatchRunner {
   std::vector<Engine<R>*> eng_;
   cudaStream_t stream_ = nullptr;
   bool concurrent_ = false;
-  bool carried_ = false;  // every instance has room for T psi and T p
+  bool carried_ = false;  // every instance carries T psi and T p
   std::vector<cudaStream_t> branch_;  // forked capture streams, one per group (concurrent mode)
   std::vector<cudaEvent_t> join_;     // [0]: fork point, [1 + g]: end of group g's chain
   cudaGraphExec_t graph_ = nullptr, refresh_ = nullptr;

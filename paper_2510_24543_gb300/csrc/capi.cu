@@ -38,6 +38,7 @@ struct egpe_handle {
   std::vector<Engine<double>*> e64;
   std::vector<Engine<float>*> e32;
   std::vector<egpe_grid> grids;
+  void* carry = nullptr;  // the FP64 engines' carried kinetic terms
 };
 
 namespace {
@@ -93,6 +94,26 @@ egpe_status validate(const egpe_grid& g, const egpe_params& p) {
     return EGPE_ERR_INVALID_ARG;
   }
   return EGPE_OK;
+}
+
+// Room for the carried kinetic terms of every FP64 engine, or of none: instances of a
+// batch share one kind of attempt, and a handle that would fit without them still does.
+// At least as much memory stays free as they take; engines without them transform.
+void alloc_carry(egpe_handle* h) {
+  size_t need = 0, free_bytes = 0, total = 0;
+  for (auto* e : h->e64) need += e->carry_bytes();
+  if (need == 0) return;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || need > free_bytes / 2 ||
+      cudaMalloc(&h->carry, need) != cudaSuccess) {
+    cudaGetLastError();
+    h->carry = nullptr;
+    return;
+  }
+  unsigned char* p = (unsigned char*)h->carry;
+  for (auto* e : h->e64) {
+    e->set_carry(p);
+    p += e->carry_bytes();
+  }
 }
 
 bool bad_inst(egpe_handle* h, int inst) { return !h || inst < 0 || inst >= h->n_inst; }
@@ -232,6 +253,7 @@ egpe_status egpe_create(const egpe_grid* grids, const egpe_params* params, int n
       }
     }
   }
+  alloc_carry(h);
   egpe_status s = sync_and_check(h);
   if (s != EGPE_OK) {
     egpe_destroy(h);
@@ -246,6 +268,7 @@ void egpe_destroy(egpe_handle* h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (auto* e : h->e64) delete e;
   for (auto* e : h->e32) delete e;
+  if (h->carry) cudaFree(h->carry);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   if (h->ev_in) cudaEventDestroy(h->ev_in);
   if (h->ev_out) cudaEventDestroy(h->ev_out);
@@ -465,13 +488,13 @@ egpe_status egpe_solver_start(egpe_handle* h, int inst, int engine, const void* 
     auto* e = h->e64[inst];
     egpe_status s = e->load_psi(psi, cudaMemcpyDeviceToDevice);
     if (s != EGPE_OK) return s;
-    return e->solve_begin(o, 0, o.max_iter, o.tol_res, o.accept_rtol, false, 0);
+    return e->solve_begin(o, 0, o.max_iter, o.tol_res, o.accept_rtol, false, 0, e->carries(o.precond));
   }
   if (engine == 1 && !h->e32.empty()) {
     auto* e = h->e32[inst];
     egpe_status s = e->load_psi(psi, cudaMemcpyDeviceToDevice);
     if (s != EGPE_OK) return s;
-    return e->solve_begin(o, 1, o.max_iter, o.tol_res, o.accept_rtol_fp32, false, 0);
+    return e->solve_begin(o, 1, o.max_iter, o.tol_res, o.accept_rtol_fp32, false, 0, false);
   }
   return EGPE_ERR_INVALID_ARG;
 }

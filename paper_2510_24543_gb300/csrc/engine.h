@@ -43,6 +43,8 @@ template <class R> struct LaunchRec {
 
 // Key of the tuning entry that sets the column tile width (kind 2).
 inline const char* const kColBytesKey = "column tile row bytes";
+// Key of the entry that says whether FP64 attempts may carry T psi and T p along.
+inline const char* const kCarryKey = "carried kinetic terms";
 
 // One tuned launch shape: rows per block (row passes), 1 = TMA-fed / 0 =
 // plain loads (column passes), or the column tile row width in bytes.
@@ -99,9 +101,13 @@ template <class R> class Engine {
   ~Engine() { destroy(); }
 
   egpe_status create(const egpe_grid& g, const egpe_params& p, cudaStream_t stream);
-  // Whether attempts of this mode carry T psi and T p along: allocates their 10 fields
-  // at the first solve that does; where they do not fit, every attempt is ATT_FULL.
-  bool ensure_carry(int mode);
+  // Room for T psi[2], T p[2] and P_V^{-1} r of an FP64 engine: kCarryFields fields that
+  // the handle allocates for all its instances or for none, and keeps.
+  static constexpr size_t kCarryFields = 10;
+  size_t carry_bytes() const { return kCarryFields * N * sizeof(C); }
+  void set_carry(void* p);
+  // Whether attempts of this mode carry T psi and T p along; if not, each is ATT_FULL.
+  bool carries(int mode) const { return sizeof(R) == 8 && carry_ && carry_on_ && carried_mode(mode); }
   void destroy();
 
   // Standalone evaluations (synchronous; device pointers of this precision).
@@ -128,8 +134,9 @@ template <class R> class Engine {
   // Stepping interface (the same phases egpe_ncg_solve runs): begin loads
   // nothing -- psi must be in slot 0 -- evaluates the start and prepares the
   // graph; launch enqueues attempts without waiting; finish reads the state.
+  // `carried`: as the caller's attempts will be.
   egpe_status solve_begin(const egpe_solve_opts& o, int fp32_phase, int max_iter, double tol_res,
-                          double accept_rtol, bool want_trace, int trace_cap);
+                          double accept_rtol, bool want_trace, int trace_cap, bool carried);
   egpe_status solve_launch(int attempts);
   egpe_status solve_poll(int& phase);
   egpe_status solve_finish(SolveRun& run, egpe_trace_entry* trace_out, int trace_cap, int trace_offset);
@@ -144,7 +151,8 @@ template <class R> class Engine {
   // Applies previously tuned shapes (by key); unknown keys are ignored.
   void set_tuning(const std::string& key, int choice) {
     if (key == kColBytesKey) return set_col_bytes(choice);
-    tune_[key] = choice;
+    if (key == kCarryKey) carry_on_ = choice != 0;
+    else tune_[key] = choice;
     drop_graphs();
   }
   void clear_tuning() {
@@ -253,8 +261,8 @@ template <class R> class Engine {
   egpe_grid grid_{};
   egpe_params prm_{};
   void* arena_ = nullptr;
-  void* carry_ = nullptr;  // tb, tp, wz
-  bool carry_failed_ = false;
+  bool carry_ = false;    // set_carry
+  bool carry_on_ = true;  // kCarryKey
   C* twx_ = nullptr;
   C* twy_ = nullptr;
   C* twz_ = nullptr;

@@ -332,27 +332,16 @@ template <class R> void Engine<R>::drop_graphs() {
   graph_ite_ = nullptr;
 }
 
-template <class R> bool Engine<R>::ensure_carry(int mode) {
-  if (sizeof(R) != 8 || !carried_mode(mode) || carry_failed_) return false;
-  if (carry_) return true;
-  // tb[2], tp[2], wz: every value is written before it is read
-  if (cudaMalloc(&carry_, 10 * N * sizeof(C)) != cudaSuccess) {
-    cudaGetLastError();
-    carry_ = nullptr;
-    carry_failed_ = true;
-    return false;
-  }
-  C* c = reinterpret_cast<C*>(carry_);
+// Every value is written before it is read.
+template <class R> void Engine<R>::set_carry(void* p) {
+  carry_ = true;
+  C* c = reinterpret_cast<C*>(p);
   for (int b = 0; b < 2; ++b) base_->tb[b] = c + 2 * b * N;
   for (int b = 0; b < 2; ++b) base_->tp[b] = c + (4 + 2 * b) * N;
   base_->wz = c + 8 * N;
-  return true;
 }
 
 template <class R> void Engine<R>::destroy() {
-  if (carry_) cudaFree(carry_);
-  carry_ = nullptr;
-  carry_failed_ = false;
   for (auto& k : tlog_) {
     cudaEventDestroy(k.a);
     cudaEventDestroy(k.b);
@@ -451,7 +440,7 @@ egpe_status Engine<R>::profile_attempt(const C* psi, int precond, int reps, std:
   EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(reset_state(&o, sizeof(R) == 4, 1 << 30, 0.0, sizeof(R) == 4 ? 1e-6 : 1e-13));
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0);
+  const AttemptKind kind = attempt_kind(carries(precond), 0);
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   EGPE_CUDA(cudaStreamSynchronize(stream));
   names.clear();
@@ -541,7 +530,7 @@ egpe_status Engine<R>::autotune(const C* psi, int precond, int reps, std::vector
   EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
   EGPE_TRY(reset_state(&o, sizeof(R) == 4, 1 << 30, 0.0, sizeof(R) == 4 ? 1e-6 : 1e-13));
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  const AttemptKind kind = attempt_kind(ensure_carry(precond), 0);
+  const AttemptKind kind = attempt_kind(carries(precond), 0);
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   EGPE_TRY(enq_attempt(o.precond, kind));  // realistic coefficients in the state
   EGPE_CUDA(cudaStreamSynchronize(stream));
@@ -1197,7 +1186,7 @@ template <class R> egpe_status Engine<R>::store_psi(void* dst, cudaMemcpyKind ki
 
 template <class R>
 egpe_status Engine<R>::solve_begin(const egpe_solve_opts& o, int fp32_phase, int max_iter, double tol_res,
-                                   double accept_rtol, bool want_trace, int trace_cap) {
+                                   double accept_rtol, bool want_trace, int trace_cap, bool carried) {
   const int mode = o.precond;
   if (want_trace && trace_cap > trace_alloc_) {
     // the trace buffer is captured by the graphs: allocate once, generously
@@ -1215,7 +1204,7 @@ egpe_status Engine<R>::solve_begin(const egpe_solve_opts& o, int fp32_phase, int
   EGPE_TRY(reset_state(&oo, fp32_phase, max_iter, tol_res, accept_rtol));
   // r and p history start at zero (beta = 0 at n = 0 reads them)
   EGPE_CUDA(cudaMemsetAsync(base_->rb[0], 0, 8 * N * sizeof(C), stream));
-  run_carried_ = ensure_carry(mode);
+  run_carried_ = carried;
   const AttemptKind kind = attempt_kind(run_carried_, 0);
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, kind));
   run_k0_ = kernels_;
@@ -1468,7 +1457,8 @@ template <class R>
 egpe_status Engine<R>::solve(const egpe_solve_opts& o, int fp32_phase, int max_iter, double tol_res,
                              double accept_rtol, SolveRun& run, egpe_trace_entry* trace_out, int trace_cap,
                              int trace_offset) {
-  EGPE_TRY(solve_begin(o, fp32_phase, max_iter, tol_res, accept_rtol, trace_out != nullptr, trace_cap));
+  EGPE_TRY(solve_begin(o, fp32_phase, max_iter, tol_res, accept_rtol, trace_out != nullptr, trace_cap,
+                       carries(o.precond)));
   const int poll = std::max(1, o.poll_every);
   const long long max_launch = max_attempts(max_iter, o.armijo_max, poll, run_carried_);
   int phase = PH_NEW_ITER;
