@@ -180,12 +180,12 @@ template <class R> class Engine {
 
  private:
   // att: whether T psi is stored for attempts that carry it along (not ATT_FULL)
-  // in, out: the caller's psi and gradient of a standalone evaluation (element-aligned)
+  // in, out: the caller's psi and gradient of a standalone evaluation (usable)
   egpe_status enq_eg(int trial, int gate, int ctrl, AttemptKind att = ATT_FULL, const C* in = nullptr,
                      C* out = nullptr);
   // A standalone evaluation of psi without waiting for it; hp and aux as after a trial.
   egpe_status enq_evaluation(const C* psi, C* grad);
-  static bool element_aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % sizeof(C) == 0; }
+  bool usable(const void* p);
   void energy_out(const DevState& hs, egpe_energy_terms& out) const;
   egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att = ATT_FULL, C* z = nullptr);
   egpe_status enq_lc(int gate, int ctrl, int pgiven);

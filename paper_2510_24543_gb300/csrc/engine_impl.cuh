@@ -12,6 +12,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "caller_mem.h"
 #include "engine.h"
 #include "host_tables.h"
 #include "kernels.cuh"
@@ -51,6 +52,30 @@ static TmaEncodeFn tma_encode_fn() {
       fn = reinterpret_cast<TmaEncodeFn>(p);
   }
   return fn;
+}
+
+// Facts about a caller's pointer, through the driver entry point as above.
+static PtrFacts ptr_facts(const void* p) {
+  typedef CUresult (*Fn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Fn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return reinterpret_cast<Fn>(f);
+  }();
+  PtrFacts o;
+  CUdeviceptr d = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute at[3] = {CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                               CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[3] = {&d, &start, &size};
+  if (!fn || fn(3, at, out, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return o;
+  o.device_ptr = d;
+  o.range_start = start;
+  o.range_size = size;
+  return o;
 }
 
 // Columns per tile of the strided passes: tile rows of col_bytes (64, 128 or
@@ -210,9 +235,8 @@ template <class R> egpe_status Engine<R>::enq_pg(int gate, const C* in) {
 
 template <class R> egpe_status Engine<R>::param_grad(const C* psi, double out[EGPE_NPARAM]) {
   EGPE_TRY(reset_state(nullptr, 0, 0, 0.0, 0.0));
-  const bool direct = element_aligned(psi);
-  if (!direct)
-    EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  const bool direct = usable(psi);
+  if (!direct) EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDefault, stream));
   EGPE_TRY(enq_pg(GATE_ALWAYS, direct ? psi : nullptr));
   DevState hs;
   EGPE_TRY(read_state(hs));
@@ -1055,15 +1079,20 @@ template <class R> egpe_status Engine<R>::read_state(DevState& hs, bool report_t
 
 // The first pass reads psi from the caller's buffer and leaves it in the psi buffer
 // (the later passes read it there, so grad may be psi), the last one writes H psi to
-// both: no copies of their own.  Buffers that are not element-aligned are copied.
+// both: no copies of their own.  Buffers that the kernels cannot take as they are
+// (caller_mem.h) are copied.
 template <class R> egpe_status Engine<R>::enq_evaluation(const C* psi, C* grad) {
   EGPE_TRY(reset_state(nullptr, 0, 0, 0.0, 0.0));
-  const bool din = element_aligned(psi), dout = element_aligned(grad);
-  if (!din) EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  const bool din = usable(psi), dout = grad && usable(grad);
+  if (!din) EGPE_CUDA(cudaMemcpyAsync(base_->psi[0], psi, 2 * N * sizeof(C), cudaMemcpyDefault, stream));
   EGPE_TRY(enq_eg(0, GATE_ALWAYS, 1, ATT_FULL, din ? psi : nullptr, dout ? grad : nullptr));
-  if (grad && !dout)
-    EGPE_CUDA(cudaMemcpyAsync(grad, base_->hp[0], 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  if (grad && !dout) EGPE_CUDA(cudaMemcpyAsync(grad, base_->hp[0], 2 * N * sizeof(C), cudaMemcpyDefault, stream));
   return EGPE_OK;
+}
+
+// Whether kernels may take the caller's two fields at p in place.
+template <class R> bool Engine<R>::usable(const void* p) {
+  return in_place(ptr_facts(p), (uint64_t)(uintptr_t)p, 2 * N * sizeof(C), sizeof(C));
 }
 
 template <class R> void Engine<R>::energy_out(const DevState& hs, egpe_energy_terms& out) const {
@@ -1109,9 +1138,9 @@ template <class R> egpe_status Engine<R>::line_coeffs(const C* psi, const C* p, 
 template <class R> egpe_status Engine<R>::precondition(int mode, const C* psi, const C* r, C* z) {
   EGPE_TRY(enq_evaluation(psi, nullptr));
   if (r) EGPE_CUDA(cudaMemcpyAsync(base_->rb[0], r, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
-  const bool dz = element_aligned(z);
+  const bool dz = usable(z);
   EGPE_TRY(enq_pc(mode, GATE_ALWAYS, 0, r ? 1 : 0, ATT_FULL, dz ? z : nullptr));
-  if (!dz) EGPE_CUDA(cudaMemcpyAsync(z, base_->z, 2 * N * sizeof(C), cudaMemcpyDeviceToDevice, stream));
+  if (!dz) EGPE_CUDA(cudaMemcpyAsync(z, base_->z, 2 * N * sizeof(C), cudaMemcpyDefault, stream));
   DevState hs;
   return read_state(hs);
 }
