@@ -38,7 +38,6 @@ struct egpe_handle {
   std::vector<Engine<double>*> e64;
   std::vector<Engine<float>*> e32;
   std::vector<egpe_grid> grids;
-  void* carry = nullptr;  // the FP64 engines' carried kinetic terms
 };
 
 namespace {
@@ -96,24 +95,41 @@ egpe_status validate(const egpe_grid& g, const egpe_params& p) {
   return EGPE_OK;
 }
 
-// Room for the carried kinetic terms of every FP64 engine, or of none: instances of a
-// batch share one kind of attempt, and a handle that would fit without them still does.
-// At least as much memory stays free as they take; engines without them transform.
-void alloc_carry(egpe_handle* h) {
-  size_t need = 0, free_bytes = 0, total = 0;
-  for (auto* e : h->e64) need += e->carry_bytes();
-  if (need == 0) return;
-  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || need > free_bytes / 2 ||
-      cudaMalloc(&h->carry, need) != cudaSuccess) {
-    cudaGetLastError();
-    h->carry = nullptr;
-    return;
+// Whether the FP64 engines get room for the carried kinetic terms, all or none:
+// instances of a batch share one kind of attempt, and a handle that fits without them
+// still does.  At least as much memory stays free as they take.
+bool room_to_carry(const egpe_grid* grids, int n_inst, egpe_precision prec) {
+  if (prec == EGPE_FP32) return false;
+  size_t points = 0, free_bytes = 0, total = 0;
+  for (int i = 0; i < n_inst; ++i) points += (size_t)grids[i].n[0] * grids[i].n[1] * grids[i].n[2];
+  const size_t fields = points * sizeof(double2);
+  const size_t base = Engine<double>::kFields * fields * (prec == EGPE_MIXED ? 3 : 2) / 2;
+  const size_t carry = Engine<double>::kCarryFields * fields;
+  return cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes >= base + 2 * carry;
+}
+
+// The engines of a handle's instances.
+egpe_status create_engines(egpe_handle* h, const egpe_grid* grids, const egpe_params* params, bool carry) {
+  for (int i = 0; i < h->n_inst; ++i) {
+    if (h->prec != EGPE_FP32) {
+      h->e64.push_back(new Engine<double>());
+      const egpe_status s = h->e64.back()->create(grids[i], params[i], h->stream, carry);
+      if (s != EGPE_OK) return s;
+    }
+    if (h->prec != EGPE_FP64) {
+      h->e32.push_back(new Engine<float>());
+      const egpe_status s = h->e32.back()->create(grids[i], params[i], h->stream, false);
+      if (s != EGPE_OK) return s;
+    }
   }
-  unsigned char* p = (unsigned char*)h->carry;
-  for (auto* e : h->e64) {
-    e->set_carry(p);
-    p += e->carry_bytes();
-  }
+  return EGPE_OK;
+}
+
+void delete_engines(egpe_handle* h) {
+  for (auto* e : h->e64) delete e;
+  for (auto* e : h->e32) delete e;
+  h->e64.clear();
+  h->e32.clear();
 }
 
 bool bad_inst(egpe_handle* h, int inst) { return !h || inst < 0 || inst >= h->n_inst; }
@@ -233,28 +249,15 @@ egpe_status egpe_create(const egpe_grid* grids, const egpe_params* params, int n
     h->own_stream = true;
   }
   h->grids.assign(grids, grids + n_inst);
-  for (int i = 0; i < n_inst; ++i) {
-    if (prec == EGPE_FP64 || prec == EGPE_MIXED) {
-      auto* e = new Engine<double>();
-      h->e64.push_back(e);
-      egpe_status s = e->create(grids[i], params[i], h->stream);
-      if (s != EGPE_OK) {
-        egpe_destroy(h);
-        return s;
-      }
-    }
-    if (prec == EGPE_FP32 || prec == EGPE_MIXED) {
-      auto* e = new Engine<float>();
-      h->e32.push_back(e);
-      egpe_status s = e->create(grids[i], params[i], h->stream);
-      if (s != EGPE_OK) {
-        egpe_destroy(h);
-        return s;
-      }
-    }
+  const bool carry = room_to_carry(grids, n_inst, prec);
+  egpe_status s = create_engines(h, grids, params, carry);
+  if (s == EGPE_ERR_OOM && carry) {  // free, but not in one piece
+    cudaGetLastError();
+    cudaStreamSynchronize(h->stream);
+    delete_engines(h);
+    s = create_engines(h, grids, params, false);
   }
-  alloc_carry(h);
-  egpe_status s = sync_and_check(h);
+  if (s == EGPE_OK) s = sync_and_check(h);
   if (s != EGPE_OK) {
     egpe_destroy(h);
     return s;
@@ -266,9 +269,7 @@ egpe_status egpe_create(const egpe_grid* grids, const egpe_params* params, int n
 void egpe_destroy(egpe_handle* h) {
   if (!h) return;
   if (h->stream) cudaStreamSynchronize(h->stream);
-  for (auto* e : h->e64) delete e;
-  for (auto* e : h->e32) delete e;
-  if (h->carry) cudaFree(h->carry);
+  delete_engines(h);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   if (h->ev_in) cudaEventDestroy(h->ev_in);
   if (h->ev_out) cudaEventDestroy(h->ev_out);

@@ -100,12 +100,10 @@ template <class R> class Engine {
   Engine& operator=(const Engine&) = delete;
   ~Engine() { destroy(); }
 
-  egpe_status create(const egpe_grid& g, const egpe_params& p, cudaStream_t stream);
-  // Room for T psi[2], T p[2] and P_V^{-1} r of an FP64 engine: kCarryFields fields that
-  // the handle allocates for all its instances or for none, and keeps.
-  static constexpr size_t kCarryFields = 10;
-  size_t carry_bytes() const { return kCarryFields * N * sizeof(C); }
-  void set_carry(void* p);
+  // Fields of the workspace, and of the carried kinetic terms of an FP64 engine
+  // (T psi[2], T p[2] and P_V^{-1} r), which a handle takes for all its instances or for none.
+  static constexpr size_t kFields = 25, kCarryFields = 10;
+  egpe_status create(const egpe_grid& g, const egpe_params& p, cudaStream_t stream, bool carry);
   // Whether attempts of this mode carry T psi and T p along; if not, each is ATT_FULL.
   bool carries(int mode) const { return sizeof(R) == 8 && carry_ && carry_on_ && carried_mode(mode); }
   void destroy();
@@ -261,7 +259,7 @@ template <class R> class Engine {
   egpe_grid grid_{};
   egpe_params prm_{};
   void* arena_ = nullptr;
-  bool carry_ = false;    // set_carry
+  bool carry_ = false;    // created with room for them
   bool carry_on_ = true;  // kCarryKey
   C* twx_ = nullptr;
   C* twy_ = nullptr;

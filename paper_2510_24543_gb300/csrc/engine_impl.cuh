@@ -260,7 +260,7 @@ template <class R> egpe_status Engine<R>::param_grad(const C* psi, double out[EG
   return EGPE_OK;
 }
 
-template <class R> egpe_status Engine<R>::create(const egpe_grid& g, const egpe_params& p, cudaStream_t s) {
+template <class R> egpe_status Engine<R>::create(const egpe_grid& g, const egpe_params& p, cudaStream_t s, bool carry) {
   grid_ = g;
   prm_ = p;
   stream = s;
@@ -272,9 +272,11 @@ template <class R> egpe_status Engine<R>::create(const egpe_grid& g, const egpe_
   EGPE_CUDA(cudaGetDevice(&dev));
   EGPE_CUDA(cudaDeviceGetAttribute(&nsm_, cudaDevAttrMultiProcessorCount, dev));
   const size_t fb = N * sizeof(C);
-  // psi[2], hp[2], ax[2], rb[2], pb[2]: 2 fields each; z: 2; W: 3  -> 25 fields
-  EGPE_CUDA(cudaMalloc(&arena_, 25 * fb));
-  EGPE_CUDA(cudaMemsetAsync(arena_, 0, 25 * fb, stream));
+  // psi[2], hp[2], ax[2], rb[2], pb[2]: 2 fields each; z: 2; W: 3  -> 25 fields;
+  // tb[2], tp[2]: 2 each; wz: 2 (every value is written before it is read)
+  carry_ = carry;
+  EGPE_CUDA(cudaMalloc(&arena_, (kFields + (carry ? kCarryFields : 0)) * fb));
+  EGPE_CUDA(cudaMemsetAsync(arena_, 0, kFields * fb, stream));
   C* f = reinterpret_cast<C*>(arena_);
   base_ = new KArgs<R>();
   std::memset((void*)base_, 0, sizeof(KArgs<R>));
@@ -286,6 +288,12 @@ template <class R> egpe_status Engine<R>::create(const egpe_grid& g, const egpe_
   for (int b = 0; b < 2; ++b) a.pb[b] = f + (16 + 2 * b) * N;
   a.z = f + 20 * N;
   a.W = f + 22 * N;
+  if (carry) {
+    C* c = f + kFields * N;
+    for (int b = 0; b < 2; ++b) a.tb[b] = c + 2 * b * N;
+    for (int b = 0; b < 2; ++b) a.tp[b] = c + (4 + 2 * b) * N;
+    a.wz = c + 8 * N;
+  }
   // twiddles W_L^m = exp(-2 pi i m / L), long double on the host
   C** tws[3] = {&twx_, &twy_, &twz_};
   for (int ax = 0; ax < 3; ++ax) {
@@ -354,15 +362,6 @@ template <class R> void Engine<R>::drop_graphs() {
       }
   if (graph_ite_) cudaGraphExecDestroy(graph_ite_);
   graph_ite_ = nullptr;
-}
-
-// Every value is written before it is read.
-template <class R> void Engine<R>::set_carry(void* p) {
-  carry_ = true;
-  C* c = reinterpret_cast<C*>(p);
-  for (int b = 0; b < 2; ++b) base_->tb[b] = c + 2 * b * N;
-  for (int b = 0; b < 2; ++b) base_->tp[b] = c + (4 + 2 * b) * N;
-  base_->wz = c + 8 * N;
 }
 
 template <class R> void Engine<R>::destroy() {
