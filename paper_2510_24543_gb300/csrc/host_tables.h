@@ -385,7 +385,8 @@ template <class R> inline LhyTableHost lhy_interp_table(const egpe_params& p) {
 // The device's records (lhy.cuh) of the tables, 16-byte aligned: per half and
 // interval the coefficients of the kTabFun functions, FP32 as they are, FP64 as
 // 64-bit fixed point with 61 - E fractional bits, sum_k |c_k| <= 2^E, followed by
-// the five exponents E (32-bit) and padding.
+// the five exponents E (32-bit) and padding.  A function below 2^-900 (a vanishing
+// prefactor) is 0: values down to 2^-63 of it must keep a normal FP64 exponent.
 template <class R> inline std::vector<R> lhy_pack_table(const LhyTableHost& T) {
   return std::vector<R>(T.coef.begin(), T.coef.end());
 }
@@ -401,6 +402,7 @@ template <> inline std::vector<double> lhy_pack_table<double>(const LhyTableHost
       for (int k = 0; k < NC; ++k) sum += fabsl(c[f * NC + k]);
       int e = 0;
       if (sum > 0) frexpl(sum, &e);  // sum < 2^e
+      if (e < -900) continue;
       ex[f] = e;
       for (int k = 0; k < NC; ++k) w[f * NC + k] = llroundl(ldexpl(c[f * NC + k], 61 - e));
     }
