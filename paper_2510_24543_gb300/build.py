@@ -23,8 +23,9 @@ UNITS = ["capi.cu", "engine_f64.cu", "engine_f32.cu", "engine_mr_f64.cu", "engin
          "engine_mr5_f32.cu", "engine_big_f64.cu", "engine_big_f32.cu"]
 # The FP32-field engine flushes denormals and uses the approximate (MUFU)
 # divide and square root: values below 1e-38 carry no weight in any sum of that
-# path, and its fields are accurate to ~1e-7 anyway.  The FP64 engine keeps
-# IEEE division and square root.
+# path, and its fields are accurate to ~1e-7 anyway.  The FP64 engine's passes form
+# reciprocals and square roots by a third-order step (csrc/lhy.cuh, within 1.35 ulp);
+# where a division or a square root is written there, it is the IEEE one.
 _FP32_FLAGS = ["-ftz=true", "-prec-div=false", "-prec-sqrt=false"]
 UNIT_FLAGS = {u: _FP32_FLAGS for u in UNITS if u.endswith("f32.cu")}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

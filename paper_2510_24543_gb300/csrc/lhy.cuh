@@ -51,7 +51,7 @@ template <> __device__ __forceinline__ float s2_min<float>() { return 1e-36f; }
 // root (MUFU, a few ulp).
 __device__ __forceinline__ double sqrt_pos(double v) {
   const double r = v * rsqrt_(v);
-  return v > 1e-300 ? r : 0.0;
+  return v <= 1e-300 ? 0.0 : r;  // NaN stays NaN
 }
 __device__ __forceinline__ float sqrt_pos(float v) { return sqrtf(v); }
 
