@@ -291,8 +291,8 @@ egpe_status egpe_retract(egpe_handle* h, int inst, const void* psi, const void* 
  * fields of the instance's grid with the library's own Stockham kernels.
  * in and out may alias.  Device pointers.  A diagnostic of the transform that
  * every other entry point uses.  FP64 lines are transformed in 64-bit fixed point
- * under a scale of their own: a line with a value of 2^1013 or more (or not
- * finite) gives NaN, a line with none above 2^-960 gives 0. */
+ * under a scale of their own: a line with a value that is not finite gives NaN,
+ * a line with none above 2^-960 gives 0. */
 egpe_status egpe_fft(egpe_handle* h, int inst, const void* in, void* out, int nfields, int inverse);
 
 /* Diagnostic: device time of every kernel of one solver attempt

@@ -41,6 +41,9 @@ template <class R> struct LaunchRec {
   long long rows = 0;
 };
 
+// Plain column passes: the pipelines' y pass, and those of the caller's own fields.
+enum PlainAxis { kAxisY = 1, kAxisZ = 2, kAxisYWide = 3 };
+
 // Key of the tuning entry that sets the column tile width (kind 2).
 inline const char* const kColBytesKey = "column tile row bytes";
 // Key of the entry that says whether FP64 attempts may carry T psi and T p along.

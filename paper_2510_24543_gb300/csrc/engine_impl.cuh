@@ -227,9 +227,9 @@ template <class R> egpe_status Engine<R>::enq_pg(int gate, const C* in) {
   KArgs<R> y = a;
   y.gin = a.W;
   y.gout = a.W;
-  EGPE_TRY(plain_col(1, 0, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 0, y, tmy()));
   EGPE_TRY(dispatch_col<ZPg>(nz, a, tmz()));
-  EGPE_TRY(plain_col(1, 1, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 1, y, tmy()));
   return dispatch_x<XInvPG>(nx, a);
 }
 
@@ -852,12 +852,15 @@ template <class R> template <int... Ls> egpe_status Engine<R>::plain_x_in(int in
 
 template <class R> template <int... Ls>
 egpe_status Engine<R>::plain_col_in(int axis, int inverse, const KArgs<R>& a, const CUtensorMap* tm) {
-  const int L = axis == 1 ? ny : nz;
+  constexpr bool W = sizeof(R) == 8;  // FP32 lines have no scale: one op for both y passes
+  const int L = axis == kAxisZ ? nz : ny;
   egpe_status s = EGPE_ERR_UNSUPPORTED;
-  (void)((L == Ls ? (s = axis == 1 ? (inverse ? launch_col<ColPlain<R, Ls, 1, true>>(a, tm)
-                                              : launch_col<ColPlain<R, Ls, 1, false>>(a, tm))
-                                   : (inverse ? launch_col<ColPlain<R, Ls, 2, true>>(a, tm)
-                                              : launch_col<ColPlain<R, Ls, 2, false>>(a, tm)),
+  (void)((L == Ls ? (s = axis == kAxisY ? (inverse ? launch_col<ColPlain<R, Ls, 1, true>>(a, tm)
+                                                   : launch_col<ColPlain<R, Ls, 1, false>>(a, tm))
+                       : axis == kAxisYWide ? (inverse ? launch_col<ColPlain<R, Ls, 1, true, W>>(a, tm)
+                                                       : launch_col<ColPlain<R, Ls, 1, false, W>>(a, tm))
+                                            : (inverse ? launch_col<ColPlain<R, Ls, 2, true, W>>(a, tm)
+                                                       : launch_col<ColPlain<R, Ls, 2, false, W>>(a, tm)),
                      true)
                   : false) ||
          ...);
@@ -889,7 +892,7 @@ template <class R> egpe_status Engine<R>::plain_x(int inverse, const KArgs<R>& a
 
 template <class R>
 egpe_status Engine<R>::plain_col(int axis, int inverse, const KArgs<R>& a, const CUtensorMap* tm) {
-  const int L = axis == 1 ? ny : nz;
+  const int L = axis == kAxisZ ? nz : ny;
   if (L == 128 || L == 256) return plain_col_big(axis, inverse, a, tm);
   if (L == 80) return plain_col_mr5(axis, inverse, a, tm);
   if (L == 48 || L == 96) return plain_col_mr(axis, inverse, a, tm);
@@ -912,9 +915,9 @@ template <class R> egpe_status Engine<R>::enq_eg(int trial, int gate, int ctrl, 
   KArgs<R> y = a;
   y.gin = a.W;
   y.gout = a.W;
-  EGPE_TRY(plain_col(1, 0, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 0, y, tmy()));
   EGPE_TRY(dispatch_col<ZEg>(nz, a, tmz()));
-  EGPE_TRY(plain_col(1, 1, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 1, y, tmy()));
   a.ctrl = ctrl;
   return dispatch_x<XInvEG>(nx, a);
 }
@@ -936,9 +939,9 @@ template <class R> egpe_status Engine<R>::enq_pc(int mode, int gate, int ctrl, i
     KArgs<R> y = a;
     y.gin = a.W;
     y.gout = a.W;
-    EGPE_TRY(plain_col(1, 0, y, tmy()));
+    EGPE_TRY(plain_col(kAxisY, 0, y, tmy()));
     EGPE_TRY(dispatch_col<ZPc>(nz, a, tmz()));
-    EGPE_TRY(plain_col(1, 1, y, tmy()));
+    EGPE_TRY(plain_col(kAxisY, 1, y, tmy()));
     a.ctrl = ctrl;
     return dispatch_x<XInvPC>(nx, a);
   }
@@ -960,11 +963,11 @@ template <class R> egpe_status Engine<R>::enq_lc(int gate, int ctrl, int pgiven)
   KArgs<R> y = a;
   y.gin = a.W;
   y.gout = a.W;
-  EGPE_TRY(plain_col(1, 0, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 0, y, tmy()));
   EGPE_TRY(dispatch_col<ZLc>(nz, a, tmz()));
   y.nf = 1;
   y.f0 = 2;
-  EGPE_TRY(plain_col(1, 1, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 1, y, tmy()));
   a.ctrl = ctrl;
   return dispatch_x<XInvLC>(nx, a);
 }
@@ -974,9 +977,9 @@ template <class R> egpe_status Engine<R>::enq_dipolar(const KArgs<R>& a) {
   KArgs<R> y = a;
   y.gin = a.W;
   y.gout = a.W;
-  EGPE_TRY(plain_col(1, 0, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 0, y, tmy()));
   EGPE_TRY(dispatch_col<ZPg>(nz, a, tmz()));
-  return plain_col(1, 1, y, tmy());
+  return plain_col(kAxisY, 1, y, tmy());
 }
 
 // Line-search and trial pipelines with T psi and T p carried along: one packed
@@ -1191,8 +1194,8 @@ template <class R> egpe_status Engine<R>::fft(const C* in, C* out, int nf, int i
     CUtensorMap my, mz;
     const bool ok = use_tma_ && make_col_map<C>(my, out + (size_t)f * N, nx, ny, nz, 1, 1, col_bytes_) &&
                     make_col_map<C>(mz, out + (size_t)f * N, nx, ny, nz, 1, 2, col_bytes_);
-    EGPE_TRY(plain_col(1, inverse, a, ok ? &my : nullptr));
-    EGPE_TRY(plain_col(2, inverse, a, ok ? &mz : nullptr));
+    EGPE_TRY(plain_col(kAxisYWide, inverse, a, ok ? &my : nullptr));
+    EGPE_TRY(plain_col(kAxisZ, inverse, a, ok ? &mz : nullptr));
   }
   EGPE_CUDA(cudaStreamSynchronize(stream));
   return EGPE_OK;
@@ -1290,9 +1293,9 @@ template <class R> egpe_status Engine<R>::enq_kin(int potential, int gate) {
   KArgs<R> y = a;
   y.gin = a.W;
   y.gout = a.W;
-  EGPE_TRY(plain_col(1, 0, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 0, y, tmy()));
   EGPE_TRY(dispatch_col<ZKin>(nz, a, tmz()));
-  EGPE_TRY(plain_col(1, 1, y, tmy()));
+  EGPE_TRY(plain_col(kAxisY, 1, y, tmy()));
   return dispatch_x<XInvKin>(nx, a);
 }
 

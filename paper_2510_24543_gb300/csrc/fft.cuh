@@ -193,7 +193,9 @@ template <bool INV, class C> __device__ __forceinline__ void dft5(C* v) {
 // extended precision 2.3e-16 -> 0.9e-16 (32^3), 2.7e-16 -> 1.0e-16 (64^3),
 // 2.8e-16 -> 1.5e-16 (256 x 16 x 128), 2.9e-16 -> 1.2e-16 (80^3).  Lines with a
 // value of at least 2^1013 (or not finite) give NaN; lines with no value above
-// 2^-960 give 0.
+// 2^-960 give 0.  Squares of such values are out of range anyway in the pipelines; the
+// plain transforms of the caller's own fields are WIDE and take values up to the
+// largest (in every pass that cost the FP64 attempt 0.5% at 128^3 and 1.8% at 96^3).
 // ----------------------------------------------------------------------------
 struct __align__(16) Q2 {
   long long x, y;
@@ -212,6 +214,8 @@ struct LineScale {
   int keep;  // 0 for a line that is taken as 0: clears the signs of its values too
   int bad;  // bits or-ed into the outputs' high words: a NaN pattern for a line that is not finite
 };
+constexpr int kLineBad = 0x7ff80000;
+constexpr int kLineBig = 0x7ffc0000;  // WIDE: finite, but exponents may overflow on the way (NaN to the others)
 
 __device__ __forceinline__ long long to_fixed(double d, const LineScale& ls) {
   const int hi = __double2hiint(d);
@@ -257,12 +261,12 @@ __device__ __forceinline__ uint2 add_bounds(uint2 a, uint2 b) {
   const int E = max((int)a.x, (int)b.x);
   return make_uint2((unsigned)E, (a.y >> min(E - (int)a.x, 31)) + (b.y >> min(E - (int)b.x, 31)) + 1u);
 }
-__device__ __forceinline__ LineScale make_scale(uint2 b) {
+template <bool WIDE> __device__ __forceinline__ LineScale make_scale(uint2 b) {
   const int E = (int)b.x;
   LineScale s;
   s.X = E < 64 ? 4096 : E + (32 - __clz((int)b.y)) - 20;
   s.keep = E < 64 ? 0 : -1;
-  s.bad = E >= 2036 ? 0x7ff80000 : 0;
+  s.bad = E >= 2036 ? (WIDE && E < 2047 ? kLineBig : kLineBad) : 0;
   return s;
 }
 
@@ -270,7 +274,7 @@ __device__ __forceinline__ LineScale make_scale(uint2 b) {
 // warp; the other row lines exchange their shares through the line's (idle)
 // exchange buffer, column lines through the slots `sc`, which are free again
 // after the transform's first exchange barrier.
-template <int L, int NF, class SI>
+template <int L, int NF, bool WIDE, class SI>
 __device__ __forceinline__ void line_scales(const double2 (&v)[NF][8], double2* sm, int fstride, int t, const SI& si,
                                             LineScale (&ls)[NF]) {
   constexpr int TPL = L / 8;
@@ -284,7 +288,7 @@ __device__ __forceinline__ void line_scales(const double2 (&v)[NF][8], double2* 
     uint2 a = si.sc[0];
 #pragma unroll 8
     for (int k = 1; k < TPL; ++k) a = add_bounds(a, si.sc[k * si.width()]);
-    ls[0] = make_scale(a);
+    ls[0] = make_scale<WIDE>(a);
   } else if constexpr (IsPow2<L>::v) {
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -292,7 +296,7 @@ __device__ __forceinline__ void line_scales(const double2 (&v)[NF][8], double2* 
       for (int off = TPL / 2; off > 0; off >>= 1)
         b[f] = add_bounds(b[f], make_uint2(__shfl_xor_sync(0xffffffffu, b[f].x, off),
                                            __shfl_xor_sync(0xffffffffu, b[f].y, off)));
-      ls[f] = make_scale(b[f]);
+      ls[f] = make_scale<WIDE>(b[f]);
     }
   } else {
 #pragma unroll
@@ -304,7 +308,7 @@ __device__ __forceinline__ void line_scales(const double2 (&v)[NF][8], double2* 
       uint2 a = p[0];
 #pragma unroll
       for (int k = 1; k < TPL; ++k) a = add_bounds(a, p[k]);
-      ls[f] = make_scale(a);
+      ls[f] = make_scale<WIDE>(a);
     }
     __syncthreads();
   }
@@ -528,7 +532,7 @@ __device__ __forceinline__ void fft_mixed(C (&v)[NF][8], C* sm, int fstride, con
   __syncthreads();  // callers may reuse the buffer
 }
 
-template <class C, int L, bool INV, int NF, class SI>
+template <class C, int L, bool INV, int NF, bool WIDE = false, class SI>
 __device__ __forceinline__ void fft_line(C (&v)[NF][8], C* sm, int fstride, const C* __restrict__ tw, int t,
                                          const SI& si) {
   if constexpr (std::is_same<C, double2>::value) {
@@ -536,7 +540,7 @@ __device__ __forceinline__ void fft_line(C (&v)[NF][8], C* sm, int fstride, cons
     const TwQ* qt = reinterpret_cast<const TwQ*>(tw);
     Q2 q[NF][8];
     LineScale ls[NF];
-    line_scales<L, NF>(v, sm, fstride, t, si, ls);
+    line_scales<L, NF, WIDE>(v, sm, fstride, t, si, ls);
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
@@ -544,9 +548,15 @@ __device__ __forceinline__ void fft_line(C (&v)[NF][8], C* sm, int fstride, cons
     if constexpr (IsPow2<L>::v) fft_passes<Q2, L, INV, NF, 0, SI, TwQ>(q, qs, fstride, qt, t, si);
     else fft_mixed<Q2, L, INV, NF, SI, TwQ>(q, qs, fstride, qt, t, si);
 #pragma unroll
-    for (int f = 0; f < NF; ++f)
+    for (int f = 0; f < NF; ++f) {
+      const bool big = WIDE && ls[f].bad == kLineBig;  // exponents 64 lower, then a product that may overflow
+      if (big) ls[f] = LineScale{ls[f].X - 64, ls[f].keep, 0};
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[f][e] = make_double2(from_fixed(q[f][e].x, ls[f]), from_fixed(q[f][e].y, ls[f]));
+      for (int e = 0; e < 8; ++e) {
+        v[f][e] = make_double2(from_fixed(q[f][e].x, ls[f]), from_fixed(q[f][e].y, ls[f]));
+        if (big) v[f][e] = make_double2(0x1p64 * v[f][e].x, 0x1p64 * v[f][e].y);
+      }
+    }
   } else {
     if constexpr (IsPow2<L>::v) fft_passes<C, L, INV, NF, 0, SI, C>(v, sm, fstride, tw, t, si);
     else fft_mixed<C, L, INV, NF, SI, C>(v, sm, fstride, tw, t, si);

@@ -156,6 +156,14 @@ template <class Op> struct LhyTabOp<Op, std::void_t<decltype(Op::LHY_TAB)>> {
   static constexpr bool v = Op::LHY_TAB;
 };
 
+// Row-pass ops that transform the caller's own fields over the whole FP64 range.
+template <class Op, class = void> struct WideOp {
+  static constexpr bool v = false;
+};
+template <class Op> struct WideOp<Op, std::void_t<decltype(Op::WIDE)>> {
+  static constexpr bool v = Op::WIDE;
+};
+
 // Every pass runs whole warps: the block reductions and the warp exchanges use
 // full-mask shuffles.  A row (x) pass gives each row L/8 threads and a column
 // pass each column L/8 threads, so a block holds a multiple of
@@ -295,7 +303,7 @@ template <class Op> __device__ __forceinline__ void xpass_body(const KArgs<typen
     C v[NV][8];
     if (ExtraGroups<Op>::v == 1 || g < NF) {
       Op::load(a, u, f, row, valid, t, v);
-      fft_line<C, L, Op::INV, NV>(v, line, fs, tw, t, si);
+      fft_line<C, L, Op::INV, NV, WideOp<Op>::v>(v, line, fs, tw, t, si);
     }
     if constexpr (!Op::POINTS) {
       Op::store(a, u, f, row, valid, t, v, acc);
@@ -651,7 +659,7 @@ template <class R_, int L_, bool INV_> struct XPlain {
   static constexpr const char* NAME = "x-plain";
   static double alg_bytes(const KArgs<R>& a) { return 2.0 * a.N * sizeof(C); }
   static constexpr int L = L_, NF = 1, NS = 0;
-  static constexpr bool INV = INV_, USES_LHY = false, POINTS = false;
+  static constexpr bool INV = INV_, USES_LHY = false, POINTS = false, WIDE = true;
   using Uni = NoUni;
   static __device__ void uniform(const KArgs<R>&, Uni&) {}
   template <int NV>
@@ -666,7 +674,7 @@ template <class R_, int L_, bool INV_> struct XPlain {
   static __device__ void finish(const KArgs<R>&, Uni&) {}
 };
 
-template <class R_, int L_, int AXIS_, bool INV_> struct ColPlain {
+template <class R_, int L_, int AXIS_, bool INV_, bool WIDE = false> struct ColPlain {
   using R = R_;
   using C = C2<R>;
   static constexpr const char* NAME = AXIS_ == 1 ? "y-pass" : "z-pass";
@@ -680,14 +688,14 @@ template <class R_, int L_, int AXIS_, bool INV_> struct ColPlain {
   template <class SI>
   static __device__ void process(const KArgs<R>& a, Uni&, int, int, int, size_t base, size_t ls, int t,
                                  C (&v)[1][8], C* sm, const C* tw, SI si, PAcc<R>*) {
-    fft_line<C, L, INV, 1>(v, sm, 0, tw, t, si);
+    fft_line<C, L, INV, 1, WIDE>(v, sm, 0, tw, t, si);
 #pragma unroll
     for (int e = 0; e < 8; ++e) a.gout[base + (size_t)Plan<L>::exit_pos(INV, t, e) * ls] = v[0][e];
   }
   static __device__ double* out(const KArgs<R>&, Uni&) { return nullptr; }
   static __device__ void finish(const KArgs<R>&, Uni&) {}
 };
-template <int L_, int AXIS_, bool INV_> struct ColMinB<ColPlain<float, L_, AXIS_, INV_>> {
+template <int L_, int AXIS_, bool INV_, bool WIDE> struct ColMinB<ColPlain<float, L_, AXIS_, INV_, WIDE>> {
   static constexpr int v = 3;
 };
 
