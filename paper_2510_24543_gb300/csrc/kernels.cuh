@@ -1152,7 +1152,9 @@ template <class R_, int L_> struct XFwdPC {
   using R = R_;
   using C = C2<R>;
   static constexpr const char* NAME = "x-fwd precond";
-  static double alg_bytes(const KArgs<R>& a) { return (a.diag ? 9.0 : 8.0) * a.N * sizeof(C); }
+  static double alg_bytes(const KArgs<R>& a) {
+    return (a.diag ? a.att != ATT_FULL ? 11.0 : 9.0 : 8.0) * a.N * sizeof(C);
+  }
   static constexpr int L = L_, NF = 2, NS = 0;
   static constexpr bool INV = false, USES_LHY = false, POINTS = false;
   using Uni = PcUni<R>;
