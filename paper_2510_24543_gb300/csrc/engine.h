@@ -191,8 +191,6 @@ template <class R> class Engine {
   egpe_status enq_pc(int mode, int gate, int ctrl, int rgiven, AttemptKind att = ATT_FULL, C* z = nullptr);
   egpe_status enq_lc(int gate, int ctrl, int pgiven);
   egpe_status enq_dipolar(const KArgs<R>& a);
-  egpe_status enq_eg_carried(int gate, int ctrl);
-  egpe_status enq_lc_carried(int mode, int gate, int ctrl);
   egpe_status enq_attempt(int mode, AttemptKind kind);
   // The current point of a run in PH_VERIFY by transform (nothing in other phases).
   egpe_status enq_verify() { return enq_eg(0, GATE_VERIFY, 1, ATT_REFRESH); }

@@ -38,7 +38,6 @@ namespace {
 constexpr int kNoAllocMaxN = 32;                         // points per axis
 constexpr size_t kNoAllocMaxPoints = 32 * 32 * 32;
 constexpr size_t kNoAllocBlocks = 1024;                  // partial-sum slots
-constexpr int kNoAllocSMs = 152;                         // SMs the row passes are spread over
 constexpr size_t kNoAllocBytes = (size_t)4 << 20;        // 4 MiB
 
 constexpr size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -57,33 +56,40 @@ static_assert(kOffEnd <= kNoAllocBytes, "no-alloc scratch layout exceeds its arr
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 constexpr int kMaxDevices = 64;
-static unsigned char* g_scratch_ptr[kMaxDevices] = {nullptr};
+struct NoAllocDevice {
+  unsigned char* scratch;
+  int sms;
+};
+static NoAllocDevice g_noalloc_dev[kMaxDevices] = {};
 static std::mutex g_scratch_mutex;
 
-// Device address of the scratch array on the current device (looked up once).
-cudaError_t noalloc_scratch(int dev, unsigned char** out) {
+// Address of the scratch array on the current device and the SMs to spread the row
+// passes over (looked up once).
+cudaError_t noalloc_device(int dev, NoAllocDevice& out) {
   std::lock_guard<std::mutex> lock(g_scratch_mutex);
-  if (!g_scratch_ptr[dev]) {
+  NoAllocDevice& d = g_noalloc_dev[dev];
+  if (!d.scratch) {
+    cudaError_t ce = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
     void* ptr = nullptr;
-    const cudaError_t ce = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
+    if (ce == cudaSuccess) ce = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
     if (ce != cudaSuccess) return ce;
     if (!ptr) return cudaErrorInvalidSymbol;
-    g_scratch_ptr[dev] = (unsigned char*)ptr;
+    d.scratch = (unsigned char*)ptr;
   }
-  *out = g_scratch_ptr[dev];
+  out = d;
   return cudaSuccess;
 }
 
-template <class Op> cudaError_t noalloc_launch_x(egpe::KArgs<double> a, int rows, cudaStream_t s) {
+template <class Op> cudaError_t noalloc_launch_x(egpe::KArgs<double> a, int rows, int nsm, cudaStream_t s) {
   using namespace egpe;
   constexpr int L = Op::L, NS = Op::NS;
-  const int mx = default_rows<Op>(rows, kNoAllocSMs);
+  const int mx = default_rows<Op>(rows, nsm);
   a.MX = mx;
   const size_t smem = L * sizeof(double2) + (Op::USES_LHY ? lhy_stage_bytes<double>(a.Q) : 0) +
                       mx * row_pass_bytes<Op>() + (NS > 0 ? sizeof(RedSmem<NS>) : 0);
   const int groups = (rows + mx - 1) / mx;
   const int grid = std::min(groups, (int)kNoAllocBlocks);
-  xpass_kernel<Op><<<grid, mx * row_groups<Op>(mx, rows, kNoAllocSMs) * L / 8, smem, s>>>(a);
+  xpass_kernel<Op><<<grid, mx * row_groups<Op>(mx, rows, nsm) * L / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -101,26 +107,26 @@ template <class Op> cudaError_t noalloc_launch_col(egpe::KArgs<double> a, int ot
   return cudaGetLastError();
 }
 
-template <int LX, int LY, int LZ> cudaError_t noalloc_pipeline(const egpe::KArgs<double>& a, cudaStream_t s) {
+template <int LX, int LY, int LZ> cudaError_t noalloc_pipeline(const egpe::KArgs<double>& a, int nsm, cudaStream_t s) {
   using namespace egpe;
   cudaError_t e;
   const int rows = a.ny * a.nz;
-  if ((e = noalloc_launch_x<XFwdEG<double, LX>>(a, rows, s)) != cudaSuccess) return e;
+  if ((e = noalloc_launch_x<XFwdEG<double, LX>>(a, rows, nsm, s)) != cudaSuccess) return e;
   egpe::KArgs<double> y = a;
   y.gin = a.W;
   y.gout = a.W;
   if ((e = noalloc_launch_col<ColPlain<double, LY, 1, false>>(y, a.nz, s)) != cudaSuccess) return e;
   if ((e = noalloc_launch_col<ZEg<double, LZ>>(a, a.ny, s)) != cudaSuccess) return e;
   if ((e = noalloc_launch_col<ColPlain<double, LY, 1, true>>(y, a.nz, s)) != cudaSuccess) return e;
-  return noalloc_launch_x<XInvEG<double, LX>>(a, rows, s);
+  return noalloc_launch_x<XInvEG<double, LX>>(a, rows, nsm, s);
 }
 
 template <int LX, int LY>
-cudaError_t noalloc_dispatch_z(int nz, const egpe::KArgs<double>& a, cudaStream_t s) {
-  return nz == 16 ? noalloc_pipeline<LX, LY, 16>(a, s) : noalloc_pipeline<LX, LY, 32>(a, s);
+cudaError_t noalloc_dispatch_z(int nz, const egpe::KArgs<double>& a, int nsm, cudaStream_t s) {
+  return nz == 16 ? noalloc_pipeline<LX, LY, 16>(a, nsm, s) : noalloc_pipeline<LX, LY, 32>(a, nsm, s);
 }
-template <int LX> cudaError_t noalloc_dispatch_y(int ny, int nz, const egpe::KArgs<double>& a, cudaStream_t s) {
-  return ny == 16 ? noalloc_dispatch_z<LX, 16>(nz, a, s) : noalloc_dispatch_z<LX, 32>(nz, a, s);
+template <int LX> cudaError_t noalloc_dispatch_y(int ny, int nz, const egpe::KArgs<double>& a, int nsm, cudaStream_t s) {
+  return ny == 16 ? noalloc_dispatch_z<LX, 16>(nz, a, nsm, s) : noalloc_dispatch_z<LX, 32>(nz, a, nsm, s);
 }
 
 }  // namespace
@@ -167,12 +173,13 @@ extern "C" egpe_status egpe_energy_grad_noalloc(const egpe_grid* grid, const egp
     set_error_msg("egpe_energy_grad_noalloc: device ordinal out of range");
     return EGPE_ERR_INVALID_ARG;
   }
-  unsigned char* base = nullptr;
-  ce = noalloc_scratch(dev, &base);
+  NoAllocDevice nd{};
+  ce = noalloc_device(dev, nd);
   if (ce != cudaSuccess) {
     set_error("cudaGetSymbolAddress", ce);
     return EGPE_ERR_CUDA;
   }
+  unsigned char* const base = nd.scratch;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const size_t N = (size_t)nx * ny * nz;
 
@@ -259,7 +266,7 @@ extern "C" egpe_status egpe_energy_grad_noalloc(const egpe_grid* grid, const egp
   a.nf = 3;
   a.f0 = 0;
 
-  ce = (nx == 16) ? noalloc_dispatch_y<16>(ny, nz, a, s) : noalloc_dispatch_y<32>(ny, nz, a, s);
+  ce = (nx == 16) ? noalloc_dispatch_y<16>(ny, nz, a, nd.sms, s) : noalloc_dispatch_y<32>(ny, nz, a, nd.sms, s);
   if (ce != cudaSuccess) {
     set_error("egpe_energy_grad_noalloc launch", ce);
     return EGPE_ERR_CUDA;

@@ -982,49 +982,32 @@ template <class R> egpe_status Engine<R>::enq_dipolar(const KArgs<R>& a) {
   return plain_col(kAxisY, 1, y, tmy());
 }
 
-// Line-search and trial pipelines with T psi and T p carried along: one packed
-// transform pair each (the dipolar convolutions of rho and of the trial densities).
-template <class R> egpe_status Engine<R>::enq_lc_carried(int mode, int gate, int ctrl) {
-  KArgs<R> a = *base_;
-  a.att = ATT_CARRIED;
-  a.gate = gate;
-  a.flag = 0;
-  a.ctrl = 0;
-  a.diag = mode == 3 ? 1 : 0;
-  a.nf = 1;
-  a.f0 = 0;
-  if constexpr (sizeof(R) == 8) {
-    EGPE_TRY(dispatch_x<XFwdLL>(nx, a));
-    EGPE_TRY(enq_dipolar(a));
-    a.ctrl = ctrl;
-    return dispatch_x<XInvLL>(nx, a);
-  }
-  return EGPE_ERR_UNSUPPORTED;
-}
-
-template <class R> egpe_status Engine<R>::enq_eg_carried(int gate, int ctrl) {
-  KArgs<R> a = *base_;
-  a.att = ATT_CARRIED;
-  a.gate = gate;
-  a.flag = 1;
-  a.ctrl = 0;
-  a.nf = 1;
-  a.f0 = 0;
-  if constexpr (sizeof(R) == 8) {
-    EGPE_TRY(dispatch_x<XFwdEL>(nx, a));
-    EGPE_TRY(enq_dipolar(a));
-    a.ctrl = ctrl;
-    return dispatch_x<XInvEL>(nx, a);
-  }
-  return EGPE_ERR_UNSUPPORTED;
-}
-
 template <class R> egpe_status Engine<R>::enq_attempt(int mode, AttemptKind kind) {
-  if constexpr (sizeof(R) == 8) {
+  if constexpr (sizeof(R) == 8) {  // the engines that carry T psi and T p along
     if (kind != ATT_FULL) {
       EGPE_TRY(enq_pc(mode, GATE_CARRIED_PC, 1, 0, kind));
-      EGPE_TRY(enq_lc_carried(mode, GATE_NEW_ITER, 1));
-      return kind == ATT_REFRESH ? enq_eg(1, GATE_ACTIVE, 1, kind) : enq_eg_carried(GATE_ACTIVE, 1);
+      // line search and trial: one packed transform pair each (the dipolar
+      // convolutions of rho and of the trial densities)
+      KArgs<R> a = *base_;
+      a.att = ATT_CARRIED;
+      a.gate = GATE_NEW_ITER;
+      a.flag = 0;
+      a.ctrl = 0;
+      a.diag = mode == 3 ? 1 : 0;
+      a.nf = 1;
+      a.f0 = 0;
+      EGPE_TRY(dispatch_x<XFwdLL>(nx, a));
+      EGPE_TRY(enq_dipolar(a));
+      a.ctrl = 1;
+      EGPE_TRY(dispatch_x<XInvLL>(nx, a));
+      if (kind == ATT_REFRESH) return enq_eg(1, GATE_ACTIVE, 1, kind);
+      a.gate = GATE_ACTIVE;
+      a.flag = 1;
+      a.ctrl = 0;
+      EGPE_TRY(dispatch_x<XFwdEL>(nx, a));
+      EGPE_TRY(enq_dipolar(a));
+      a.ctrl = 1;
+      return dispatch_x<XInvEL>(nx, a);
     }
   }
   EGPE_TRY(enq_pc(mode, GATE_NEW_ITER, 1, 0));

@@ -447,10 +447,7 @@ template <class Op> struct ColDefaultM {
 };
 // FP64: threads per SM the passes ask for (registers 65536 / this).  The fixed-point
 // lines wait on integer chains, which more warps hide.
-#ifndef EGPE_COL64
-#define EGPE_COL64 512
-#endif
-constexpr int COL64 = EGPE_COL64;
+constexpr int kCol64Threads = 512;
 // Launch bounds of a column kernel: the run-time width keeps ColMaxThreads; a
 // compile-time width MC has exactly MC L/8 threads, and the FP32 plain y/z
 // passes (the ColPlain op, small epilogue) of up to 256 threads ask for three
@@ -459,7 +456,7 @@ constexpr int COL64 = EGPE_COL64;
 // pass takes 24 us with three blocks of 192 and 33 us with two.
 template <class Op> struct ColMinB {
   static constexpr int threads = ColDefaultM<Op>::v * (Op::L / 8);
-  static constexpr int want = sizeof(typename Op::R) == 8 ? COL64 : !IsPow2<Op::L>::v ? 576 : 0;
+  static constexpr int want = sizeof(typename Op::R) == 8 ? kCol64Threads : !IsPow2<Op::L>::v ? 576 : 0;
   static constexpr int v = want > threads ? want / threads : 1;
 };
 template <class Op, int MC> struct ColBounds {
