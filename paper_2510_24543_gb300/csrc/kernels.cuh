@@ -1050,6 +1050,10 @@ template <class R> __device__ __forceinline__ void pc_uniform(const KArgs<R>& a,
       u.mu[i] = __ldcg(&a.st->mu[i]);
       u.shift[i] = __ldcg(&a.st->shift[i]);
       u.floor_[i] = fl * u.shift[i];
+      if (u.direct) {  // P_V = 1: r itself is transformed (the z pass has its own shift)
+        u.shift[i] = -1e300;
+        u.floor_[i] = 1.0;
+      }
     }
   } else {
     R c[6];
@@ -1070,8 +1074,7 @@ template <class R> __device__ __forceinline__ R pv_at(const PcUni<R>& u, int i, 
   return P > fl ? P : fl;
 }
 // r_i = H_i psi_i - mu_i psi_i (stored unless given) and w_i = P_V^{-1} r_i when
-// diag, at CH points: both components (NV = 2, i = 0) or component i alone.  In a
-// direct pass w_i = r_i.
+// diag, at CH points: both components (NV = 2, i = 0) or component i alone.
 template <class R, int CH, int NV>
 __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u, int i, const size_t (&idx)[CH],
                                             C2<R> (&w)[NV][CH]) {
@@ -1099,7 +1102,7 @@ __device__ __forceinline__ void pc_residual(const KArgs<R>& a, const PcUni<R>& u
         r = cmk<C>(fma_(-mu, p[k][j].x, r.x), fma_(-mu, p[k][j].y, r.y));
         pick(a.rb, u.nsel)[(size_t)c * N + idx[j]] = r;
       }
-      if (a.diag && !u.direct) {
+      if (a.diag) {
         r = cscale(r, rcp_(pv_at(u, c, c ? bb[j].y : bb[j].x)));
         if (a.att != ATT_FULL) a.wz[(size_t)c * N + idx[j]] = r;
       }
@@ -1210,12 +1213,13 @@ template <class R_, int L_> struct ZPc {
     fft_line<C, L, false, 1>(v, sm, 0, tw, t, si);
     const R kxy = kq_xy(a, x, y);
     const R sh = a.invN * (f == 0 ? u.shift[0] : u.shift[1]);
+    if (u.direct) {  // (shift + |k|^2/2) / N
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      // invN / (shift + |k|^2/2), numerator and denominator over N; a direct pass
-      // multiplies by (shift + |k|^2/2) / N
-      const R q = sh + (kxy + u.kz[e]);
-      v[0][e] = cscale(v[0][e], u.direct ? q : a.invN * a.invN * rcp_(q));
+      for (int e = 0; e < 8; ++e) v[0][e] = cscale(v[0][e], sh + (kxy + u.kz[e]));
+    } else {
+      // invN / (shift + |k|^2/2), numerator and denominator over N
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[0][e] = cscale(v[0][e], a.invN * a.invN * rcp_(sh + (kxy + u.kz[e])));
     }
     col_after<L>(sm, si);
     fft_line<C, L, true, 1>(v, sm, 0, tw, t, si);
