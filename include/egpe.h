@@ -365,7 +365,9 @@ egpe_status egpe_set_wait_limit(egpe_handle* h, long long polls);
  * every pass of an attempt is one launch per group of up to 16 instances of
  * one grid shape; finished instances leave the launches at the next poll.
  * Each instance's arithmetic, controller and result are those of a solve of
- * that instance alone.  Reports then carry the shared wall time, graph
+ * that instance alone (after an end that its transformed evaluation did not
+ * confirm, up to rounding: the next full transforms come with the batch's
+ * count of attempts).  Reports then carry the shared wall time, graph
  * replays and kernel launches of the whole batch. */
 egpe_status egpe_ncg_solve(egpe_handle* h, void* const* psi_inout, const egpe_solve_opts* opts,
                            egpe_report* reports);

@@ -119,7 +119,7 @@ struct DevState {
   double E, mu[2], shift[2], nmuL[2], norm2[2];
   // iteration scalars
   double res, beta, c[2], alpha0, alpha, alpha_prev, theta[2], pnorm2[2];
-  double Ep, Epp, coef_a[2], coef_b[2], E_trial, dE_last, psip[2];
+  double Ep, Epp, coef_a[2], coef_b[2], coef_d[2], E_trial, dE_last, psip[2];  // coef_d = coef_a - 1
   double rz, rz_prev;  // Re<r, P^{-1} r> of this and of the previous iteration (PR+ beta)
   double dV, invN;
   long long ffts;

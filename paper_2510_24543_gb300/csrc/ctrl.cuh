@@ -92,6 +92,7 @@ __device__ inline void set_retraction(DevState* st) {
       st->coef_a[i] = 1.0 / sqrt(st->norm2[i]);
       st->coef_b[i] = 0.0;
     }
+    st->coef_d[i] = st->coef_a[i] - 1.0;
   }
 }
 

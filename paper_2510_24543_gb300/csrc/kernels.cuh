@@ -707,7 +707,7 @@ template <int L_, int AXIS_, bool INV_, bool WIDE> struct ColMinB<ColPlain<float
 // ----------------------------------------------------------------------------
 template <class R> struct EgUni {
   int cur, slot, nsel;
-  R ca[2], cb[2];
+  R ca[2], cb[2];  // ca: a - 1 in FP32
 };
 
 // Controller step after an energy/gradient evaluation (last block, one thread):
@@ -735,7 +735,8 @@ template <class R_, int L_> struct XFwdEG {
     u.slot = a.flag ? (u.cur ^ 1) : u.cur;
     u.nsel = __ldcg(&a.st->n) & 1;
     R c[4];
-    load_uniforms<R, 4>({&a.st->coef_a[0], &a.st->coef_a[1], &a.st->coef_b[0], &a.st->coef_b[1]}, c);
+    const double* ca = sizeof(R) == 4 ? a.st->coef_d : a.st->coef_a;
+    load_uniforms<R, 4>({&ca[0], &ca[1], &a.st->coef_b[0], &a.st->coef_b[1]}, c);
     u.ca[0] = c[0];
     u.ca[1] = c[1];
     u.cb[0] = c[2];
@@ -748,11 +749,13 @@ template <class R_, int L_> struct XFwdEG {
     const R n1 = cabs2(p1), n2 = cabs2(p2);
     return cmk<C>(fma_(a.d12, n2, a.d11 * n1), fma_(a.d22, n2, a.d21 * n1));
   }
-  // ca p + cb q.  The large term is the exact product inside the FMA: rounded on its
-  // own, ca p (ca within a few units of 1 near convergence) is off in one direction
-  // at nearly every point, and the FP32 norms after a solve drift with it.
+  // a p + b q.  FP32: p + ((a - 1) p + b q).  Near convergence a is within a few units
+  // of 1: rounded to 24 bits it moves the norm by up to 6e-8, and a p rounded on its
+  // own is off in one direction at nearly every point.  FP64: a p is the exact product
+  // inside the FMA.
   static __device__ C trial(R ca, C p, R cb, C q) {
-    return cmk<C>(fma_(ca, p.x, cb * q.x), fma_(ca, p.y, cb * q.y));
+    if constexpr (sizeof(R) == 4) return cmk<C>(p.x + fma_(ca, p.x, cb * q.x), p.y + fma_(ca, p.y, cb * q.y));
+    else return cmk<C>(fma_(ca, p.x, cb * q.x), fma_(ca, p.y, cb * q.y));
   }
   static __device__ C point(const KArgs<R>& a, const Uni& u, int i, size_t idx) {
     const C p = (a.gin ? a.gin : pick(a.psi, u.cur))[(size_t)i * a.N + idx];
