@@ -182,10 +182,9 @@ template <bool INV, class C> __device__ __forceinline__ void dft5(C* v) {
 // * Scale.  B >= sum_j (|Re x_j| + |Im x_j|) over the line bounds every
 //   intermediate value and output of the transform.  With q = x 2^s, s the largest
 //   with 2^s B <= 2^62, nothing overflows, sums are exact, and an input is rounded
-//   towards minus infinity by at most one unit: 2^-62 to 2^-61 B.  For a line whose
-//   values are comparable that is up to 2^-60 L of a typical value (|Re| + |Im|: 2^-53
-//   at L = 128, 2^-55 on average and half that off its mean), against 2^-53 of each value
-//   in FP64.
+//   towards minus infinity by at most one unit, 2^-62 to 2^-61 B.  For a line whose
+//   values are comparable that is 2^-62 L to 2^-61 L of a typical |Re| + |Im| (at most
+//   2^-54 at L = 128), against 2^-53 of each value in FP64.
 // * Products.  Twiddles and constants carry 62 fractional bits as two signed
 //   32-bit limbs; a product is three 32 x 32 + 64 multiply-adds, right to two
 //   units.
